@@ -297,16 +297,11 @@ int kh_hdegree_exact_noalloc(int64_t n, const int64_t *rowptr, const int32_t *co
 #define KH_COMPACT_OFF 1
 #define KH_COMPACT_ALWAYS 2
 /* KH_OP_LEVEL_UNION: how the level >= 2 list union (Alg. 2 with Alg. 5's
- * trim) schedules a node's lists over the warps of its CTA.
- * KH_LEVELU_STEPPED: barrier-separated steps, the trim once per step;
- * KH_LEVELU_FREE: warps claim lists and trim from their own view of the rank
- * counts, meeting only to compact the hash set;
- * KH_LEVELU_GROUPED: as free, with groups of 32, 16, ..., 1 lanes claiming
- * lists in place of whole warps: per node, the fewest lanes whose step of
- * 4 keys a lane covers the keys a list is expected to give at or above the
- * starting level (sum of |B[w]| 2^(k[w] - t) over the lists, over their
- * number); with slices = d > 1 (a power of two up to 64) a group covers 1/d
- * of those keys (0: the default).  KH_VAR_AUTO: grouped.  The lists are the
+ * trim) reads a node's lists.  KH_VAR_AUTO and KH_LEVELU_GROUPED: groups of 2,
+ * 8 or 32 lanes claim lists, by the keys a list is expected to give at or above
+ * the running level (|B[w]| 2^(k[w] - t)); with slices = d > 1 (a power of two
+ * up to 64) by 1/d of those keys (0: the default).  KH_LEVELU_FREE and
+ * KH_LEVELU_STEPPED (one schedule by now): a warp per list.  The lists are the
  * same every way. */
 #define KH_OP_LEVEL_UNION 2
 #define KH_LEVELU_STEPPED 1

@@ -72,7 +72,6 @@ int ensure_work(Graph& g) {
     if ((rc = dalloc(g.ctx, &g.listW, n, "listW"))) return rc;
     if ((rc = dalloc(g.ctx, &g.listC[0], n, "listC0"))) return rc;
     if ((rc = dalloc(g.ctx, &g.listC[1], n, "listC1"))) return rc;
-    if ((rc = dalloc(g.ctx, &g.listH, n, "listH"))) return rc;
     if ((rc = dalloc(g.ctx, &g.fresh, n, "fresh"))) return rc;
     if ((rc = dalloc(g.ctx, &g.deadbm, ((n + 127) / 128) * 4, "deadbm"))) return rc;
     if ((rc = dalloc(g.ctx, &g.degX, n, "degX"))) return rc;
@@ -189,29 +188,18 @@ int ensure_lists(Graph& g) {
     const int64_t need_keys = (int64_t)(g.hmax - 1) * g.n * g.cap;
     if (g.keys && g.keys_levels * g.n * g.cap < need_keys) {
         dfree(&g.keys);
-        dfree(&g.ltop);
     }
-    if (g.lsz && g.lvl_alloc < g.hmax) {
-        dfree(&g.lsz);
-        dfree(&g.lk);
-    }
+    if (g.meta && g.lvl_alloc < g.hmax) dfree(&g.meta);
     int rc;
     if (need_keys > 0) {
         if ((rc = dalloc(g.ctx, &g.keys, (size_t)need_keys, "sample lists"))) return rc;
-        if ((rc = dalloc(g.ctx, &g.ltop, (size_t)(g.hmax - 1) * (size_t)g.n, "list top ranks")))
-            return rc;
         g.keys_levels = g.hmax - 1;
     }
-    if (!g.lsz) g.lvl_alloc = g.hmax;
-    if ((rc = dalloc(g.ctx, &g.lsz, (size_t)g.lvl_alloc * g.n, "list sizes"))) return rc;
-    if ((rc = dalloc(g.ctx, &g.lk, (size_t)g.lvl_alloc * g.n, "list levels"))) return rc;
+    if (!g.meta) g.lvl_alloc = g.hmax;
+    if ((rc = dalloc(g.ctx, &g.meta, (size_t)g.lvl_alloc * g.n, "list metas"))) return rc;
     if ((rc = dalloc(g.ctx, &g.rho, (size_t)g.n, "list change ranks"))) return rc;
     if ((rc = ensure_split(g))) return rc;
-    if (!g.ranks_valid) {
-        launch_ranks(g, g.ctx->stream);
-        g.ranks_valid = true;
-    }
-    return KH_OK;
+    return ensure_positions(g);
 }
 
 int ensure_bfs_scratch(Graph& g, int64_t ctas, bool bitmaps) {
@@ -250,9 +238,11 @@ static void free_graph_arrays(Graph& g) {
     dfree(&g.rank);
     dfree(&g.alive);
     dfree(&g.keys);
-    dfree(&g.ltop);
-    dfree(&g.lsz);
-    dfree(&g.lk);
+    dfree(&g.meta);
+    dfree(&g.key32);
+    dfree(&g.clsw);
+    dfree(&g.wrank);
+    dfree(&g.lu_stage);
     dfree(&g.d32);
     dfree(&g.d64);
     dfree(&g.core32);
@@ -268,7 +258,6 @@ static void free_graph_arrays(Graph& g) {
     dfree(&g.state);
     dfree(&g.queues);
     dfree(&g.gbitmaps);
-    dfree(&g.listH);
     dfree(&g.fresh);
     dfree(&g.rho);
     dfree(&g.loss);
@@ -311,8 +300,7 @@ static void free_graph_arrays(Graph& g) {
     dfree(&g.cp_tmp);
     dfree(&g.cp_sums);
     dfree(&g.part_keys);
-    dfree(&g.part_size);
-    dfree(&g.part_t);
+    dfree(&g.part_meta);
     dfree(&g.part_done);
     dfree(&g.part_stop);
     dfree(&g.part_lb);
@@ -615,17 +603,18 @@ int kh_footprint(int64_t n, int64_t nnz, int32_t h, int64_t M_or_0, double eps, 
     const int64_t cap = (M + 3) & ~(int64_t)3;
     // the graph: CSR, ranks, state
     int64_t b = 8 * (n + 1) + 4 * nnz + n + (int64_t)sizeof(kh::DevState);
-    // per-node work arrays of ensure_work (alive, d, core, rounds, stamps, seven
+    // per-node work arrays of ensure_work (alive, d, core, rounds, stamps, six
     // node lists, fresh, degrees, bounds, loss and its list, best neighbours,
     // removed-node bitmap)
-    b += n * (1 + 4 + 8 + 4 + 8 + 4 + 4 + 7 * 4 + 1 + 4 + 8 + 4 + 4 + 4) + n / 8 + 64;
-    // level lists 1..h-1 (cap keys per node and level), sizes and levels of
-    // 1..h, change ranks, top ranks
-    b += (int64_t)(h - 1) * n * cap * 4 + (int64_t)h * n * 5 + n + (int64_t)(h - 1) * n;
-    // split parts of heavy nodes: at most nnz / 1365 slots (ceil(deg/2048) <=
-    // deg/1365 for deg > 4096), each cap keys plus counters
-    const int64_t parts = nnz / 1365;
-    b += parts * (cap * 4 + 29) + 4 * n;
+    b += n * (1 + 4 + 8 + 4 + 8 + 4 + 4 + 6 * 4 + 1 + 4 + 8 + 4 + 4 + 4) + n / 8 + 64;
+    // level lists 1..h-1 (cap words per node and level), meta words of 1..h,
+    // change ranks, positions and their class tables, the union's stage slots
+    b += (int64_t)(h - 1) * n * cap * 4 + (int64_t)h * n * 4 + n + 4 * n + n / 32 + 1024 +
+         (int64_t)12 * 160 * cap * 4;
+    // split parts of heavy nodes: at most nnz / 409 slots (ceil(deg/512) <=
+    // deg/409 for deg > 2048), each cap keys plus counters
+    const int64_t parts = nnz / 409;
+    b += parts * (cap * 4 + 32) + 4 * n;
     // the peel's compaction buffers (graphs of at least 65536 nodes)
     if (n >= 65536) b += 2 * 8 * (n + 1) + 2 * 4 * nnz + 2 * 4 * (n + 1) + 16 * (n + 1) + 64 * 1024;
     *bytes = b + (1 << 20);
@@ -692,6 +681,7 @@ int kh_set_sampling(kh_graph* G, uint64_t seed, int64_t M_or_0, double eps, doub
     if (seed != g.seed) {
         g.seed = seed;
         g.ranks_valid = false;
+        g.pos_valid = false;
     }
     return KH_OK;
 }

@@ -8,9 +8,11 @@
 //                                              old graph), 0 removed earlier
 //   keys     uint32[(h-1) * n * cap]           B[v,i] for levels i = 1..h-1, one
 //                                              fixed slot of cap >= M keys per
-//                                              (level, node); key = r << 27 | id,
-//                                              grouped by rank, highest first
-//   lsz      int32[h * n], lk uint8[h * n]     |B[v,i]| and k[v,i], i = 1..h
+//                                              (level, node), as keys r << 27 |
+//                                              position by falling rank, or as a
+//                                              bitmap over positions (kh_sampled.cu)
+//   meta     uint32[h * n]                     |B[v,i]|, k[v,i], highest rank, form
+//   key32    uint32[n]                         r << 27 | position of each node
 //   d32 / d64                                  deg_h (exact) or estimate (sampled)
 //   seen     int32[n]                          stamp array for frontier dedup
 //   lists    int32[n] x 4                      removed set, frontiers, work lists
@@ -69,9 +71,8 @@ constexpr int kProfKinds = 5;
 // needs no memset nodes.
 constexpr int kRcBfs = 0;          // refine BFS work counter
 constexpr int kRcRefineWork = 1;   // refine last-level list work counter
-constexpr int kRcRefineHeavy = 2;  // refine level-1 heavy count (h = 1)
 constexpr int kRcLevelWork = 3;    // + i: refresh level i work counter, i = 1..kMaxH
-constexpr int kRcLevelHeavy = 20;  // + i: refresh level i heavy count
+constexpr int kRcSubWork = 20;     // + i: split-part work counter of level i (0: the refine)
 constexpr int kRcW = 37;           // + i: work list of level i (0: exact affected nodes)
 constexpr int kRcF = 54;           // + hop: frontier written by that hop (exact)
 constexpr int kRcC = 71;           // + i: changed nodes at level i
@@ -93,7 +94,6 @@ struct DevState {
     unsigned long long bytes[kProfKinds];  // algorithmic bytes per kernel class
     int err;                     // kErr* bits
     int early;                   // exact early stop taken this round
-    int nH;                      // heavy nodes deferred by the level-1 kernel
     int nQ;                      // refine list size (stale nodes due this round)
     unsigned long long minU;     // min of the upper bounds d over alive nodes
     int rc[kRcCount];            // per-round counters (kRc*)
@@ -249,11 +249,16 @@ struct Graph {
     uint8_t *rank;
     uint8_t *alive;
     uint32_t *keys;
-    uint8_t *ltop;          // highest rank of each stored list (levels 1..h-1)
     int64_t keys_levels;    // allocated levels in keys
-    int32_t *lsz;
-    uint8_t *lk;
-    int64_t lvl_alloc;      // allocated levels in lsz/lk
+    uint32_t *meta;         // meta word of each list (kh_sampled.cu)
+    int64_t lvl_alloc;      // allocated levels in meta
+    // positions of the nodes by descending rank (kh_sampled.cu: k_pos_*)
+    bool pos_valid;
+    uint32_t *key32;
+    int32_t *clsw;
+    uint8_t *wrank;
+    uint32_t *lu_stage;     // k_levelU: compaction stage, one slot per CTA
+    int64_t lu_stage_cap;
     int32_t *d32;
     unsigned long long *d64;
     int32_t *core32;
@@ -270,7 +275,6 @@ struct Graph {
     int32_t *queues;
     uint32_t *gbitmaps;
     int64_t scratch_ctas;
-    int32_t *listH;         // heavy nodes deferred by the level-1 warp kernel
     // batches of graphs packed in one CSR (all nullptr for a single graph)
     int32_t *gid;           // graph of each node
     int64_t *vtx_off;       // first node of each graph, ngraphs + 1 entries
@@ -339,8 +343,7 @@ struct Graph {
     int64_t part_cap;
     int64_t part_cap_keys;  // cap the slots were sized for
     uint32_t *part_keys;
-    int32_t *part_size;
-    uint8_t *part_t;
+    uint32_t *part_meta;
     int32_t *part_done;
     int32_t *part_stop;
     unsigned long long *part_lb;
@@ -403,6 +406,8 @@ int ensure_work(Graph& g);
 int ensure_lists(Graph& g);
 // part slots for the split heavy nodes of the level passes (kh_sampled.cu)
 int ensure_split(Graph& g);
+// ranks, and the positions the sampled lists use (kh_sampled.cu)
+int ensure_positions(Graph& g);
 int ensure_bfs_scratch(Graph& g, int64_t ctas, bool bitmaps);
 // A device allocation through the context's fault-injection counter.
 int alloc_bytes(kh_ctx* ctx, void** p, size_t bytes, const char* what);

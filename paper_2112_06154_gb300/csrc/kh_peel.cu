@@ -66,7 +66,15 @@ struct PeelState {
     unsigned long long* mr;
     int32_t* left;       // alive nodes per graph (batches: per-graph early stop)
     const int32_t* gid;  // graph of each node; nullptr for a single graph
+    uint32_t* meta;      // sampled: list meta words, zeroed when a node leaves
+    int64_t meta_n;      //   words per level
+    int levels;          //   stored levels
 };
+
+// A removed node's lists are no longer members of any union.
+__device__ __forceinline__ void drop_lists(const PeelState& p, int64_t v) {
+    for (int i = 0; i < p.levels; ++i) p.meta[(size_t)i * (size_t)p.meta_n + (size_t)v] = 0u;
+}
 
 __device__ __forceinline__ int graph_of(const PeelState& p, int64_t v) {
     return p.gid ? p.gid[v] : 0;
@@ -255,6 +263,7 @@ __global__ void k_select(uint8_t* __restrict__ alive, const T* __restrict__ d, i
                 round_of[v] = round;
                 alive[v] = 2;
                 seen[v] = round * kPhaseStride;
+                drop_lists(p, v);
             } else {
                 ++keep;
             }
@@ -392,7 +401,7 @@ __global__ void k_dense_sum(const uint8_t* __restrict__ alive, const T* __restri
 // EstDense: the nodes whose scheduled round has come leave (the removal order
 // is given, not chosen by d).
 __global__ void k_select_sched(uint8_t* __restrict__ alive, const int32_t* __restrict__ sched,
-                               int64_t n, const int32_t* __restrict__ vl, DevState* st,
+                               int64_t n, const int32_t* __restrict__ vl, DevState* st, PeelState p,
                                int32_t* __restrict__ R, int32_t* __restrict__ seen,
                                int32_t* __restrict__ round_of) {
     if (st->n_alive == 0) return;
@@ -410,6 +419,7 @@ __global__ void k_select_sched(uint8_t* __restrict__ alive, const int32_t* __res
                 round_of[v] = round;
                 alive[v] = 2;
                 seen[v] = round * kPhaseStride;
+                drop_lists(p, v);
             } else {
                 ++keep;
             }
@@ -625,7 +635,7 @@ LbArgs lb_args(const Graph& g) {
     return a;
 }
 
-PeelState peel_state(const Graph& g) {
+PeelState peel_state(const Graph& g, bool sampled) {
     PeelState p;
     p.c = g.pc;
     p.mn = g.pmn;
@@ -633,6 +643,9 @@ PeelState peel_state(const Graph& g) {
     p.mu = g.pmu;
     p.left = g.pleft;
     p.gid = g.gid;
+    p.meta = sampled ? g.meta : nullptr;
+    p.meta_n = g.n;
+    p.levels = sampled ? g.hmax : 0;
     return p;
 }
 
@@ -645,12 +658,12 @@ int refine(Graph& g, bool sampled, cudaStream_t s) {
     prof_begin(g, kProfPeel, s);
     if (sampled)
         k_collect<unsigned long long><<<grid, kPeelThreads, 0, s>>>(
-            g.alive, g.fresh, g.vcount, g.vlist, la, g.d64, g.dense ? 1 : 0, g.state, peel_state(g),
+            g.alive, g.fresh, g.vcount, g.vlist, la, g.d64, g.dense ? 1 : 0, g.state, peel_state(g, sampled),
             g.listB);
     else
         k_collect<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.fresh, g.vcount, g.vlist, la,
                                                          g.d32, g.dense ? 1 : 0, g.state,
-                                                         peel_state(g), g.listB);
+                                                         peel_state(g, sampled), g.listB);
     count_launch(g, 1);
     prof_end(g, kProfPeel, s);
     if (sampled) return launch_level(g, g.h, g.listB, &g.state->nQ, 0, 0, s, 2);
@@ -665,6 +678,7 @@ int start_peel(Graph& g, bool sampled, cudaStream_t s) {
     int rc = KH_OK;
     if (sampled) {
         // every list below each node's last level; the last level itself stays lazy
+        KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.meta, 0, sizeof(uint32_t) * (size_t)g.hmax * (size_t)g.n, s));
         for (int i = 1; i < g.hmax && rc == KH_OK; ++i)
             rc = launch_level(g, i, nullptr, nullptr, g.n, 0, s, 0, 1);
         if (rc) return rc;
@@ -677,7 +691,7 @@ int start_peel(Graph& g, bool sampled, cudaStream_t s) {
         launch_stale_exact(g, nullptr, nullptr, s);
     }
     const LbArgs la = lb_args(g);
-    k_min_lb<<<grid, kPeelThreads, 0, s>>>(g.alive, g.fresh, g.n, la, g.state, peel_state(g));
+    k_min_lb<<<grid, kPeelThreads, 0, s>>>(g.alive, g.fresh, g.n, la, g.state, peel_state(g, sampled));
     count_launch(g, 1);
     rc = refine(g, sampled, s);
     if (rc) return rc;
@@ -694,7 +708,7 @@ int start_peel(Graph& g, bool sampled, cudaStream_t s) {
 // affects, then the end of the round.
 int refresh_and_finish(Graph& g, bool sampled, cudaStream_t s) {
     const int grid = peel_grid(g);
-    const PeelState ps = peel_state(g);
+    const PeelState ps = peel_state(g, sampled);
     int rc = KH_OK;
     if (!sampled) {
         // the ball of R in the old graph: alive degrees drop (hop 1), the
@@ -745,7 +759,7 @@ int launch_round(Graph& g, bool sampled, cudaStream_t s) {
             k_dense_sum<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.d32, g.vcount, g.vlist,
                                                                g.state, g.dsum, g.n + 1);
         k_select_sched<<<grid, kPeelThreads, 0, s>>>(g.alive, g.sched, g.vcount, g.vlist, g.state,
-                                                     g.listR, g.seen, g.round_of);
+                                                     peel_state(g, sampled), g.listR, g.seen, g.round_of);
         count_launch(g, 2);
         prof_end(g, kProfPeel, s);
         return refresh_and_finish(g, sampled, s);
@@ -764,7 +778,7 @@ int launch_round(Graph& g, bool sampled, cudaStream_t s) {
     rc = refine(g, sampled, s);
     if (rc) return rc;
     prof_begin(g, kProfPeel, s);
-    const PeelState ps = peel_state(g);
+    const PeelState ps = peel_state(g, sampled);
     if (sampled) {
         k_select<unsigned long long, unsigned long long><<<grid, kPeelThreads, 0, s>>>(
             g.alive, g.d64, g.vcount, g.vlist, g.state, ps, g.core64, g.round_of, g.listR, g.seen);
@@ -841,6 +855,7 @@ int run_estimate_all(Graph& g) {
     if (rc) return rc;
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.alive, 1, (size_t)g.n, s));
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(&g.state->err, 0, sizeof(int), s));
+    KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.meta, 0, sizeof(uint32_t) * (size_t)g.hmax * (size_t)g.n, s));
     for (int i = 1; i <= g.hmax && rc == KH_OK; ++i)
         rc = launch_level(g, i, nullptr, nullptr, g.n, 0, s, 0, 0);
     if (rc) return rc;

@@ -7,19 +7,26 @@
 // smallest level whose rank-filtered N(v;i,X) has at most M members, so B and
 // k depend only on the alive set, the ranks and M.
 //
-// Level 1 (T = {v} plus alive neighbours, no repeats): one warp per node, a
-// 32-bin rank histogram, kappa from its suffix sums, a second pass writes the
-// members grouped by rank.
+// Positions.  Nodes are numbered by descending rank (k_pos_*): every node has a
+// position, the positions of one rank class start at a multiple of 32, and
+// the nodes of rank >= j occupy the first clsw[j] 32-bit words of a bitmap over
+// positions.  A list key is r << 27 | position.
 //
-// Levels >= 2: one CTA per node with an open-addressing hash set of packed keys
-// (r << 27 | id) in shared memory.  Warps stream the neighbours' lists
-// (coalesced 32-key chunks).  A running threshold t starts at max_w k[w,i-1];
-// keys below t are skipped, and because each list is grouped by rank from the
-// highest, a warp stops reading a list at its first key below t.  After every
-// chunk step the CTA raises t to the smallest level whose count of distinct
-// keys is <= M (Alg. 5's trim), and compacts the set when dead entries pile
-// up.  The last level only needs |B[v,h]| and k[v,h] for the estimate of
-// Alg. 1, so it writes no list.
+// A stored list has one of two forms (a flag in its meta word): sparse, |B| keys
+// grouped by rank, highest first; or dense, the first clsw[k] words of the
+// bitmap over positions, when those are fewer words than |B| (a ball of more
+// than about n/32 nodes).
+//
+// Level 1 (T = {v} plus alive neighbours, no repeats): one warp per node, the
+// counts S_j by ballots, kappa from them, a second pass writes the members
+// grouped by rank.
+//
+// Levels >= 2: one CTA per node (k_levelU, see there).  A running threshold t
+// starts at max_w k[w,i-1]; keys below t are skipped, and because each list is
+// ordered by rank from the highest, a list is left at its first key below t.
+// As the union grows t rises to the smallest level whose count of distinct
+// members is <= M (Alg. 5's trim).  The last level only needs |B[v,h]| and
+// k[v,h] for the estimate of Alg. 1, so it writes no list.
 //
 // A node's (|B|, k) pair changes exactly when B[v,i] or k[v,i] changes: with k
 // fixed, the new list is a subset of the old one (nodes only leave), so equal
@@ -31,15 +38,40 @@ namespace kh {
 namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
-constexpr uint32_t kEmpty = 0xffffffffu;
 constexpr int kL1Threads = 256;
-constexpr int kLuThreads = 256;
+constexpr int kLuThreads = 128;
+constexpr int kLuWarps = kLuThreads / 32;
+constexpr int kLuPerSm = 12;  // CTAs per SM of k_levelU
+
+// Meta word of a list (one per level and node): |B| in bits 0-13, k in bits
+// 14-19, the highest rank present in bits 20-24, the dense-form flag, and a
+// flag that is set while the node is alive (a removed node's word is zero).
+constexpr uint32_t kMetaAlive = 1u << 31;
+constexpr uint32_t kMetaDense = 1u << 30;
+__device__ __forceinline__ int meta_size(uint32_t m) { return (int)(m & 0x3fffu); }
+__device__ __forceinline__ int meta_k(uint32_t m) { return (int)((m >> 14) & 63u); }
+__device__ __forceinline__ int meta_top(uint32_t m) { return (int)((m >> 20) & 31u); }
+__device__ __forceinline__ uint32_t meta_pack(int S, int k, int top, bool dense) {
+    return kMetaAlive | (dense ? kMetaDense : 0u) | ((uint32_t)top << 20) | ((uint32_t)k << 14) |
+           (uint32_t)S;
+}
+constexpr uint32_t kMetaSizeK = (1u << 20) - 1u;  // the (|B|, k) part
+
+// First word of a graph's part of wrank (graph q of a batch; its positions are
+// local to the graph).  A graph of n' nodes needs at most n'/32 + 32 words.
+// (A multiple of 4: wrank is read four words at a time.)
+__host__ __device__ __forceinline__ int64_t word_base(int64_t first_node, int64_t q) {
+    return ((first_node >> 5) + 36 * q + 3) & ~(int64_t)3;
+}
 
 struct LevelArgs {
     const int64_t* rowptr;
     const int32_t* col;
     const uint8_t* alive;
-    const uint8_t* rank;
+    const uint32_t* key32;     // r << 27 | position of each node
+    const int32_t* clsw;       // per graph 33 entries: words covering the ranks >= j
+    const uint8_t* wrank;      // rank class of each bitmap word
+    const int64_t* vtx_off;    // batches: first node of each graph
     int64_t n;
     int level;                 // level to compute; 0: each node's last level h(v)
     int h;                     // h of every node when hv is nullptr
@@ -49,20 +81,19 @@ struct LevelArgs {
     const int32_t* Mv;         // per-node M (batches)
     int64_t cap;
     uint32_t* keys;            // level i lists at keys + (i-1) n cap
-    int32_t* lsz;              // |B[v,i]| at lsz + (i-1) n
-    uint8_t* lk;               // k[v,i] at lk + (i-1) n
-    uint8_t* ltop;             // highest rank in B[v,i] at ltop + (i-1) n, stored levels only
+    uint32_t* meta;            // level i meta words at meta + (i-1) n
     unsigned long long* est;   // estimate (at a node's last level)
     const int32_t* worklist;
     const int* d_count;
     int64_t count_static;
     int track;
-    int group_lists;           // free union: lane groups per list (0: a warp per list)
-    int group_div;             // grouped: a group covers 1/group_div of the expected keys
+    int group_lists;           // union: lane groups per list (0: a warp per list)
+    int group_shift;           // a group covers 1/2^group_shift of the expected keys
+    int lg;                    // hash form of the union's set: 2^lg slots
+    int bm_words;              // bitmap form: words that fit (0: never)
+    uint32_t* stage;           // per CTA: cap keys (compaction of the hash form)
     int32_t* changed;
     int* n_changed;
-    int32_t* heavy;            // level 1: nodes of degree > kL1Heavy, for the CTA kernel
-    int* n_heavy;
     int* work_ctr;
     int* err;
     unsigned long long* updates;
@@ -81,12 +112,11 @@ struct LevelArgs {
     unsigned long long* stopped;
     int8_t* rho;  // tracked passes: top rank of each changed list's changes
     unsigned long long* min_done;  // refine: per-graph minimum of the completed values
-    // split heavy nodes (k_levelU): partial sets of cap keys per part slot,
-    // their sizes and levels, parts finished per split node (at its first
-    // slot), each heavy node's first slot, the part items (part_cap 0: no split)
+    // split heavy nodes (k_levelU): partial sets of cap words per part slot,
+    // their meta words, parts finished per split node (at its first slot),
+    // each heavy node's first slot, the part items (part_cap 0: no split)
     uint32_t* part_keys;
-    int32_t* part_size;
-    uint8_t* part_t;
+    uint32_t* part_meta;
     int32_t* part_done;
     int32_t* part_stop;             // per split node: some part stopped early (refine)
     unsigned long long* part_lb;    // per split node: the largest partial estimate above T
@@ -98,10 +128,14 @@ struct LevelArgs {
 };
 
 constexpr int kL1Heavy = 512;
+constexpr int kL1BlockHeavy = 64;
 // k_levelU splits nodes of more than kSplitDeg neighbours into parts of
-// kSplitChunk neighbours each
-constexpr int kSplitDeg = 4096;
-constexpr int kSplitChunk = 2048;
+// kSplitChunk neighbours each.  One CTA reads 2048 lists in about 40 us, as long
+// as a whole launch of a middle round; below that the parts' own set-up costs
+// more than the shorter tail gives (sampled (k,3)-cores of Chung-Lu n = 200k /
+// R-MAT 18: 688 / 311 ms with 4096 and 2048, 659 / 297 ms with 2048 and 512).
+constexpr int kSplitDeg = 2048;
+constexpr int kSplitChunk = 512;
 
 // What one node computes in this launch: its level, whether that is its last
 // level h(v) (estimate) or an intermediate one (list), its M, and where its
@@ -110,15 +144,11 @@ struct NodeLevel {
     int lvl;
     bool last;
     bool skip;
-    int64_t M;
+    int M;
     const uint32_t* keys_in;
-    uint32_t* keys_out;
-    const int32_t* lsz_in;
-    const uint8_t* lk_in;
-    const uint8_t* ltop_in;
-    int32_t* lsz_out;
-    uint8_t* lk_out;
-    uint8_t* ltop_out;  // nullptr at a node's last level (no list is stored)
+    uint32_t* keys_out;  // nullptr at a node's last level (no list is stored)
+    const uint32_t* meta_in;
+    uint32_t* meta_out;
 };
 
 __device__ __forceinline__ NodeLevel node_level(const LevelArgs& a, int v) {
@@ -127,17 +157,13 @@ __device__ __forceinline__ NodeLevel node_level(const LevelArgs& a, int v) {
     nl.lvl = a.level ? a.level : hvv;
     nl.last = nl.lvl == hvv;
     nl.skip = nl.lvl > hvv || (nl.last && a.skip_last);
-    nl.M = a.Mv ? (int64_t)a.Mv[v] : a.M;
+    nl.M = a.Mv ? a.Mv[v] : (int)a.M;
     const size_t nn = (size_t)a.n, lc = nn * (size_t)a.cap;
     const int L = nl.lvl;
     nl.keys_in = L >= 2 ? a.keys + (size_t)(L - 2) * lc : nullptr;
     nl.keys_out = (!nl.last && a.keys) ? a.keys + (size_t)(L - 1) * lc : nullptr;
-    nl.lsz_in = L >= 2 ? a.lsz + (size_t)(L - 2) * nn : nullptr;
-    nl.lk_in = L >= 2 ? a.lk + (size_t)(L - 2) * nn : nullptr;
-    nl.ltop_in = L >= 2 ? a.ltop + (size_t)(L - 2) * nn : nullptr;
-    nl.lsz_out = a.lsz + (size_t)(L - 1) * nn;
-    nl.lk_out = a.lk + (size_t)(L - 1) * nn;
-    nl.ltop_out = (!nl.last && a.ltop) ? a.ltop + (size_t)(L - 1) * nn : nullptr;
+    nl.meta_in = L >= 2 ? a.meta + (size_t)(L - 2) * nn : nullptr;
+    nl.meta_out = a.meta + (size_t)(L - 1) * nn;
     return nl;
 }
 
@@ -152,39 +178,34 @@ __device__ __forceinline__ unsigned long long estimate_of(int S, int kappa, int 
     return d;
 }
 
-__device__ __forceinline__ void record_change(const LevelArgs& a, const NodeLevel& nl, int v, int S,
-                                              int kappa) {
-    const int old_s = nl.lsz_out[v];
-    const int old_k = nl.lk_out[v];
-    nl.lsz_out[v] = S;
-    nl.lk_out[v] = (uint8_t)kappa;
-    if (a.track) atomicAdd(a.lvl_work + nl.lvl, 1ull);
-    if (a.track && (old_s != S || old_k != kappa)) {
+__device__ __forceinline__ void record_change(const LevelArgs& a, const NodeLevel& nl, int v,
+                                              uint32_t m) {
+    const uint32_t old = nl.meta_out[v];
+    nl.meta_out[v] = m;
+    if (!a.track) return;
+    atomicAdd(a.lvl_work + nl.lvl, 1ull);
+    if ((old ^ m) & kMetaSizeK) {
         atomicAdd(a.lvl_changed + nl.lvl, 1ull);
         const int p = atomicAdd(a.n_changed, 1);
         if (p < a.n) a.changed[p] = v;
     }
 }
 
-// rho of a tracked list about to be rewritten with (S, kappa): -2 when it is
-// unchanged (same size and level imply the same members, as the level never
-// rises and a list only gains members below its old level), else the highest
-// rank among the members that left and, if the level fell, old level - 1 (the
-// members that entered rank below the old level).  At level 1 the members that
-// leave are exactly the removed ones.  Warp-wide; every lane gets the result.
-__device__ __forceinline__ int level1_rho_warp(const LevelArgs& a, const NodeLevel& nl, int v,
-                                               int S, int kappa, int lane) {
-    const int old_s = nl.lsz_out[v], old_k = nl.lk_out[v];
-    if (old_s == S && old_k == kappa) return -2;
+// rho of a tracked list about to be rewritten with (S, kappa): the highest rank
+// among the members that left and, if the level fell, old level - 1 (the
+// members that entered rank below the old level); a list with the same size
+// and level is unchanged and keeps none.  At level 1 the members that leave are
+// exactly the neighbours removed in this round (alive == 2): a removal
+// refreshes every neighbour's level-1 list in its round.  dead_top: the highest
+// rank among those neighbours (-1: none).
+__device__ __forceinline__ void level1_rho(const LevelArgs& a, const NodeLevel& nl, int v, int S,
+                                           int kappa, int dead_top) {
+    const uint32_t old = nl.meta_out[v];
+    const int old_k = meta_k(old);
+    if (meta_size(old) == S && old_k == kappa) return;
     int r = kappa != old_k ? old_k - 1 : -1;
-    const uint32_t* old = nl.keys_out + (size_t)v * (size_t)a.cap;
-    const int m = min(old_s, (int)a.cap);
-    for (int p = lane; p < m; p += 32) {
-        const uint32_t key = old[p];
-        if (a.alive[key & kIdMask] != 1) r = max(r, (int)(key >> kIdBits));
-    }
-    for (int off = 16; off > 0; off >>= 1) r = max(r, __shfl_xor_sync(kFull, r, off));
-    return r;
+    if (dead_top >= old_k) r = max(r, dead_top);
+    a.rho[v] = (int8_t)r;
 }
 
 // Bytes a node's level-1 computation must move: row offsets, the row, the
@@ -193,81 +214,104 @@ __device__ __forceinline__ unsigned long long level1_bytes(int64_t deg, int S, i
     return 8ull + 5ull * (unsigned long long)deg + (last ? 8ull : 4ull * (unsigned long long)S) + 5ull;
 }
 
+// Lane j adds #{lanes : r >= j} to its count (r = -1: no key).  Ranks are
+// geometric, so a warp's 32 keys need about 7 ballots (no shared-memory
+// atomics: half the keys of a histogram would fall on one address).
+__device__ __forceinline__ void add_rank_counts(int r, int lane, int& S) {
+#pragma unroll 1
+    for (int j = 0; j < 32; ++j) {
+        const uint32_t b = __ballot_sync(kFull, r >= j);
+        if (!b) break;
+        if (lane == j) S += __popc(b);
+    }
+}
+
+// kappa, the list size at kappa and the highest rank present from the counts
+// S_j held by lane j.
+__device__ __forceinline__ void level_of_counts(int S, int M, int& kappa, int& Skap, int& top) {
+    const uint32_t over = __ballot_sync(kFull, S > M);
+    kappa = over ? 32 - __clz(over) : 0;
+    const int Sk = __shfl_sync(kFull, S, kappa & 31);
+    Skap = kappa < 32 ? Sk : 0;
+    const uint32_t nz = __ballot_sync(kFull, S > 0);
+    top = nz ? 31 - __clz(nz) : 0;
+}
+
+// Level 1.  One warp per node; rows longer than kL1Heavy are gathered per block
+// and done by all its warps after the warp-per-node pass.
 __global__ void __launch_bounds__(kL1Threads) k_level1(LevelArgs a) {
-    __shared__ int s_hist[kL1Threads / 32][32];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    int* hist = s_hist[wib];
+    __shared__ int s_off[kL1Threads / 32][32];
+    __shared__ int s_heavy[kL1BlockHeavy];
+    __shared__ int s_nheavy, s_kappa, s_S, s_top, s_dead;
+    __shared__ int s_cnt[32];
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    int* off = s_off[wib];
     const int64_t total = a.worklist ? (int64_t)(*a.d_count) : a.count_static;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     unsigned long long my_bytes = 0;
-    for (int64_t idx = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; idx < total; idx += nw) {
+    if (tid == 0) s_nheavy = 0;
+    __syncthreads();
+    for (int64_t idx = ((int64_t)blockIdx.x * blockDim.x + tid) >> 5; idx < total; idx += nw) {
         const int v = a.worklist ? a.worklist[idx] : (int)idx;
         if (a.alive[v] != 1) continue;
         const NodeLevel nl = node_level(a, v);
         if (nl.skip || nl.lvl != 1) continue;
         const int64_t b = a.rowptr[v], e = a.rowptr[v + 1];
         if (e - b > kL1Heavy) {
-            if (lane == 0) {
-                const int p = atomicAdd(a.n_heavy, 1);
-                if (p < a.n) a.heavy[p] = v;
+            int slot = 0;
+            if (lane == 0) slot = atomicAdd(&s_nheavy, 1);
+            slot = __shfl_sync(kFull, slot, 0);
+            if (slot < kL1BlockHeavy) {
+                if (lane == 0) s_heavy[slot] = v;
+                continue;
             }
-            continue;
         }
-        hist[lane] = 0;
-        __syncwarp();
+        const uint32_t kv = a.key32[v];
+        const int rv = (int)(kv >> kIdBits);
+        int S = rv >= lane ? 1 : 0, dead = -1;
         for (int64_t k0 = b; k0 < e; k0 += 32) {
-            const int64_t k = k0 + lane;
-            if (k < e) {
-                const int32_t u = a.col[k];
-                if (a.alive[u] == 1) atomicAdd(&hist[a.rank[u]], 1);
+            int r = -1;
+            if (k0 + lane < e) {
+                const int32_t u = a.col[k0 + lane];
+                const int au = a.alive[u];
+                const int ru = (int)(a.key32[u] >> kIdBits);
+                if (au == 1) r = ru;
+                if (au == 2) dead = max(dead, ru);
             }
+            add_rank_counts(r, lane, S);
         }
-        const int rv = a.rank[v];
-        if (lane == 0) atomicAdd(&hist[rv], 1);
-        __syncwarp();
-        // S_j = #{u in T : r[u] >= j}, lane j holds S_j
-        int S = hist[lane];
-        for (int off = 1; off < 32; off <<= 1) {
-            const int t = __shfl_down_sync(kFull, S, off);
-            if (lane + off < 32) S += t;
-        }
-        const uint32_t over = __ballot_sync(kFull, S > nl.M);
-        const int kappa = over ? 32 - __clz(over) : 0;
-        const int Sk = __shfl_sync(kFull, S, kappa & 31);
-        const int Skap = kappa < 32 ? Sk : 0;
-        const uint32_t nz = __ballot_sync(kFull, S > 0);
-        const int top = nz ? 31 - __clz(nz) : 0;  // highest rank present
+        int kappa, Skap, top;
+        level_of_counts(S, nl.M, kappa, Skap, top);
         if (lane == 0) my_bytes += level1_bytes(e - b, Skap, nl.last);
         if (nl.last) {
             if (lane == 0) {
-                const unsigned long long e = estimate_of(Skap, kappa, rv, nl.M);
-                a.est[v] = e;
-                if (a.min_done) atomicMin(a.min_done + (a.gid ? a.gid[v] : 0), e);
-                record_change(a, nl, v, Skap, kappa);
+                const unsigned long long est = estimate_of(Skap, kappa, rv, nl.M);
+                a.est[v] = est;
+                if (a.min_done) atomicMin(a.min_done + (a.gid ? a.gid[v] : 0), est);
+                record_change(a, nl, v, meta_pack(Skap, kappa, top, false));
                 atomicAdd(a.updates, 1ull);
             }
             continue;
         }
         if (a.track) {
-            // rho: the old list is read before it is overwritten
-            const int r = level1_rho_warp(a, nl, v, Skap, kappa, lane);
-            if (lane == 0 && r > -2) a.rho[v] = (int8_t)r;
+            dead = __reduce_max_sync(kFull, dead);
+            if (lane == 0) level1_rho(a, nl, v, Skap, kappa, dead);
         }
         // members grouped by rank, highest first: rank j starts at S_{j+1}
         const int above = __shfl_down_sync(kFull, S, 1);
         __syncwarp();
-        hist[lane] = lane < 31 ? above : 0;
+        off[lane] = lane < 31 ? above : 0;
         __syncwarp();
         uint32_t* out = nl.keys_out + (size_t)v * (size_t)a.cap;
         for (int64_t k0 = b; k0 < e; k0 += 32) {
-            const int64_t k = k0 + lane;
-            if (k < e) {
-                const int32_t u = a.col[k];
+            if (k0 + lane < e) {
+                const int32_t u = a.col[k0 + lane];
                 if (a.alive[u] == 1) {
-                    const int r = a.rank[u];
+                    const uint32_t key = a.key32[u];
+                    const int r = (int)(key >> kIdBits);
                     if (r >= kappa) {
-                        const int p = atomicAdd(&hist[r], 1);
-                        if (p < a.cap) out[p] = ((uint32_t)r << kIdBits) | (uint32_t)u;
+                        const int p = atomicAdd(&off[r], 1);
+                        if (p < a.cap) out[p] = key;
                         else atomicOr(a.err, kErrList);
                     }
                 }
@@ -275,197 +319,161 @@ __global__ void __launch_bounds__(kL1Threads) k_level1(LevelArgs a) {
         }
         if (lane == 0) {
             if (rv >= kappa) {
-                const int p = atomicAdd(&hist[rv], 1);
-                if (p < a.cap) out[p] = ((uint32_t)rv << kIdBits) | (uint32_t)v;
+                const int p = atomicAdd(&off[rv], 1);
+                if (p < a.cap) out[p] = kv;
                 else atomicOr(a.err, kErrList);
             }
-            if (nl.ltop_out) nl.ltop_out[v] = (uint8_t)top;
-            record_change(a, nl, v, Skap, kappa);
+            record_change(a, nl, v, meta_pack(Skap, kappa, top, false));
         }
         __syncwarp();
     }
-    for (int off = 16; off > 0; off >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, off);
-    if (lane == 0 && my_bytes) atomicAdd(a.bytes, my_bytes);
-}
-
-// Level 1 for the nodes of degree > kL1Heavy deferred by k_level1: one CTA per node.
-__global__ void __launch_bounds__(kL1Threads) k_level1_heavy(LevelArgs a) {
-    __shared__ int s_hist[32];
-    __shared__ int s_kappa, s_S, s_top;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int nh = *a.n_heavy;
-    for (int idx = blockIdx.x; idx < nh; idx += gridDim.x) {
-        const int v = a.heavy[idx];
-        const NodeLevel nl = node_level(a, v);  // deferred by k_level1: level 1, not skipped
-        if (tid < 32) s_hist[tid] = 0;
+    __syncthreads();
+    const int nh = min(s_nheavy, kL1BlockHeavy);
+    for (int j = 0; j < nh; ++j) {
+        const int v = s_heavy[j];
+        const NodeLevel nl = node_level(a, v);
+        if (tid < 32) s_cnt[tid] = 0;
+        if (tid == 0) s_dead = -1;
         __syncthreads();
         const int64_t b = a.rowptr[v], e = a.rowptr[v + 1];
-        for (int64_t k = b + tid; k < e; k += blockDim.x) {
-            const int32_t u = a.col[k];
-            if (a.alive[u] == 1) atomicAdd(&s_hist[a.rank[u]], 1);
+        const uint32_t kv = a.key32[v];
+        const int rv = (int)(kv >> kIdBits);
+        int S = wib == 0 && rv >= lane ? 1 : 0, dead = -1;
+        for (int64_t k0 = b + wib * 32; k0 < e; k0 += blockDim.x) {
+            int r = -1;
+            if (k0 + lane < e) {
+                const int32_t u = a.col[k0 + lane];
+                const int au = a.alive[u];
+                const int ru = (int)(a.key32[u] >> kIdBits);
+                if (au == 1) r = ru;
+                if (au == 2) dead = max(dead, ru);
+            }
+            add_rank_counts(r, lane, S);
         }
-        const int rv = a.rank[v];
-        if (tid == 0) atomicAdd(&s_hist[rv], 1);
+        if (S) atomicAdd(&s_cnt[lane], S);
+        if (a.track) {
+            dead = __reduce_max_sync(kFull, dead);
+            if (lane == 0 && dead >= 0) atomicMax(&s_dead, dead);
+        }
         __syncthreads();
         if (tid < 32) {
-            int S = s_hist[lane];
-            for (int off = 1; off < 32; off <<= 1) {
-                const int t = __shfl_down_sync(kFull, S, off);
-                if (lane + off < 32) S += t;
-            }
-            const uint32_t over = __ballot_sync(kFull, S > nl.M);
-            const int kappa = over ? 32 - __clz(over) : 0;
-            const int Sk = __shfl_sync(kFull, S, kappa & 31);
+            S = s_cnt[lane];
+            int kappa, Skap, top;
+            level_of_counts(S, nl.M, kappa, Skap, top);
             const int above = __shfl_down_sync(kFull, S, 1);
-            const uint32_t nz = __ballot_sync(kFull, S > 0);
-            s_hist[lane] = lane < 31 ? above : 0;
+            __syncwarp();
+            s_cnt[lane] = lane < 31 ? above : 0;
             if (lane == 0) {
                 s_kappa = kappa;
-                s_S = kappa < 32 ? Sk : 0;
-                s_top = nz ? 31 - __clz(nz) : 0;
+                s_S = Skap;
+                s_top = top;
             }
         }
         __syncthreads();
         const int kappa = s_kappa, Skap = s_S;
         if (nl.last) {
             if (tid == 0) {
-                const unsigned long long e = estimate_of(Skap, kappa, rv, nl.M);
-                a.est[v] = e;
-                if (a.min_done) atomicMin(a.min_done + (a.gid ? a.gid[v] : 0), e);
-                record_change(a, nl, v, Skap, kappa);
+                const unsigned long long est = estimate_of(Skap, kappa, rv, nl.M);
+                a.est[v] = est;
+                if (a.min_done) atomicMin(a.min_done + (a.gid ? a.gid[v] : 0), est);
+                record_change(a, nl, v, meta_pack(Skap, kappa, s_top, false));
                 atomicAdd(a.updates, 1ull);
-                atomicAdd(a.bytes, level1_bytes(e - b, Skap, 1));
+                my_bytes += level1_bytes(e - b, Skap, 1);
             }
         } else {
-            if (a.track && tid < 32) {
-                // rho (one warp); the old list is read before it is overwritten
-                const int r = level1_rho_warp(a, nl, v, Skap, kappa, lane);
-                if (lane == 0 && r > -2) a.rho[v] = (int8_t)r;
-            }
-            __syncthreads();
+            if (a.track && tid == 0) level1_rho(a, nl, v, Skap, kappa, s_dead);
             uint32_t* out = nl.keys_out + (size_t)v * (size_t)a.cap;
             for (int64_t k = b + tid; k < e; k += blockDim.x) {
                 const int32_t u = a.col[k];
                 if (a.alive[u] == 1) {
-                    const int r = a.rank[u];
+                    const uint32_t key = a.key32[u];
+                    const int r = (int)(key >> kIdBits);
                     if (r >= kappa) {
-                        const int p = atomicAdd(&s_hist[r], 1);
-                        if (p < a.cap) out[p] = ((uint32_t)r << kIdBits) | (uint32_t)u;
+                        const int p = atomicAdd(&s_cnt[r], 1);
+                        if (p < a.cap) out[p] = key;
                         else atomicOr(a.err, kErrList);
                     }
                 }
             }
             if (tid == 0) {
                 if (rv >= kappa) {
-                    const int p = atomicAdd(&s_hist[rv], 1);
-                    if (p < a.cap) out[p] = ((uint32_t)rv << kIdBits) | (uint32_t)v;
+                    const int p = atomicAdd(&s_cnt[rv], 1);
+                    if (p < a.cap) out[p] = kv;
                     else atomicOr(a.err, kErrList);
                 }
-                if (nl.ltop_out) nl.ltop_out[v] = (uint8_t)s_top;
-                record_change(a, nl, v, Skap, kappa);
-                atomicAdd(a.bytes, level1_bytes(e - b, Skap, 0));
+                record_change(a, nl, v, meta_pack(Skap, kappa, s_top, false));
+                my_bytes += level1_bytes(e - b, Skap, 0);
             }
         }
         __syncthreads();
     }
+    for (int o = 16; o > 0; o >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, o);
+    if (lane == 0 && my_bytes) atomicAdd(a.bytes, my_bytes);
 }
+
+// ---- levels >= 2: the union of the neighbours' lists -------------------------
 
 // A flag another CTA of this launch may set (read past the L1 cache).
 __device__ __forceinline__ int ld_acquire(const int32_t* p) {
     return *(volatile const int32_t*)p;
 }
 
-// Insert `key` into the shared hash set; returns its slot if it was not
-// there, -1 if it was (or the probe limit was reached).
-__device__ __forceinline__ int set_insert(uint32_t* tab, int lg, uint32_t key, int* err) {
-    const uint32_t mask = (1u << lg) - 1u;
+// Hash form of the set: open addressing, a slot holds ~key (0: empty).
+// Returns whether `key` was new.
+__device__ __forceinline__ bool set_insert(uint32_t* tab, int lg, uint32_t key, int* err) {
+    const uint32_t mask = (1u << lg) - 1u, x = ~key;
     uint32_t s = ((key & kIdMask) * 0x9E3779B1u) >> (32 - lg);
+#pragma unroll 1
     for (uint32_t probe = 0; probe <= mask; ++probe) {
         // most keys of a union are repeats: a plain read settles them without an atomic
         const uint32_t cur = *(volatile uint32_t*)(tab + s);
-        if (cur == key) return -1;
-        if (cur == kEmpty) {
-            const uint32_t prev = atomicCAS(tab + s, kEmpty, key);
-            if (prev == kEmpty) return (int)s;
-            if (prev == key) return -1;
+        if (cur == x) return false;
+        if (cur == 0u) {
+            const uint32_t prev = atomicCAS(tab + s, 0u, x);
+            if (prev == 0u) return true;
+            if (prev == x) return false;
         }
         s = (s + 1u) & mask;
     }
     atomicOr(err, kErrProbe);
-    return -1;
+    return false;
 }
 
-// Whether `key` is in the shared hash set (linear probing, no deletions
-// between rebuilds).
+// Whether `key` is in the hash form (linear probing, no deletions between rebuilds).
 __device__ __forceinline__ bool set_contains(const uint32_t* tab, int lg, uint32_t key) {
-    const uint32_t mask = (1u << lg) - 1u;
+    const uint32_t mask = (1u << lg) - 1u, x = ~key;
     uint32_t s = ((key & kIdMask) * 0x9E3779B1u) >> (32 - lg);
+#pragma unroll 1
     for (uint32_t probe = 0; probe <= mask; ++probe) {
-        const uint32_t x = tab[s];
-        if (x == key) return true;
-        if (x == kEmpty) return false;
+        const uint32_t cur = tab[s];
+        if (cur == x) return true;
+        if (cur == 0u) return false;
         s = (s + 1u) & mask;
     }
     return false;
 }
 
-// Grouped union: a lane group's step covers 1/kGroupDivDefault of the keys a
-// list is expected to give (the rest take further steps).
-constexpr int kGroupDivDefault = 1;
+constexpr int kKeysPerLane = 4;  // words one lane loads per step (one 16-byte vector)
 
-// Keys one thread loads per step (one 16-byte vector); a warp's chunk.
-constexpr int kKeysPerLane = 4;
-constexpr int kChunkKeys = 32 * kKeysPerLane;
-// Nodes up to this degree use the flat (list, chunk) schedule of k_levelU.
-constexpr int kFlatMax = kLuThreads;
+// Lists of a chunk of kLuThreads neighbours, by how a warp reads them: short
+// ones (up to about 8 keys expected at or above t: 2 lanes a list), middle
+// (up to 64: 8 lanes), long (a warp a list) and dense (8 lanes).
+constexpr int kBuckets = 4;
+constexpr int kShort = 0, kMiddle = 1, kDense = 2, kLong = 3;
 
-// Shared memory of k_levelU for a table of 2^lg slots: keys, the compaction
-// stage (scap keys: a compaction keeps the keys at or above the level trimmed
-// from the complete counts, at most M), and the list of used slots (16-bit
-// indices; a set holds at most half its slots plus what the warps insert
-// before they stop for a compaction, under 2048).
-__host__ __device__ __forceinline__ int levelU_used_cap(int hcap) { return (hcap >> 1) + 2048; }
-
-int levelU_stage_cap(int lg, int64_t M) {
-    const int64_t half = (int64_t)1 << (lg - 1);
-    const int64_t need = (M + 64 + 3) & ~(int64_t)3;
-    return (int)(need < half ? need : half);
-}
-
-size_t levelU_smem(int lg, int scap) {
-    const size_t hcap = (size_t)1 << lg;
-    return hcap * 4 + (size_t)scap * 4 + (size_t)levelU_used_cap((int)hcap) * 2;
-}
-
-// Drop the keys below t from the hash set: empty their slots, re-insert the
-// rest (all threads of the CTA).
-__device__ __forceinline__ void compact_set(uint32_t* tab, uint32_t* stage, uint16_t* used, int lg,
-                                            int scap, int ucap, int tc, int* s_nused,
-                                            int* s_nstage, int* err) {
-    const int tid = threadIdx.x;
-    const int nu = min(*s_nused, ucap);
-    if (tid == 0) *s_nstage = 0;
-    __syncthreads();
-    for (int i = tid; i < nu; i += blockDim.x) {
-        const int slot = used[i];
-        const uint32_t key = tab[slot];
-        tab[slot] = kEmpty;
-        if ((int)(key >> kIdBits) >= tc) {
-            const int p = atomicAdd(s_nstage, 1);
-            if (p < scap) stage[p] = key;
-            else atomicOr(err, kErrProbe);
-        }
-    }
-    __syncthreads();
-    if (tid == 0) *s_nused = 0;
-    __syncthreads();
-    const int ns = min(*s_nstage, scap);
-    for (int i = tid; i < ns; i += blockDim.x) {
-        const int slot = set_insert(tab, lg, stage[i], err);
-        if (slot >= 0) used[atomicAdd(s_nused, 1)] = (uint16_t)slot;
-    }
-    __syncthreads();
-}
+// Shared state of one node's union.
+struct UnionShared {
+    int hist[32];                // distinct members per rank
+    int cls[33];                 // words covering the ranks >= j (this node's graph)
+    int t, tot, exit, creq, used, nstage, rho, last, off_done;
+    int kmax[kLuWarps];
+    int nq[kBuckets], cq[kBuckets];  // lists per bucket, lists claimed
+    unsigned long long T, part;  // early-stop threshold; partial estimate
+    int32_t w[kLuThreads];       // per neighbour of the chunk: its node (or list index)
+    uint16_t sz[kLuThreads];     //   and size
+    uint8_t q[kBuckets][kLuThreads];
+    int idx, v;                  // the CTA's next item
+};
 
 // The warp's view of the union's rank counts: lane j gets S_j = #{distinct
 // keys inserted so far with rank >= j}.  Read while other warps insert, the
@@ -481,173 +489,363 @@ __device__ __forceinline__ int snapshot_counts(const int* s_hist, int lane) {
     return S;
 }
 
-// The union of free-running warps (k_levelU<true>): the warps' lanes form
-// groups of G (G = 32: a warp per list); each group claims whole lists from a
-// shared counter and reads its list 4 G keys per step (four keys per lane)
-// until a key below the running level t shows (lists are grouped by rank,
-// highest first).  After every step the warp raises t from its snapshot of
-// the rank counts (Alg. 5's trim) and, in a refine, tests the partial
-// estimate against T.  The CTA meets at a barrier only to compact the set
-// (once it holds more than half its slots: at most one step per warp and one
-// more from each other warp follow before they stop, so the set never fills)
-// and at the end, where warp 0 trims from the complete counts.  Small groups
-// suit many lists that each give a few keys above t: a warp step then covers
-// 32 / G lists instead of one.
-// Returns true when the refine stopped early (s_part holds the bound).
-__device__ __forceinline__ bool free_union(const LevelArgs& a, const NodeLevel& nl, uint32_t* tab,
-                                        uint32_t* stage, uint16_t* used, int lg, int hcap,
-                                        int scap, int ucap,
-                                        int* s_hist, int* s_t, int* s_nused, int* s_nstage,
-                                        int* s_exit, unsigned long long* s_part, int* s_item,
-                                        int* s_creq, unsigned long long T, int vin, bool can_stop,
-                                        int mode, int first, int64_t b, int l0, int L, int rv,
-                                        int G, unsigned long long& my_bytes) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    if (tid == 0) {
-        *s_item = 0;
-        *s_creq = 0;
+// What the walk over a node's lists needs besides the shared state.
+struct UnionCtx {
+    uint32_t* tab;
+    const uint32_t* lists;   // list of neighbour w at lists + w cap
+    const uint8_t* wrank;    // rank class of the graph's bitmap words
+    int64_t cap;
+    int lg, M, rv, stop_first;   // stop_first: first part slot (mode 1 refine) or -1
+    bool hash, can_stop, vin, other;  // other: lists written by other CTAs of this launch (merge)
+    const int32_t* part_stop;
+    int* err;
+};
+
+// Read the chunk's lists, bucket by bucket (long and dense lists first: they
+// raise t most).  Groups of 2^lgG lanes claim a list and read it 4 words per
+// lane and step; a warp claims for all its idle groups at once.  Sparse lists end
+// at their first key below the running level t; dense lists at the last word of
+// the ranks >= t.  After a step that inserted, once the counts can matter, the
+// warp raises t from its snapshot of the rank counts (Alg. 5's trim) and, in a
+// refine, tests the partial estimate against T.  The bucket and the lane's open
+// list stay in (bk, li, pos), so that the hash form can stop for a compaction.
+// (One loop for all buckets, and no unrolling below: with a copy per bucket the
+// kernel outgrew the instruction cache, 18 of 33 stall cycles per instruction.)
+template <bool LAST, bool PARTS>
+__device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, int& bk, int& li, int& pos,
+                                           unsigned long long& my_bytes) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t* lp = nullptr;
+    int sz = 0;
+    if (li >= 0) {  // a list kept over a compaction
+        lp = c.lists + (size_t)sh.w[li] * (size_t)c.cap;
+        sz = sh.sz[li];
     }
-    __syncthreads();
-    // this group's open list (kept across a compaction): index (-1: none,
-    // -2: the last claim found no list left), position, size
-    int cli = -1, cpos = 0, csz = 0;
-    const uint32_t* clp = nullptr;
-    // every step claims a list or reads 4 keys of one: a bound on the steps
-    // that no correct run reaches (past it: error flag, and the union ends)
-    const long long cap64 = (long long)L * ((long long)a.cap / 4 + 2) + 4096;
-    int steps_left = cap64 < 0x7fffffffLL ? (int)cap64 : 0x7fffffff;
+#pragma unroll 1
     for (;;) {
-        for (;;) {
-            // one read for the whole warp: lanes that saw the flags at different
-            // moments would leave the loop apart and stall the warp's shuffles
-            int stop = 0;
-            if (lane == 0) stop = *(volatile int*)s_creq | *(volatile int*)s_exit;
-            if (__shfl_sync(kFull, stop, 0)) break;
-            if (--steps_left < 0) {
-                if (lane == 0) {
-                    atomicOr(a.err, kErrLoop);
-                    atomicCAS(s_exit, 0, 3);
-                }
-                break;
-            }
-            // groups without an open list claim the next lists (a list that
-            // turns out dead, or with nothing at or above t, is passed over)
-            for (int tries = 0; tries < 4; ++tries) {
-                const bool need = cli == -1;
-                const uint32_t nb = __ballot_sync(kFull, need && (lane & (G - 1)) == 0);
-                if (!nb) break;
-                const int lead = __ffs(nb) - 1;
-                int base = 0;
-                if (lane == lead) base = atomicAdd(s_item, __popc(nb));
-                base = __shfl_sync(kFull, base, lead);
-                int c = base + __popc(nb & ((1u << lane) - 1u)), sz = 0, w = -1;
-                if (need && (lane & (G - 1)) == 0 && c < L) {
-                    if (mode == 2) {
-                        sz = __ldcg(a.part_size + first + c);
-                    } else {
-                        w = a.col[b + l0 + c];
-                        // a list whose highest rank is below t has nothing to give
-                        if (a.alive[w] == 1 && (int)nl.ltop_in[w] >= *(volatile int*)s_t)
-                            sz = min(nl.lsz_in[w], (int)a.cap);
-                    }
-                }
-                const int src = lane & ~(G - 1);
-                c = __shfl_sync(kFull, c, src);
-                sz = __shfl_sync(kFull, sz, src);
-                w = __shfl_sync(kFull, w, src);
-                if (need) {
-                    if (c >= L) {
-                        cli = -2;
-                    } else if (sz > 0) {
-                        cli = l0 + c;
-                        cpos = 0;
-                        csz = sz;
-                        clp = mode == 2 ? a.part_keys + (size_t)(first + c) * (size_t)a.cap
-                                        : nl.keys_in + (size_t)w * (size_t)a.cap;
-                    }
+        // one read for the whole warp: lanes that saw a flag at different
+        // moments would part ways before the ballots
+        int stop = 0;
+        if (lane == 0) stop = *(volatile int*)&sh.exit | *(volatile int*)&sh.creq;
+        if (__shfl_sync(kFull, stop, 0) || bk < 0) return;
+        const bool dense = bk == kDense;
+        const int lgG = bk == kLong ? 5 : bk == kShort ? 1 : 3;
+        const int lead = lane >> lgG << lgG;
+        const uint32_t need = __ballot_sync(kFull, li == -1 && lane == lead);
+        if (need) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&sh.cq[bk], __popc(need));
+            base = __shfl_sync(kFull, base, 0);
+            if (li == -1) {
+                const int i = base + __popc(need & ((1u << lead) - 1u));
+                li = -2;
+                if (i < sh.nq[bk]) {
+                    li = (int)sh.q[bk][i];
+                    pos = (lane - lead) * kKeysPerLane;
+                    lp = c.lists + (size_t)sh.w[li] * (size_t)c.cap;
+                    sz = sh.sz[li];
                 }
             }
-            if (__all_sync(kFull, cli == -2)) break;
-            const int t = *(volatile int*)s_t;
-            bool below = false;
-            const int p = cpos + (lane & (G - 1)) * kKeysPerLane;
-            if (cli >= 0 && p < csz) {
-                const uint4 k4 = mode == 2 ? __ldcg(reinterpret_cast<const uint4*>(clp + p))
-                                           : *reinterpret_cast<const uint4*>(clp + p);
+        }
+        if (__all_sync(kFull, li == -2)) {
+            do --bk;
+            while (bk >= 0 && sh.nq[bk] == 0);
+            if (bk < 0) return;
+            li = -1;
+            continue;
+        }
+        const int t = *(volatile int*)&sh.t;
+        int ins = 0;
+        bool done = false;
+        if (li >= 0) {
+            const int end = dense ? sh.cls[t] : sz;
+            if (pos < end) {
+                const uint4 k4 = PARTS && c.other ? __ldcg(reinterpret_cast<const uint4*>(lp + pos))
+                                         : *reinterpret_cast<const uint4*>(lp + pos);
                 const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
-                if (mode != 2) my_bytes += 4ull * (unsigned long long)min(kKeysPerLane, csz - p);
+                my_bytes += 4ull * (unsigned long long)min(kKeysPerLane, end - pos);
+                if (dense) {
 #pragma unroll
-                for (int q = 0; q < kKeysPerLane; ++q) {
-                    if (p + q < csz) {
-                        const uint32_t key = kk[q];
-                        const int r = (int)(key >> kIdBits);
-                        if (r >= t) {
-                            const int slot = set_insert(tab, lg, key, a.err);
-                            if (slot >= 0) {
-                                const int u = atomicAdd(s_nused, 1);
-                                if (u < ucap) used[u] = (uint16_t)slot;
-                                else atomicOr(a.err, kErrProbe);
-                                atomicAdd(&s_hist[r], 1);
+                    for (int q = 0; q < kKeysPerLane; ++q) {
+                        if (pos + q < end) {
+                            uint32_t nw = kk[q] & ~*(volatile uint32_t*)(c.tab + pos + q);
+                            if (nw) nw &= ~atomicOr(c.tab + pos + q, nw);
+                            if (nw) {
+                                atomicAdd(&sh.hist[c.wrank[pos + q]], __popc(nw));
+                                ins += __popc(nw);
                             }
+                        }
+                    }
+                } else if (!c.hash) {
+#pragma unroll
+                    for (int q = 0; q < kKeysPerLane; ++q) {
+                        const int r = pos + q < end ? (int)(kk[q] >> kIdBits) : -1;
+                        if (r < t) {
+                            done = true;
                         } else {
-                            below = true;
+                            uint32_t* wp = c.tab + ((kk[q] & kIdMask) >> 5);
+                            const uint32_t bit = 1u << (kk[q] & 31u);
+                            if (!(*(volatile uint32_t*)wp & bit) && !(atomicOr(wp, bit) & bit)) {
+                                atomicAdd(&sh.hist[r], 1);
+                                ++ins;
+                            }
+                        }
+                    }
+                } else {
+                    uint4 kq = k4;
+#pragma unroll 1
+                    for (int q = 0; q < kKeysPerLane; ++q) {
+                        const uint32_t key = kq.x;
+                        kq.x = kq.y;
+                        kq.y = kq.z;
+                        kq.z = kq.w;
+                        const int r = pos + q < end ? (int)(key >> kIdBits) : -1;
+                        if (r < t) {
+                            done = true;
+                            break;
+                        }
+                        if (set_insert(c.tab, c.lg, key, c.err)) {
+                            atomicAdd(&sh.hist[r], 1);
+                            ++ins;
                         }
                     }
                 }
             }
-            // ranks only fall along a list: after a key below t the rest is below t
-            const uint32_t bal = __ballot_sync(kFull, below);
-            if (cli >= 0) {
-                const uint32_t gmask = G == 32 ? kFull : (((1u << G) - 1u) << (lane & ~(G - 1)));
-                cpos += kKeysPerLane * G;
-                if ((bal & gmask) || cpos >= csz) cli = -1;
+            pos += kKeysPerLane << lgG;
+            done |= pos - (lane - lead) * kKeysPerLane >= end;  // the group's next step starts past the end
+        }
+        // ranks only fall along a list: after a key below t the rest is below t
+        const uint32_t fin = __ballot_sync(kFull, done) >> lead;
+        if (li >= 0 && (lgG == 5 ? fin : fin & ((1u << (1 << lgG)) - 1u))) li = -1;
+        if (!__any_sync(kFull, ins)) continue;
+        // members added: the trim and the early stop can only matter once the
+        // union holds more than M (k > 0) or more than T members
+        ins = __reduce_add_sync(kFull, ins);
+        int tot = 0;
+        if (lane == 0) {
+            tot = atomicAdd(&sh.tot, ins) + ins;
+            if (c.hash && atomicAdd(&sh.used, ins) + ins > (1 << (c.lg - 1))) *(volatile int*)&sh.creq = 1;
+        }
+        tot = __shfl_sync(kFull, tot, 0);
+        if (tot <= c.M && !(LAST && c.can_stop && (unsigned long long)tot > sh.T)) continue;
+        const int S = snapshot_counts(sh.hist, lane);
+        const uint32_t over = __ballot_sync(kFull, S > c.M);
+        const int pmax = over ? 31 - __clz(over) : -1;
+        if (pmax + 1 > t) {
+            const int Sn = __shfl_sync(kFull, S, (pmax + 1) & 31);
+            if (lane == 0) {
+                atomicMax(&sh.t, pmax + 1);
+                *(volatile int*)&sh.tot = pmax < 31 ? Sn : 0;
             }
-            // trim from this warp's snapshot; the early-stop test in a refine
-            const int S = snapshot_counts(s_hist, lane);
-            const uint32_t over = __ballot_sync(kFull, S > nl.M);
-            const int pmax = over ? 31 - __clz(over) : -1;
-            if (lane == 0 && pmax + 1 > t) atomicMax(s_t, pmax + 1);
-            if (can_stop) {
-                const int Sp = S + ((!vin && rv >= lane) ? 1 : 0);
-                const uint32_t fits = __ballot_sync(kFull, Sp <= nl.M);
-                const int k = fits ? __ffs(fits) - 1 : 32;
-                const int Sk = __shfl_sync(kFull, Sp, k & 31);
-                const unsigned long long pe = estimate_of(k < 32 ? Sk : 0, k, rv, nl.M);
-                if (lane == 0 && pe > T) {
-                    atomicMax(s_part, pe);
-                    atomicCAS(s_exit, 0, 1);
+        }
+        if (LAST && c.can_stop) {
+            // Def. 4.1 on the keys inserted so far plus v itself: a subset
+            // of N(v;h) led by v, so by Prop. 4.2 at most the final estimate
+            const int Sp = S + ((!c.vin && c.rv >= lane) ? 1 : 0);
+            const uint32_t fits = __ballot_sync(kFull, Sp <= c.M);
+            const int k = fits ? __ffs(fits) - 1 : 32;
+            const int Sk = __shfl_sync(kFull, Sp, k & 31);
+            const unsigned long long pe = estimate_of(k < 32 ? Sk : 0, k, c.rv, c.M);
+            if (lane == 0) {
+                if (pe > sh.T) {
+                    atomicMax(&sh.part, pe);
+                    atomicCAS(&sh.exit, 0, 1);
                 }
                 // a part stops too once another part of the node has shown d(v) > T
-                if (mode == 1 && lane == 0 && ld_acquire(a.part_stop + first)) atomicCAS(s_exit, 0, 2);
+                if (PARTS && c.stop_first >= 0 && ld_acquire(c.part_stop + c.stop_first))
+                    atomicCAS(&sh.exit, 0, 2);
             }
-            if (lane == 0 && *(volatile int*)s_nused > (hcap >> 1)) *(volatile int*)s_creq = 1;
         }
-        __syncthreads();
-        if (*(volatile int*)s_exit) return true;
-        if (!*(volatile int*)s_creq) break;  // every list claimed and read
-        // compaction: trim from the complete counts first, then drop keys below t
-        if (tid < 32) {
-            const int S = snapshot_counts(s_hist, lane);
-            const uint32_t over = __ballot_sync(kFull, S > nl.M);
-            const int pmax = over ? 31 - __clz(over) : -1;
-            if (lane == 0 && pmax + 1 > *s_t) *s_t = pmax + 1;
-        }
-        __syncthreads();
-        compact_set(tab, stage, used, lg, scap, ucap, *s_t, s_nused, s_nstage, a.err);
-        if (tid == 0) *s_creq = 0;
-        __syncthreads();
     }
-    // the level from the complete counts
-    if (tid < 32) {
-        const int S = snapshot_counts(s_hist, lane);
-        const uint32_t over = __ballot_sync(kFull, S > nl.M);
-        const int pmax = over ? 31 - __clz(over) : -1;
-        if (lane == 0 && pmax + 1 > *s_t) *s_t = pmax + 1;
-    }
-    __syncthreads();
-    return false;
 }
 
+// Compaction of the hash form: the keys at or above the level trimmed from the
+// complete counts (at most M) are staged in global memory and put back.
+__device__ __forceinline__ void compact_set(const LevelArgs& a, UnionShared& sh, uint32_t* tab, int M) {
+    const int tid = threadIdx.x, lane = tid & 31, C = 1 << a.lg;
+    const int S = snapshot_counts(sh.hist, lane);
+    const uint32_t over = __ballot_sync(kFull, S > M);
+    const int tc = max(sh.t, over ? 32 - __clz(over) : 0);
+    uint32_t* stage = a.stage + (size_t)blockIdx.x * (size_t)a.cap;
+    if (tid == 0) sh.nstage = 0;
+    __syncthreads();
+    if (tid == 0) sh.t = tc;
+#pragma unroll 1
+    for (int i = tid; i < C; i += kLuThreads) {
+        const uint32_t x = tab[i];
+        if (!x) continue;
+        tab[i] = 0u;
+        if ((int)(~x >> kIdBits) >= tc) {
+            const int p = atomicAdd(&sh.nstage, 1);
+            if (p < a.cap) stage[p] = ~x;
+            else atomicOr(a.err, kErrProbe);
+        }
+    }
+    __syncthreads();
+    const int ns = min(sh.nstage, (int)a.cap);
+#pragma unroll 1
+    for (int i = tid; i < ns; i += kLuThreads) set_insert(tab, a.lg, stage[i], a.err);
+    if (tid == 0) {
+        sh.used = ns;
+        sh.tot = ns;
+        sh.creq = 0;
+    }
+    __syncthreads();
+}
+
+// Write the finished union (members of rank >= kappa) as a list at `out` and
+// return its meta word.  hist must hold the complete counts; it is used up.
+// A bitmap with fewer words than members is stored as it is (dense form).
+// Otherwise the bitmap is read out in word order, which is rank order: each warp
+// takes a quarter of the words, four per lane and step, at the offset of the
+// earlier quarters' members.  The hash form goes by per-rank offsets.
+__device__ __forceinline__ uint32_t write_list(const LevelArgs& a, UnionShared& sh, const uint32_t* tab,
+                                               bool bm, const uint8_t* wrank, uint32_t* out, int S,
+                                               int kappa, int top) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (!bm) {
+        __syncthreads();
+        if (warp == 0) {  // start of each rank, highest first
+            const int c = lane >= kappa ? sh.hist[lane] : 0;
+            int incl = c;  // over the ranks >= lane
+            for (int off = 1; off < 32; off <<= 1) {
+                const int x = __shfl_down_sync(kFull, incl, off);
+                if (lane + off < 32) incl += x;
+            }
+            sh.hist[lane] = incl - c;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int i = tid; i < (1 << a.lg); i += kLuThreads) {
+            const uint32_t x = tab[i];
+            if (!x) continue;
+            const uint32_t key = ~x;
+            const int r = (int)(key >> kIdBits);
+            if (r < kappa) continue;
+            const int p = atomicAdd(&sh.hist[r], 1);
+            if (p < a.cap) out[p] = key;
+            else atomicOr(a.err, kErrList);
+        }
+        return meta_pack(S, kappa, top, false);
+    }
+    const int W = sh.cls[kappa];
+    if (W < S) {
+#pragma unroll 1
+        for (int i = tid; i < W; i += kLuThreads) out[i] = tab[i];
+        return meta_pack(S, kappa, top, true);
+    }
+    const int per = ((W + 4 * kLuThreads - 1) / (4 * kLuThreads)) * 128;  // words per warp
+    const int b = warp * per, e = min(W, b + per);
+    int cnt = 0;
+#pragma unroll 1
+    for (int i = b + lane; i < e; i += 32) cnt += __popc(tab[i]);
+    cnt = __reduce_add_sync(kFull, cnt);
+    if (lane == 0) sh.kmax[warp] = cnt;
+    __syncthreads();
+    int base = 0;
+    for (int i = 0; i < kLuWarps - 1; ++i) base += i < warp ? sh.kmax[i] : 0;
+#pragma unroll 1
+    for (int i0 = b; i0 < e; i0 += 128) {
+        const int i = i0 + lane * 4;
+        uint4 x = make_uint4(0u, 0u, 0u, 0u);
+        if (i < e) x = *reinterpret_cast<const uint4*>(tab + i);
+        if (i + 1 >= e) x.y = 0u;
+        if (i + 2 >= e) x.z = 0u;
+        if (i + 3 >= e) x.w = 0u;
+        const int c = __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+        int incl = c;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(kFull, incl, off);
+            if (lane >= off) incl += y;
+        }
+        int p = base + incl - c;
+        base += __shfl_sync(kFull, incl, 31);
+        if (!c) continue;
+        if (p + c > a.cap) {
+            atomicOr(a.err, kErrList);
+            continue;
+        }
+        const uint32_t rk = *reinterpret_cast<const uint32_t*>(wrank + i);  // ranks of the four words
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t key0 = (((rk >> (8 * q)) & 31u) << kIdBits) | ((uint32_t)(i + q) << 5);
+#pragma unroll 1
+            for (uint32_t y = x.x; y; y &= y - 1) out[p++] = key0 | (uint32_t)(__ffs(y) - 1);
+            x.x = x.y;
+            x.y = x.z;
+            x.z = x.w;
+        }
+    }
+    return meta_pack(S, kappa, top, false);
+}
+
+// Highest rank among the members of the old list (size, level and form in
+// `old`) that are not in the new union, where every member of rank >= the new
+// level (<= the old one) is kept; -1 if none left.
+__device__ __forceinline__ int lost_rank(const LevelArgs& a, const UnionShared& sh, const uint32_t* tab,
+                                         bool bm, int W0, const uint8_t* wrank,
+                                         const uint32_t* old_list, uint32_t old) {
+    const int tid = threadIdx.x;
+    int r = -1;
+    if (old & kMetaDense) {
+        const int W = bm ? min(sh.cls[meta_k(old)], W0) : sh.cls[meta_k(old)];
+#pragma unroll 1
+        for (int i = tid; i < W; i += kLuThreads) {
+            uint32_t x = old_list[i];
+            if (!x) continue;
+            const int rw = wrank[i];
+            if (rw <= r) break;  // the ranks of the words only fall
+            if (bm) {
+                if (x & ~tab[i]) r = rw;
+            } else {
+                for (; x; x &= x - 1)
+                    if (!set_contains(tab, a.lg, ((uint32_t)rw << kIdBits) | ((uint32_t)i << 5) |
+                                                     (uint32_t)(__ffs(x) - 1)))
+                        r = rw;
+            }
+        }
+    } else {
+        const int m = min(meta_size(old), (int)a.cap);
+#pragma unroll 1
+        for (int p = tid; p < m; p += kLuThreads) {
+            const uint32_t key = old_list[p];
+            const int rk = (int)(key >> kIdBits);
+            if (rk <= r) break;  // the ranks of the list only fall
+            const int w = (int)((key & kIdMask) >> 5);
+            const bool in = bm ? w < W0 && ((tab[w] >> (key & 31u)) & 1u) : set_contains(tab, a.lg, key);
+            if (!in) r = rk;
+        }
+    }
+    return r;
+}
+
+// Give a heavy node its part slots and part items (one thread).
+__device__ __forceinline__ void plan_parts(const LevelArgs& a, int v, int deg) {
+    const int P = (deg + kSplitChunk - 1) / kSplitChunk;
+    const int base = atomicAdd(a.n_sub, P);
+    if ((int64_t)base + P <= a.part_cap) {
+        for (int j = 0; j < P; ++j) {
+            a.sub_v[base + j] = v;
+            a.sub_j[base + j] = j;
+        }
+        a.split_first[v] = base;
+    } else {
+        // cannot happen: part_cap covers every heavy node of the graph at once
+        for (int64_t j = base; j < a.part_cap && j < (int64_t)base + P; ++j) a.sub_v[j] = -1;
+        atomicOr(a.err, kErrList);
+    }
+}
+
+// Levels >= 2, one CTA of 128 threads per node.
+//
+// The set of distinct members is a bitmap over positions in shared memory
+// when the words of the ranks >= t0 (t0 = max k[w,i-1], where the union
+// starts) fit, else an open-addressing hash set of keys.  In the bitmap an
+// insert is one shared load and, when new, one atomic OR: no probing, no list
+// of used slots and no compaction, and the output is in rank order by itself.
+// The neighbours' meta words are read once per chunk of 128 into shared
+// memory and sorted into buckets by what a list will give (walk_lists).
+//
 // Heavy nodes (degree > kSplitDeg) are split: part j unions the lists of
 // neighbours [j kSplitChunk, (j+1) kSplitChunk) into its own trimmed partial
 // set, and the CTA that finishes a node's last part merges the partial sets.
@@ -657,528 +855,335 @@ __device__ __forceinline__ bool free_union(const LevelArgs& a, const NodeLevel& 
 // some partial set, and for j >= t* = max_p t_p the counts S_j of the union of
 // the partial sets equal those of the full union.  The merge therefore runs the
 // same running-threshold union over the partial sets from t = t*.
-// FREE: the union's warps run free instead of in barrier-separated steps (see
-// the FREE branch below); both give the same lists.
-template <bool FREE>
-__global__ void __launch_bounds__(kLuThreads, 6) k_levelU(LevelArgs a, int lg, int scap) {
-    extern __shared__ __align__(16) uint32_t s_dyn[];
-    const int hcap = 1 << lg;
-    const int ucap = levelU_used_cap(hcap);
-    uint32_t* tab = s_dyn;
-    uint32_t* stage = s_dyn + hcap;                                         // scap keys
-    uint16_t* used = reinterpret_cast<uint16_t*>(s_dyn + hcap + scap);      // ucap slots
-    __shared__ int s_hist[32];
-    __shared__ int s_src, s_t, s_nused, s_nstage, s_compact;
-    __shared__ int s_vin, s_exit;                // own key in the table; early stop taken
-    __shared__ int s_rho, s_last;
-    __shared__ int s_item, s_creq;              // free mode: list claims; compaction request
-    __shared__ float s_ex;                      // grouped free mode: expected keys x 2^t
-    __shared__ unsigned long long s_T, s_part;  // early-stop threshold; partial estimate
-    // flat mode (degree <= kFlatMax): per neighbour list its node, size, first
-    // chunk index (exclusive prefix of 128-key chunk counts) and the first
-    // chunk that showed a key below t (INT_MAX while none has)
-    __shared__ int32_t s_w[kFlatMax];
-    __shared__ int32_t s_sz[kFlatMax];
-    __shared__ int32_t s_off[kFlatMax];
-    __shared__ int32_t s_dead[kFlatMax];
-    __shared__ int s_wsum[kLuThreads / 32];
-    __shared__ int s_total;
+//
+// What bounds it: instruction issue on whole-graph passes (81% issue-active on
+// the Chung-Lu n = 200k level-2 pass, 2.25 ms), latency in the rounds, whose
+// launches are a few nodes per CTA.  A node is a chain of dependent loads (its
+// row, the meta words, the lists) with little work between, so 12 CTAs of 128
+// threads and 16 KB (M <= 1638) keep 12 nodes per SM in flight; 256 threads
+// x 6 or 64 x 16 took 10-30% longer, and so did 25 KB of shared memory, which
+// would hold a bitmap of all 200k positions, with 8 CTAs.
+// Measured (start: one 256-thread CTA per node, hash set, 27 KB): estimates of
+// R-MAT 22 at h = 3 251 -> 78 ms, (k,3)-core of Chung-Lu n = 200k 1080 -> 659 ms,
+// (k,2)-core of Chung-Lu n = 50k at M = 1200 919 -> 538 ms.
+//
+// LAST: nodes at their last level (estimate, refine); LIST: nodes below it
+// (stored lists); PARTS: the parts of the split nodes, which the launch before
+// planned.  One kernel for all of it runs out of the instruction cache.
+template <bool LAST, bool LIST, bool PARTS>
+__global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
+    extern __shared__ __align__(16) uint32_t tab[];
+    __shared__ UnionShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nwarps = kLuThreads / 32;
-    const int64_t total = a.worklist ? (int64_t)(*a.d_count) : a.count_static;
-    const int64_t nsub = a.n_sub ? min((int64_t)(*a.n_sub), a.part_cap) : 0;
-    if (total + nsub == 0) return;
+    const int64_t total = PARTS        ? min((int64_t)(*a.n_sub), a.part_cap)
+                          : a.worklist ? (int64_t)(*a.d_count)
+                                       : a.count_static;
+    if (total == 0) return;
     unsigned long long my_bytes = 0;
     // the table starts empty once per launch; every node leaves it empty again
-    for (int i = tid; i < hcap; i += blockDim.x) tab[i] = kEmpty;
+#pragma unroll 1
+    for (int i = tid * 4; i < (1 << a.lg); i += kLuThreads * 4)
+        *reinterpret_cast<uint4*>(tab + i) = make_uint4(0u, 0u, 0u, 0u);
+    // the CTA's next item: a node, or (PARTS) a part of a split node
+    const int* items = PARTS ? a.sub_v : a.worklist;
+    if (tid == 0) {
+        const int i = atomicAdd(a.work_ctr, 1);
+        sh.idx = i;
+        if (i < total) sh.v = items ? items[i] : i;
+    }
+    int cls_graph = -1;
     for (;;) {
-        if (tid == 0) s_src = atomicAdd(a.work_ctr, 1);
         __syncthreads();
-        const int64_t idx = s_src;
-        if (idx >= total + nsub) break;
+        const int64_t idx = sh.idx;
+        if (idx >= total) break;
         // mode 0: a whole node; 1: one part of a split node (2: its merge)
-        int v, mode = 0, part = 0;
-        if (idx < total) {
-            v = a.worklist ? a.worklist[idx] : (int)idx;
-        } else {
-            v = a.sub_v[idx - total];
-            part = a.sub_j[idx - total];
-            mode = 1;
+        int mode = PARTS ? 1 : 0;
+        const int v = sh.v, part = PARTS ? a.sub_j[idx] : 0;
+        int next = 0;
+        if (tid == 0) next = atomicAdd(a.work_ctr, 1);
+        bool skip = PARTS && v < 0;  // a part the plan could not place
+        NodeLevel nl{};
+        int64_t b = 0;
+        int deg = 0;
+        uint32_t kv = 0;
+        int g = 0;
+        if (!skip) {
+            nl = node_level(a, v);
+            b = a.rowptr[v];
+            deg = (int)(a.rowptr[v + 1] - b);
+            kv = a.key32[v];
+            g = a.gid ? a.gid[v] : 0;
+            skip = a.alive[v] != 1 || nl.skip || nl.lvl < 2 || (!LIST && !nl.last) || (!LAST && nl.last);
+            if (!PARTS && !skip && a.part_cap > 0 && deg > kSplitDeg) {
+                // a heavy node is done in parts by the launch that follows
+                skip = true;
+                if (tid == 0) plan_parts(a, v, deg);
+            }
         }
-        if (v < 0) {  // a part the plan could not place
+        if (skip) {
             __syncthreads();
+            if (tid == 0) {
+                sh.idx = next;
+                if (next < total) sh.v = items ? items[next] : next;
+            }
             continue;
         }
-        const NodeLevel nl = node_level(a, v);
-        const int64_t b = a.rowptr[v], e = a.rowptr[v + 1];
-        const int deg = (int)(e - b);
-        // a heavy node is done by its parts (k_split_plan gave it slots)
-        if (a.alive[v] != 1 || nl.skip || nl.lvl < 2 ||
-            (mode == 0 && a.part_cap > 0 && deg > kSplitDeg)) {
-            __syncthreads();
-            continue;
-        }
-        const int rv = a.rank[v];
-        const int first = mode ? a.split_first[v] : -1;
+        const int rv = (int)(kv >> kIdBits);
+        const bool last = LAST && (!LIST || nl.last);
+        const int first = PARTS && mode ? a.split_first[v] : -1;
         const int nparts = (deg + kSplitChunk - 1) / kSplitChunk;
+        const uint8_t* wrank = a.wrank + (a.gid ? word_base(a.vtx_off[g], g) : 0);
+        if (g != cls_graph) {
+            if (tid < 33) sh.cls[tid] = a.clsw[(size_t)g * 33 + tid];
+            cls_graph = g;
+        }
+        // A node's level never rises as nodes leave, and mostly stays: start one
+        // below its last known level.  If the union then holds more than M at that
+        // level, the level is the old one; if not, the node is done again from t0.
+        const uint32_t last_meta = !PARTS || mode == 0 ? nl.meta_out[v] : 0u;
+        int t_spec = last_meta & kMetaAlive ? meta_k(last_meta) - 1 : -1;
         for (;;) {  // a node's last part continues as its merge (mode 2)
             // lists: neighbours [l0, l1) (modes 0, 1) or partial sets [0, nparts) (mode 2)
-            const int l0 = mode == 1 ? part * kSplitChunk : 0;
-            const int l1 = mode == 0 ? deg : (mode == 1 ? min(deg, l0 + kSplitChunk) : nparts);
+            const int l0 = PARTS && mode == 1 ? part * kSplitChunk : 0;
+            const int l1 = !PARTS || mode == 0 ? deg : (PARTS && mode == 1 ? min(deg, l0 + kSplitChunk) : nparts);
             const int L = l1 - l0;
-            if (tid < 32) s_hist[tid] = 0;
-            if (tid == 0) {
-                s_t = 0;
-                s_ex = 0.f;
-                s_nused = 0;
-                s_vin = 0;
-                s_exit = 0;
-                s_part = 0;
-                unsigned long long T = ~0ull;
-                if (a.stop_c && nl.last && mode != 2) {
-                    const int g = a.gid ? a.gid[v] : 0;
-                    T = stop_level(a.stop_c[g] > a.stop_mu[g] ? a.stop_c[g] : a.stop_mu[g]);
-                }
-                s_T = T;
-            }
-            __syncthreads();
-            const bool can_stop = s_T != ~0ull;
             // t starts at max k[w,i-1] over alive neighbours (Prop. 3.1), or at
             // the largest level of the partial sets (merge)
-            // (grouped free union) also sum |B[w]| 2^k[w]: over 2^t it is the
-            // expected number of keys at or above t (ranks halve per level)
+            int w0 = 0;
+            uint32_t m0 = 0;
             int myk = 0;
-            float ex = 0.f;
-            for (int li = l0 + tid; li < l1; li += blockDim.x) {
-                int k = 0, sz = 0;
-                if (mode == 2) {
-                    k = (int)__ldcg(a.part_t + first + li);
-                    sz = FREE && a.group_lists ? __ldcg(a.part_size + first + li) : 0;
+#pragma unroll 1
+            for (int li = l0 + tid; li < l1; li += kLuThreads) {
+                uint32_t m;
+                int32_t w;
+                if (PARTS && mode == 2) {
+                    w = li;
+                    m = __ldcg(a.part_meta + first + li);
                 } else {
-                    const int32_t w = a.col[b + li];
-                    if (a.alive[w] == 1) {
-                        k = (int)nl.lk_in[w];
-                        sz = FREE && a.group_lists ? min(nl.lsz_in[w], (int)a.cap) : 0;
-                    }
+                    w = a.col[b + li];
+                    m = nl.meta_in[w];
                 }
-                myk = max(myk, k);
-                ex += (float)sz * (float)(1u << (k & 31));
+                if (li == l0 + tid) {
+                    w0 = w;
+                    m0 = m;
+                }
+                myk = max(myk, meta_k(m));  // a removed neighbour's word is zero
             }
-            for (int off = 16; off > 0; off >>= 1) {
-                myk = max(myk, __shfl_down_sync(kFull, myk, off));
-                ex += __shfl_down_sync(kFull, ex, off);
+            myk = __reduce_max_sync(kFull, myk);
+            if (lane == 0) sh.kmax[warp] = myk;
+            if (tid < 32) sh.hist[tid] = 0;
+            if (tid < kBuckets) {
+                sh.nq[tid] = 0;
+                sh.cq[tid] = 0;
             }
-            if (lane == 0 && myk) atomicMax(&s_t, myk);
-            if (lane == 0 && ex > 0.f) atomicAdd(&s_ex, ex);
+            if (tid == 0) {
+                sh.exit = 0;
+                sh.creq = 0;
+                sh.part = 0;
+                unsigned long long T = ~0ull;
+                if (a.stop_c && last && !(PARTS && mode == 2))
+                    T = stop_level(a.stop_c[g] > a.stop_mu[g] ? a.stop_c[g] : a.stop_mu[g]);
+                sh.T = T;
+            }
             __syncthreads();
-            if (tid == 0 && rv >= s_t) {
-                const int slot = set_insert(tab, lg, ((uint32_t)rv << kIdBits) | (uint32_t)v, a.err);
-                if (slot >= 0) {
-                    used[s_nused++] = (uint16_t)slot;
-                    s_hist[rv] += 1;
-                    s_vin = 1;
+            int t0 = sh.kmax[0];
+#pragma unroll
+            for (int i = 1; i < kLuWarps; ++i) t0 = max(t0, sh.kmax[i]);
+            // (a refine that may stop early starts at t0: its partial estimate
+            // needs the low ranks)
+            const bool guess = t_spec > t0 && (sh.T == ~0ull || a.est[v] <= sh.T);
+            if (guess) t0 = t_spec;
+            const bool bm = sh.cls[t0] <= a.bm_words;
+            const int W0 = sh.cls[t0];
+            const bool vin = rv >= t0;
+            if (tid == 0) {
+                sh.t = t0;
+                sh.tot = sh.used = vin ? 1 : 0;
+                if (vin) {
+                    if (bm) tab[(kv & kIdMask) >> 5] = 1u << (kv & 31u);
+                    else set_insert(tab, a.lg, kv, a.err);
+                    sh.hist[rv] = 1;
                 }
             }
+            UnionCtx c;
+            c.tab = tab;
+            c.lists = PARTS && mode == 2 ? a.part_keys + (size_t)first * (size_t)a.cap : nl.keys_in;
+            c.wrank = wrank;
+            c.cap = a.cap;
+            c.lg = a.lg;
+            c.M = nl.M;
+            c.rv = rv;
+            c.can_stop = sh.T != ~0ull;
+            c.stop_first = PARTS && mode == 1 && c.can_stop ? first : -1;
+            c.vin = vin;
+            c.hash = !bm;
+            c.other = PARTS && mode == 2;
+            c.part_stop = a.part_stop;
+            c.err = a.err;
+            for (int c0 = l0; c0 < l1; c0 += kLuThreads) {
+                if (c0 > l0) {
+                    __syncthreads();  // the previous chunk's lists are read
+                    if (sh.exit) break;
+                    if (tid < kBuckets) {
+                        sh.nq[tid] = 0;
+                        sh.cq[tid] = 0;
+                    }
+                    const int li = c0 + tid;
+                    m0 = 0;
+                    if (li < l1) {
+                        w0 = PARTS && mode == 2 ? li : a.col[b + li];
+                        m0 = PARTS && mode == 2 ? __ldcg(a.part_meta + first + li) : nl.meta_in[w0];
+                    }
+                    __syncthreads();
+                }
+                // a list whose highest rank is below t has nothing to give
+                const int t = c0 > l0 ? sh.t : t0;
+                int bk = -1;
+                if (c0 + tid < l1 && (m0 & kMetaAlive) && meta_size(m0) > 0 && meta_top(m0) >= t) {
+                    // expected keys at or above t: ranks halve per level
+                    const int ex = meta_size(m0) >> (t - meta_k(m0)) >> a.group_shift;
+                    bk = m0 & kMetaDense ? kDense : !a.group_lists || ex > 64 ? kLong : ex > 8 ? kMiddle : kShort;
+                    sh.w[tid] = w0;
+                    sh.sz[tid] = (uint16_t)min(meta_size(m0), (int)a.cap);
+                }
+#pragma unroll
+                for (int q = 0; q < kBuckets; ++q) {
+                    const uint32_t mq = __ballot_sync(kFull, bk == q);
+                    if (!mq) continue;
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(&sh.nq[q], __popc(mq));
+                    base = __shfl_sync(kFull, base, 0);
+                    if (bk == q) sh.q[q][base + __popc(mq & ((1u << lane) - 1u))] = (uint8_t)tid;
+                }
+                __syncthreads();
+                int bucket = kBuckets - 1, li = -1, pos = 0;
+                // a compaction keeps at most M keys, well under the trigger, so every
+                // pass reads on; a bound no correct run reaches ends the union
+                for (int pass = 0;; ++pass) {
+                    walk_chunk<LAST, PARTS>(c, sh, bucket, li, pos, my_bytes);
+                    if (bm) break;
+                    __syncthreads();
+                    if (!sh.creq || sh.exit) break;
+                    if (pass > kLuThreads * (kMaxM / kKeysPerLane + 4)) {
+                        if (tid == 0) atomicOr(a.err, kErrLoop);
+                        break;
+                    }
+                    compact_set(a, sh, tab, nl.M);
+                }
+            }
+            // the next item's node, while the last lists are read
+            int nv = 0;
+            if (tid == 0 && next < total) nv = items ? items[next] : next;
             __syncthreads();
-            bool stopped = false;
-            if constexpr (FREE) {
-                // lanes per list: a warp, or (grouped) the fewest whose step of
-                // 4 G keys covers the keys a list is expected to give at or
-                // above the starting level
-                int G = 32;
-                if (a.group_lists) {
-                    const float per = s_ex / (float)(1u << (s_t & 31)) / (float)(L > 0 ? L : 1);
-                    while (G > 1 && (float)(kKeysPerLane * (G >> 1) * a.group_div) >= per) G >>= 1;
+            const bool stopped = LAST && sh.exit != 0;
+            const int Sl = snapshot_counts(sh.hist, lane);
+            const uint32_t over = __ballot_sync(kFull, Sl > nl.M);
+            const int kappa = max(sh.t, over ? 32 - __clz(over) : 0);
+            const int Sk = __shfl_sync(kFull, Sl, kappa & 31);
+            const int S = kappa < 32 ? Sk : 0;
+            const uint32_t nz = __ballot_sync(kFull, Sl > 0);
+            const int top = nz && 31 - __clz(nz) >= kappa ? 31 - __clz(nz) : 0;
+            const int lists_bytes = 8 * L;  // columns and meta words
+            bool merge = false, lost = false;
+            const bool redo = guess && !stopped && kappa == t0;  // the level fell
+            uint32_t meta = 0;
+            if (!stopped && !redo && ((PARTS && mode == 1) || !last)) {
+                // the list of the node, or of the part
+                uint32_t* out = PARTS && mode == 1 ? a.part_keys + (size_t)(first + part) * (size_t)a.cap
+                                          : nl.keys_out + (size_t)v * (size_t)a.cap;
+                if (a.track && !(PARTS && mode == 1)) {
+                    const uint32_t old = nl.meta_out[v];
+                    lost = meta_size(old) != S || meta_k(old) != kappa;
+                    if (lost) {
+                        if (tid == 0) sh.rho = kappa != meta_k(old) ? meta_k(old) - 1 : -1;
+                        const int r = __reduce_max_sync(
+                            kFull, lost_rank(a, sh, tab, bm, W0, wrank, out, old));
+                        __syncthreads();  // the old list is read before it is overwritten
+                        if (lane == 0 && r >= 0) atomicMax(&sh.rho, r);
+                        __syncthreads();
+                    }
                 }
-                stopped = free_union(a, nl, tab, stage, used, lg, hcap, scap, ucap, s_hist, &s_t,
-                                     &s_nused,
-                                     &s_nstage, &s_exit, &s_part, &s_item, &s_creq, s_T, s_vin,
-                                     can_stop, mode, first, b, l0, L, rv, G, my_bytes);
-            } else {
-            // Flat mode, whole nodes of degree <= kFlatMax: every (list, 128-key
-            // chunk) pair is one work item, warps take items in order, one per
-            // step, so long and short lists balance; a list is dropped once a
-            // chunk shows a key below t.
-            const bool flat = mode == 0 && deg <= kFlatMax;
-            if (flat) {
-                int cnt = 0;
-                const int t0 = s_t;
-                if (tid < deg) {
-                    const int32_t w = a.col[b + tid];
-                    int sz = 0;
-                    // a list whose highest rank is below t has nothing to give
-                    if (a.alive[w] == 1 && (int)nl.ltop_in[w] >= t0) sz = min(nl.lsz_in[w], (int)a.cap);
-                    s_w[tid] = w;
-                    s_sz[tid] = sz;
-                    s_dead[tid] = INT_MAX;
-                    cnt = (sz + kChunkKeys - 1) / kChunkKeys;
-                }
-                int inc = cnt;  // block-wide exclusive scan of the chunk counts
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int x = __shfl_up_sync(kFull, inc, off);
-                    if (lane >= off) inc += x;
-                }
-                if (lane == 31) s_wsum[warp] = inc;
-                __syncthreads();
-                int before = 0;
-                for (int w2 = 0; w2 < warp; ++w2) before += s_wsum[w2];
-                if (tid < deg) s_off[tid] = before + inc - cnt;
-                if (tid == kLuThreads - 1) s_total = before + inc;
-                __syncthreads();
+                meta = write_list(a, sh, tab, bm, wrank, out, S, kappa, top);
             }
-            int fbase = 0;  // flat mode: first item of this step
-            // Grouped mode: G lanes share one list and read G*4 consecutive keys
-            // per step; G shrinks as the number of lists grows, so that many
-            // lists are open at once (hubs: one lane per list)
-            int G = 32;
-            while (G > 1 && (kLuThreads / G) < L) G >>= 1;
-            const int ngroups = kLuThreads / G;
-            const int gid = tid / G, gl = tid % G;
-            const uint32_t gmask = (G == 32) ? kFull : (((1u << G) - 1u) << (lane & ~(G - 1)));
-            const int step = kKeysPerLane * G;
-            int li = l0 + gid;  // list index of this group's current list
-            int pos = 0;
-            bool any = true;
-            while (any) {
-                const int t = *(volatile int*)&s_t;
-                if (flat) {
-                    const int c = fbase + warp;
-                    if (c < s_total) {
-                        int lo = 0, hi = deg - 1;  // last list whose first chunk is <= c
-                        while (lo < hi) {
-                            const int mid = (lo + hi + 1) >> 1;
-                            if (s_off[mid] <= c) lo = mid;
-                            else hi = mid - 1;
-                        }
-                        // chunks after one with a key below t hold only keys below t;
-                        // warps of one step run unordered, so an earlier chunk of the
-                        // same list is still read even when a later one was seen first
-                        if (c <= __shfl_sync(kFull, s_dead[lo], 0)) {
-                            const int sz = s_sz[lo];
-                            const int p = (c - s_off[lo]) * kChunkKeys + lane * kKeysPerLane;
-                            bool below = false;
-                            if (p < sz) {
-                                const uint4 k4 = *reinterpret_cast<const uint4*>(
-                                    nl.keys_in + (size_t)s_w[lo] * (size_t)a.cap + p);
-                                const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
-#pragma unroll
-                                for (int q = 0; q < kKeysPerLane; ++q) {
-                                    if (p + q < sz) {
-                                        const uint32_t key = kk[q];
-                                        const int r = (int)(key >> kIdBits);
-                                        my_bytes += 4;
-                                        if (r >= t) {
-                                            const int slot = set_insert(tab, lg, key, a.err);
-                                            if (slot >= 0) {
-                                                const int u = atomicAdd(&s_nused, 1);
-                                                if (u < ucap) used[u] = (uint16_t)slot;
-                                                else atomicOr(a.err, kErrProbe);
-                                                atomicAdd(&s_hist[r], 1);
-                                            }
-                                        } else {
-                                            below = true;
-                                        }
-                                    }
-                                }
-                            }
-                            // ranks only fall along a list: the rest of it is below t
-                            if (__any_sync(kFull, below) && lane == 0) atomicMin(&s_dead[lo], c);
-                        }
-                    }
-                    fbase += nwarps;
-                }
-                // advance to a list with keys left (group-uniform)
-                const uint32_t* lp = nullptr;
-                int sz = 0;
-                while (!flat && li < l1) {
-                    if (mode == 2) {
-                        sz = __ldcg(a.part_size + first + li);
-                        lp = a.part_keys + (size_t)(first + li) * (size_t)a.cap;
-                        if (sz > pos) break;
-                    } else {
-                        const int32_t w = a.col[b + li];
-                        if (a.alive[w] == 1 && (int)nl.ltop_in[w] >= t) {
-                            sz = min(nl.lsz_in[w], (int)a.cap);
-                            lp = nl.keys_in + (size_t)w * (size_t)a.cap;
-                            if (sz > pos) break;
-                        }
-                    }
-                    li += ngroups;
-                    pos = 0;
-                }
-                bool below = false;
-                if (!flat && li < l1) {
-                    const int p = pos + gl * kKeysPerLane;
-                    if (p < sz) {
-                        const uint4 k4 = mode == 2 ? __ldcg(reinterpret_cast<const uint4*>(lp + p))
-                                                   : *reinterpret_cast<const uint4*>(lp + p);
-                        const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
-#pragma unroll
-                        for (int q = 0; q < kKeysPerLane; ++q) {
-                            if (p + q < sz) {
-                                const uint32_t key = kk[q];
-                                const int r = (int)(key >> kIdBits);
-                                if (mode != 2) my_bytes += 4;
-                                if (r >= t) {
-                                    const int slot = set_insert(tab, lg, key, a.err);
-                                    if (slot >= 0) {
-                                        const int u = atomicAdd(&s_nused, 1);
-                                        if (u < ucap) used[u] = (uint16_t)slot;
-                                        else atomicOr(a.err, kErrProbe);
-                                        atomicAdd(&s_hist[r], 1);
-                                    }
-                                } else {
-                                    below = true;
-                                }
-                            }
-                        }
-                    }
-                }
-                const uint32_t bal = __ballot_sync(kFull, below);
-                if (!flat && li < l1) {
-                    if ((bal & gmask) || pos + step >= sz) {
-                        li += ngroups;
-                        pos = 0;
-                    } else {
-                        pos += step;
-                    }
-                }
-                any = __syncthreads_or(flat ? fbase < s_total : li < l1);
-                if (warp == 0) {
-                    // smallest level >= t with at most M distinct members (Alg. 5's
-                    // trim): lane j holds S_j = #{distinct keys with rank >= j}
-                    int S = s_hist[lane];
-                    for (int off = 1; off < 32; off <<= 1) {
-                        const int x = __shfl_down_sync(kFull, S, off);
-                        if (lane + off < 32) S += x;
-                    }
-                    const uint32_t over = __ballot_sync(kFull, S > nl.M);
-                    const int pmax = over ? 31 - __clz(over) : -1;
-                    if (can_stop) {
-                        // Def. 4.1 on the keys inserted so far plus v itself: a subset
-                        // of N(v;h) led by v, so by Prop. 4.2 at most the final estimate
-                        const int Sp = S + ((!s_vin && rv >= lane) ? 1 : 0);
-                        const uint32_t fits = __ballot_sync(kFull, Sp <= nl.M);
-                        const int k = fits ? __ffs(fits) - 1 : 32;
-                        const int Sk = __shfl_sync(kFull, Sp, k & 31);
-                        const unsigned long long pe = estimate_of(k < 32 ? Sk : 0, k, rv, nl.M);
-                        if (lane == 0 && pe > s_T) {
-                            s_exit = 1;
-                            s_part = pe;
-                        }
-                        // a part stops too once another part of the node has
-                        // shown d(v) > T
-                        if (mode == 1 && lane == 0 && !s_exit && ld_acquire(a.part_stop + first))
-                            s_exit = 2;
-                    }
-                    if (lane == 0) {
-                        const int told = s_t;
-                        s_t = max(told, pmax + 1);
-                        s_compact = s_nused > (hcap >> 1);
-                        s_nstage = 0;
-                    }
-                }
-                __syncthreads();
-                if (s_exit && any) {  // (with every list read, finish: the exact value is kept)
-                    stopped = true;
-                    break;
-                }
-                if (s_compact) {
-                    // drop keys below t: empty their slots, re-insert the rest
-                    const int tc = s_t, nu = min(s_nused, ucap);
-                    for (int i = tid; i < nu; i += blockDim.x) {
-                        const int slot = used[i];
-                        const uint32_t key = tab[slot];
-                        tab[slot] = kEmpty;
-                        if ((int)(key >> kIdBits) >= tc) {
-                            const int p = atomicAdd(&s_nstage, 1);
-                            if (p < scap) stage[p] = key;
-                            else atomicOr(a.err, kErrProbe);
-                        }
-                    }
-                    __syncthreads();
-                    if (tid == 0) s_nused = 0;
-                    __syncthreads();
-                    const int ns = min(s_nstage, scap);
-                    for (int i = tid; i < ns; i += blockDim.x) {
-                        const int slot = set_insert(tab, lg, stage[i], a.err);
-                        if (slot >= 0) used[atomicAdd(&s_nused, 1)] = (uint16_t)slot;
-                    }
-                    __syncthreads();
-                }
-            }
-            }  // stepped union
-            if (stopped) {
-                // d(v) > T: v stays stale, its lower bound raised to the partial estimate
-                const int nu = min(s_nused, ucap);
-                for (int i = tid; i < nu; i += blockDim.x) tab[used[i]] = kEmpty;
-                if (mode == 0) {
+            if (redo) {
+                t_spec = -1;
+            } else if (PARTS && mode == 1) {
+                // a part: its partial set, or (refine) the estimate above T that
+                // it already shows; the node's last part finishes it
+                if (stopped) {
                     if (tid == 0) {
-                        a.lb[v] = s_part;
-                        a.fresh[v] = 0;
-                        atomicAdd(a.stopped, 1ull);  // a lower bound only: not an update
-                        my_bytes += 8ull + 10ull * (unsigned long long)deg + 9ull;
+                        if (sh.exit == 1) atomicMax(a.part_lb + first, sh.part);
+                        a.part_stop[first] = 1;
                     }
-                    break;
+                } else if (tid == 0) {
+                    a.part_meta[first + part] = meta;
                 }
-                // a part: its partial set (a sub-multiset of N(v; h) led by v)
-                // already estimates above T; the node's last part finishes it
-                if (tid == 0) {
-                    if (s_exit == 1) atomicMax(a.part_lb + first, s_part);
-                    a.part_stop[first] = 1;
-                }
-            }
-            const int kappa = s_t;
-            const int nu = min(s_nused, ucap);
-            int S = 0;
-            for (int j = kappa; j < 32; ++j) S += s_hist[j];
-            __syncthreads();
-            if (mode == 1 && stopped) {
-                if (tid == 0) my_bytes += 10ull * (unsigned long long)L;
-            } else if (mode == 1) {
-                // this part's trimmed set, grouped by rank (highest first), and its level
-                if (tid < 32) {
-                    int above = 0;
-                    for (int j = tid + 1; j < 32; ++j) above += s_hist[j];
-                    __syncwarp();  // every lane has read before any lane writes
-                    s_hist[tid] = above;
-                }
-                __syncthreads();
-                uint32_t* out = a.part_keys + (size_t)(first + part) * (size_t)a.cap;
-                for (int i = tid; i < nu; i += blockDim.x) {
-                    const int slot = used[i];
-                    const uint32_t key = tab[slot];
-                    tab[slot] = kEmpty;
-                    const int r = (int)(key >> kIdBits);
-                    if (r >= kappa) {
-                        const int p = atomicAdd(&s_hist[r], 1);
-                        if (p < a.cap) out[p] = key;
-                        else atomicOr(a.err, kErrList);
-                    }
-                }
-                if (tid == 0) {
-                    a.part_size[first + part] = S;
-                    a.part_t[first + part] = (uint8_t)kappa;
-                    my_bytes += 10ull * (unsigned long long)L;
-                }
-            }
-            if (mode == 1) {
+                if (tid == 0) my_bytes += lists_bytes;
                 __threadfence();
                 __syncthreads();
-                if (tid == 0) s_last = atomicAdd(a.part_done + first, 1) == nparts - 1;
+                if (tid == 0) sh.last = atomicAdd(a.part_done + first, 1) == nparts - 1;
                 __syncthreads();
-                if (!s_last) break;
-                __threadfence();  // the other parts' sets are visible from here on
-                if (__ldcg(a.part_stop + first)) {
-                    // some part showed d(v) > T: v stays stale with that lower bound
-                    if (tid == 0) {
-                        a.lb[v] = __ldcg(a.part_lb + first);
-                        a.fresh[v] = 0;
-                        atomicAdd(a.stopped, 1ull);
-                        a.part_stop[first] = 0;
-                        a.part_lb[first] = 0;
-                        a.part_done[first] = 0;
+                if (sh.last) {
+                    __threadfence();  // the other parts' sets are visible from here on
+                    if (__ldcg(a.part_stop + first)) {
+                        // some part showed d(v) > T: v stays stale with that lower bound
+                        __syncthreads();  // every thread has read the flag
+                        if (tid == 0) {
+                            a.lb[v] = __ldcg(a.part_lb + first);
+                            a.fresh[v] = 0;
+                            atomicAdd(a.stopped, 1ull);
+                            a.part_stop[first] = 0;
+                            a.part_lb[first] = 0;
+                            a.part_done[first] = 0;
+                        }
+                    } else {
+                        merge = true;
                     }
-                    break;
                 }
-                mode = 2;
-                continue;
-            }
-            if (tid == 0) my_bytes += 8ull + 5ull + (mode == 0 ? 10ull * (unsigned long long)deg : 0ull);
-            if (nl.last) {
+            } else if (stopped) {
+                // d(v) > T: v stays stale, its lower bound raised to the partial estimate
+                if (tid == 0) {
+                    a.lb[v] = sh.part;
+                    a.fresh[v] = 0;
+                    atomicAdd(a.stopped, 1ull);  // a lower bound only: not an update
+                    my_bytes += 17ull + lists_bytes;
+                }
+            } else if (last) {
                 if (tid == 0) {
                     const unsigned long long est = estimate_of(S, kappa, rv, nl.M);
                     a.est[v] = est;
-                    if (a.min_done) atomicMin(a.min_done + (a.gid ? a.gid[v] : 0), est);
-                    record_change(a, nl, v, S, kappa);
+                    if (a.min_done) atomicMin(a.min_done + g, est);
+                    record_change(a, nl, v, meta_pack(S, kappa, top, false));
                     atomicAdd(a.updates, 1ull);
-                    my_bytes += 8;
+                    my_bytes += 21ull + (!PARTS || mode == 0 ? lists_bytes : 0);
                 }
-                for (int i = tid; i < nu; i += blockDim.x) tab[used[i]] = kEmpty;
             } else {
-                if (a.track) {
-                    // rho (see level1_rho_warp): an old member left iff its key is
-                    // not in the new union, where every key of rank >= kappa is kept
-                    const int old_s = nl.lsz_out[v], old_k = nl.lk_out[v];
-                    if (old_s != S || old_k != kappa) {
-                        if (tid == 0) s_rho = kappa != old_k ? old_k - 1 : -1;
-                        __syncthreads();
-                        const uint32_t* old = nl.keys_out + (size_t)v * (size_t)a.cap;
-                        const int m = min(old_s, (int)a.cap);
-                        int r = -1;
-                        for (int p = tid; p < m; p += blockDim.x) {
-                            const uint32_t key = old[p];
-                            if (!set_contains(tab, lg, key)) r = max(r, (int)(key >> kIdBits));
-                        }
-                        for (int off = 16; off > 0; off >>= 1) r = max(r, __shfl_xor_sync(kFull, r, off));
-                        if (lane == 0 && r >= 0) atomicMax(&s_rho, r);
-                        __syncthreads();  // the old list is read before it is overwritten
-                        if (tid == 0) a.rho[v] = (int8_t)s_rho;
-                    }
-                }
-                // write members grouped by rank, highest first, emptying the table
-                if (tid < 32) {
-                    const uint32_t nz = __ballot_sync(kFull, tid >= kappa && s_hist[tid] > 0);
-                    if (tid == 0 && nl.ltop_out) nl.ltop_out[v] = (uint8_t)(nz ? 31 - __clz(nz) : 0);
-                    __syncwarp();
-                    int above = 0;
-                    for (int j = tid + 1; j < 32; ++j) above += s_hist[j];
-                    __syncwarp();
-                    s_hist[tid] = above;  // start offset of rank tid
-                }
-                __syncthreads();
-                uint32_t* out = nl.keys_out + (size_t)v * (size_t)a.cap;
-                for (int i = tid; i < nu; i += blockDim.x) {
-                    const int slot = used[i];
-                    const uint32_t key = tab[slot];
-                    tab[slot] = kEmpty;
-                    const int r = (int)(key >> kIdBits);
-                    if (r >= kappa) {
-                        const int p = atomicAdd(&s_hist[r], 1);
-                        if (p < a.cap) out[p] = key;
-                        else atomicOr(a.err, kErrList);
-                    }
-                }
                 if (tid == 0) {
-                    record_change(a, nl, v, S, kappa);
-                    my_bytes += 4ull * (unsigned long long)S;
+                    if (lost) a.rho[v] = (int8_t)sh.rho;
+                    record_change(a, nl, v, meta);
+                    my_bytes += 13ull + (!PARTS || mode == 0 ? lists_bytes : 0) + 4ull * (unsigned long long)S;
                 }
             }
-            if (mode == 2 && tid == 0) a.part_done[first] = 0;  // ready for the next launch
+            __syncthreads();  // the table and the shared state are read
+            const int clear = bm ? W0 : 1 << a.lg;
+#pragma unroll 1
+            for (int i = tid * 4; i < clear; i += kLuThreads * 4)
+                *reinterpret_cast<uint4*>(tab + i) = make_uint4(0u, 0u, 0u, 0u);
+            if (PARTS && mode == 2 && tid == 0) a.part_done[first] = 0;  // ready for the next launch
+            if (merge || redo) {
+                if (merge) mode = 2;
+                __syncthreads();
+                continue;
+            }
+            if (tid == 0) {
+                sh.idx = next;
+                sh.v = nv;
+            }
             break;
         }
-        __syncthreads();
     }
     for (int off = 16; off > 0; off >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, off);
     if (lane == 0 && my_bytes) atomicAdd(a.bytes, my_bytes);
-}
-
-// Plan the split of the heavy nodes of a level pass: every listed node that
-// computes a level >= 2 and has more than kSplitDeg neighbours gets
-// ceil(deg / kSplitChunk) consecutive part slots and part items.
-__global__ void k_split_plan(LevelArgs a) {
-    const int64_t total = a.worklist ? (int64_t)(*a.d_count) : a.count_static;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += stride) {
-        const int v = a.worklist ? a.worklist[idx] : (int)idx;
-        const int64_t deg = a.rowptr[v + 1] - a.rowptr[v];
-        if (deg <= kSplitDeg || a.alive[v] != 1) continue;
-        const NodeLevel nl = node_level(a, v);
-        if (nl.skip || nl.lvl < 2) continue;
-        const int P = (int)((deg + kSplitChunk - 1) / kSplitChunk);
-        const int base = atomicAdd(a.n_sub, P);
-        if ((int64_t)base + P <= a.part_cap) {
-            for (int j = 0; j < P; ++j) {
-                a.sub_v[base + j] = v;
-                a.sub_j[base + j] = j;
-            }
-            a.split_first[v] = base;
-        } else {
-            // cannot happen: part_cap covers every heavy node of the graph at once
-            for (int64_t j = base; j < a.part_cap && j < (int64_t)base + P; ++j) a.sub_v[j] = -1;
-            atomicOr(a.err, kErrList);
-        }
-    }
 }
 
 // Rank filter for the neighbours of changed lists.  Level i of u is the
@@ -1190,7 +1195,7 @@ __global__ void k_split_plan(LevelArgs a) {
 // level only while u is fresh.
 struct MarkFilter {
     const int8_t* rho;    // nullptr: no filter
-    const uint8_t* lk;    // k[u, phase]
+    const uint32_t* meta; // meta words of level `phase`
     const uint8_t* hv;    // per-node h (batches) or nullptr
     int h;
     const uint8_t* fresh;
@@ -1199,7 +1204,7 @@ struct MarkFilter {
 __device__ __forceinline__ bool level_may_change(const MarkFilter& f, int u, int rw, int level) {
     const int hu = f.hv ? (int)f.hv[u] : f.h;
     const bool known = level < hu || (level == hu && f.fresh[u]);
-    return !known || rw >= (int)f.lk[u] - 1;
+    return !known || rw >= meta_k(f.meta[u]) - 1;
 }
 
 // Alive neighbours of the listed nodes (two lists, the second optional and
@@ -1292,16 +1297,10 @@ __global__ void k_mark_nbrs(const int64_t* __restrict__ rowptr, const int32_t* _
     if (lane == 0 && my_bytes) atomicAdd(bytes, my_bytes);
 }
 
-// Alg. 1 on a level list of size S and level kappa, with the node of rank
-// r_first counted first (it is a member of the list's neighbourhood).
-__device__ __forceinline__ unsigned long long est_first(int S, int kappa, int r_first, int64_t M) {
-    const int T = S - (r_first >= kappa ? 1 : 0);
-    unsigned long long d = (unsigned long long)T << kappa;
-    if (kappa > 0) {
-        const unsigned long long f = (unsigned long long)M << (kappa - 1);
-        if (f > d) d = f;
-    }
-    return d;
+// Alg. 1 on a list (its meta word), with the node of rank r_first counted
+// first (it is a member of the list's neighbourhood).
+__device__ __forceinline__ unsigned long long est_first(uint32_t m, int r_first, int64_t M) {
+    return estimate_of(meta_size(m), meta_k(m), r_first, M);
 }
 
 // Mark nodes stale at the last level h and give each a lower bound of its
@@ -1316,17 +1315,17 @@ __device__ __forceinline__ unsigned long long est_first(int S, int kappa, int r_
 // neighbour w gives a sub-multiset N(w; h-1) of N(v; h) led by v, so one
 // neighbour's term is still a lower bound, at O(1) cost instead of O(deg).
 constexpr int kStaleScan = 64;
+constexpr int kStaleThreads = 256;
 
 __global__ void k_stale_sampled(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                                 const uint8_t* __restrict__ alive, const uint8_t* __restrict__ rank,
-                                const int32_t* __restrict__ lsz, const uint8_t* __restrict__ lk,
-                                int h_all, const uint8_t* __restrict__ hv, int64_t M_all,
+                                const uint32_t* __restrict__ meta, int h_all, const uint8_t* __restrict__ hv, int64_t M_all,
                                 const int32_t* __restrict__ Mv, int only_h,
                                 const int32_t* __restrict__ list, const int* __restrict__ nlist,
                                 int64_t n, uint8_t* __restrict__ fresh,
                                 unsigned long long* __restrict__ lb, unsigned long long* bytes,
                                 const int32_t* __restrict__ bestnb) {
-    __shared__ unsigned long long s_max[kLuThreads / 32];
+    __shared__ unsigned long long s_max[kStaleThreads / 32];
     __shared__ int s_heavy[kBlockHeavy];
     __shared__ int s_nheavy;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1347,10 +1346,9 @@ __global__ void k_stale_sampled(const int64_t* __restrict__ rowptr, const int32_
             if (alive[w] == 1) {  // warp-uniform
                 if (lane == 0) {
                     const int64_t M = Mv ? (int64_t)Mv[v] : M_all;
-                    const size_t off = (size_t)(h - 2) * (size_t)n;
+                    const uint32_t* prev = meta + (size_t)(h - 2) * (size_t)n;
                     const int rv = rank[v];
-                    lb[v] = umax64(est_first(lsz[off + v], lk[off + v], rv, M),
-                                   est_first(lsz[off + w], lk[off + w], rv, M));
+                    lb[v] = umax64(est_first(prev[v], rv, M), est_first(prev[w], rv, M));
                     fresh[v] = 0;
                     my_bytes += 29ull + 9ull;
                 }
@@ -1367,17 +1365,17 @@ __global__ void k_stale_sampled(const int64_t* __restrict__ rowptr, const int32_
             }
         }
         const int64_t M = Mv ? (int64_t)Mv[v] : M_all;
-        const int32_t* lsz_prev = h >= 2 ? lsz + (size_t)(h - 2) * (size_t)n : nullptr;
-        const uint8_t* lk_prev = h >= 2 ? lk + (size_t)(h - 2) * (size_t)n : nullptr;
+        const uint32_t* prev = h >= 2 ? meta + (size_t)(h - 2) * (size_t)n : nullptr;
         unsigned long long m = 0;
-        if (lsz_prev) {
+        if (prev) {
             const int rv = rank[v];
             for (int64_t k = b + lane; k < e; k += 32) {
                 const int32_t w = col[k];
-                if (alive[w] == 1) m = umax64(m, est_first(lsz_prev[w], lk_prev[w], rv, M));
+                const uint32_t mw = prev[w];
+                if (mw & kMetaAlive) m = umax64(m, est_first(mw, rv, M));
             }
             for (int off = 16; off > 0; off >>= 1) m = umax64(m, __shfl_down_sync(kFull, m, off));
-            m = umax64(m, est_first(lsz_prev[v], lk_prev[v], rv, M));
+            m = umax64(m, est_first(prev[v], rv, M));
         }
         if (lane == 0) {
             lb[v] = m;
@@ -1391,22 +1389,22 @@ __global__ void k_stale_sampled(const int64_t* __restrict__ rowptr, const int32_
         const int v = s_heavy[j];
         const int h = hv ? (int)hv[v] : h_all;
         const int64_t M = Mv ? (int64_t)Mv[v] : M_all;
-        const int32_t* lsz_prev = h >= 2 ? lsz + (size_t)(h - 2) * (size_t)n : nullptr;
-        const uint8_t* lk_prev = h >= 2 ? lk + (size_t)(h - 2) * (size_t)n : nullptr;
+        const uint32_t* prev = h >= 2 ? meta + (size_t)(h - 2) * (size_t)n : nullptr;
         unsigned long long m = 0;
         const int64_t b = rowptr[v], e = rowptr[v + 1];
-        if (lsz_prev) {
+        if (prev) {
             const int rv = rank[v];
             for (int64_t k = b + threadIdx.x; k < e; k += blockDim.x) {
                 const int32_t w = col[k];
-                if (alive[w] == 1) m = umax64(m, est_first(lsz_prev[w], lk_prev[w], rv, M));
+                const uint32_t mw = prev[w];
+                if (mw & kMetaAlive) m = umax64(m, est_first(mw, rv, M));
             }
             for (int off = 16; off > 0; off >>= 1) m = umax64(m, __shfl_down_sync(kFull, m, off));
             if (lane == 0) s_max[warp] = m;
             __syncthreads();
             if (threadIdx.x == 0) {
                 for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = umax64(m, s_max[w]);
-                m = umax64(m, est_first(lsz_prev[v], lk_prev[v], rv, M));
+                m = umax64(m, est_first(prev[v], rv, M));
             }
         }
         if (threadIdx.x == 0) {
@@ -1486,9 +1484,8 @@ int ensure_split(Graph& g) {
             return rc;
         KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.part_lb, 0, sizeof(unsigned long long) * pc, s));
     }
-    if (!g.part_size && (rc = alloc_bytes(g.ctx, (void**)&g.part_size, sizeof(int32_t) * pc, "split part sizes")))
+    if (!g.part_meta && (rc = alloc_bytes(g.ctx, (void**)&g.part_meta, sizeof(uint32_t) * pc, "split part metas")))
         return rc;
-    if (!g.part_t && (rc = alloc_bytes(g.ctx, (void**)&g.part_t, pc, "split part levels"))) return rc;
     if (!g.sub_v && (rc = alloc_bytes(g.ctx, (void**)&g.sub_v, sizeof(int32_t) * pc, "split part nodes")))
         return rc;
     if (!g.sub_j && (rc = alloc_bytes(g.ctx, (void**)&g.sub_j, sizeof(int32_t) * pc, "split part indices")))
@@ -1499,11 +1496,110 @@ int ensure_split(Graph& g) {
     return KH_OK;
 }
 
+namespace {
+// Slots of the hash form: a compaction is due past half of them and leaves at
+// most M <= 4/5 of that; until every warp has stopped for it, each may add two
+// more steps of 128 keys (1024 in all, at most a quarter of the slots).
 int table_lg(int64_t M) {
-    // capacity >= 2 (M + keys inserted per step) rounded up to a power of two
-    int lg = 10;
-    while ((int64_t(1) << lg) < 2 * (M + (int64_t)kKeysPerLane * kLuThreads)) ++lg;
+    int lg = 12;
+    while ((int64_t(1) << lg) * 2 < 5 * M) ++lg;
     return lg;
+}
+
+// The bitmap form may use as many words as the hash form has slots; position
+// classes are whole words only while the padded positions fit the key.
+bool positions_aligned(const Graph& g) { return g.n + 1024 <= (int64_t)1 << kIdBits; }
+
+// ---- positions: nodes numbered by descending rank ----------------------------
+// Per graph and rank class: its nodes (pass 0), then its first position;
+// pass 1 hands the positions out.  Counters are taken per warp and class.
+__global__ void k_pos_pass(const uint8_t* __restrict__ rank, const int32_t* __restrict__ gid, int64_t n,
+                           int* __restrict__ cnt, uint32_t* __restrict__ key32) {
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t nround = (n + 31) & ~(int64_t)31;
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nround; u += stride) {
+        const bool in = u < n;
+        const uint32_t r = in ? rank[u] : 0;
+        const uint32_t slot = in ? (uint32_t)(gid ? gid[u] : 0) * 32u + r : 0xffffffffu;
+        const uint32_t peers = __match_any_sync(kFull, slot);
+        const int lead = __ffs(peers) - 1;
+        int base = 0;
+        if (in && lane == lead) base = atomicAdd(cnt + slot, __popc(peers));
+        base = __shfl_sync(kFull, base, lead);
+        if (in && key32) key32[u] = (r << kIdBits) | (uint32_t)(base + __popc(peers & ((1u << lane) - 1u)));
+    }
+}
+
+// One warp per graph: clsw from the class counts, the counts become each
+// class's first position, wrank of the graph's words.
+__global__ void k_pos_classes(int* __restrict__ cnt, int64_t ngraphs, const int64_t* __restrict__ vtx_off,
+                              int32_t* __restrict__ clsw, uint8_t* __restrict__ wrank, int aligned) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < ngraphs; q += nw) {
+        const int c = cnt[q * 32 + lane];
+        const int size = aligned ? (c + 31) >> 5 : c;  // words, or (unaligned) positions
+        int incl = size;                               // over the ranks >= lane
+        for (int off = 1; off < 32; off <<= 1) {
+            const int x = __shfl_down_sync(kFull, incl, off);
+            if (lane + off < 32) incl += x;
+        }
+        const int above = incl - size;
+        cnt[q * 32 + lane] = aligned ? above << 5 : above;
+        clsw[q * 33 + lane] = aligned ? incl : 0x7fffffff;
+        if (lane == 0) clsw[q * 33 + 32] = aligned ? 0 : 0x7fffffff;
+        if (!aligned) continue;
+        uint8_t* wr = wrank + word_base(vtx_off ? vtx_off[q] : 0, q);
+        for (int r = 0; r < 32; ++r) {
+            const int w0 = __shfl_sync(kFull, above, r), w1 = __shfl_sync(kFull, incl, r);
+            for (int w = w0 + lane; w < w1; w += 32) wr[w] = (uint8_t)r;
+        }
+    }
+}
+}  // namespace
+
+// Ranks, and what the sampled path derives from them and from M.
+int ensure_positions(Graph& g) {
+    cudaStream_t s = g.ctx->stream;
+    const int64_t ng = g.gid ? g.ngraphs : 1;
+    int rc;
+    if (!g.ranks_valid) {
+        launch_ranks(g, s);
+        g.ranks_valid = true;
+        g.pos_valid = false;
+    }
+    if (!g.key32 && (rc = alloc_bytes(g.ctx, (void**)&g.key32, sizeof(uint32_t) * (size_t)g.n, "positions")))
+        return rc;
+    if (!g.clsw && (rc = alloc_bytes(g.ctx, (void**)&g.clsw, sizeof(int32_t) * 65 * (size_t)ng, "rank classes")))
+        return rc;
+    if (!g.wrank && (rc = alloc_bytes(g.ctx, (void**)&g.wrank, (size_t)word_base(g.n, ng) + 4, "word ranks")))
+        return rc;
+    // compaction stage of the hash form, one slot per CTA of k_levelU
+    if (g.lu_stage && g.lu_stage_cap < g.cap) {
+        KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
+        cudaFree(g.lu_stage);
+        g.lu_stage = nullptr;
+    }
+    if (!g.lu_stage) {
+        if ((rc = alloc_bytes(g.ctx, (void**)&g.lu_stage,
+                              sizeof(uint32_t) * (size_t)g.ctx->sm_count * kLuPerSm * (size_t)g.cap, "union stage")))
+            return rc;
+        g.lu_stage_cap = g.cap;
+    }
+    if (g.pos_valid || g.n == 0) return KH_OK;
+    int* cnt = g.clsw + 33 * ng;  // 32 class counters per graph behind the table
+    const int aligned = positions_aligned(g) ? 1 : 0;
+    KH_CUDA_TRY(g.ctx, cudaMemsetAsync(cnt, 0, sizeof(int) * 32 * (size_t)ng, s));
+    const int grid = (int)((g.n + 255) / 256 < g.ctx->sm_count * 8 ? (g.n + 255) / 256 : g.ctx->sm_count * 8);
+    k_pos_pass<<<grid, 256, 0, s>>>(g.rank, g.gid, g.n, cnt, nullptr);
+    k_pos_classes<<<(int)((ng + 7) / 8 < 1024 ? (ng + 7) / 8 : 1024), 256, 0, s>>>(cnt, ng, g.vtx_off, g.clsw,
+                                                                                  g.wrank, aligned);
+    k_pos_pass<<<grid, 256, 0, s>>>(g.rank, g.gid, g.n, cnt, g.key32);
+    count_launch(g, 3);
+    KH_CUDA_TRY(g.ctx, cudaGetLastError());
+    g.pos_valid = true;
+    return KH_OK;
 }
 
 int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
@@ -1514,7 +1610,10 @@ int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
     a.rowptr = g.rowptr;
     a.col = g.col;
     a.alive = g.alive;
-    a.rank = g.rank;
+    a.key32 = g.key32;
+    a.clsw = g.clsw;
+    a.wrank = g.wrank;
+    a.vtx_off = g.vtx_off;
     a.n = g.n;
     a.level = round_mode == 2 ? 0 : level;  // the refine computes each node's last level
     a.h = g.h;
@@ -1524,16 +1623,14 @@ int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
     a.Mv = g.Mv;
     a.cap = g.cap;
     a.keys = g.keys;
-    a.lsz = g.lsz;
-    a.lk = g.lk;
-    a.ltop = g.ltop;
+    a.meta = g.meta;
+    a.stage = g.lu_stage;
     a.est = g.d64;
     a.worklist = worklist;
     a.d_count = d_count;
     a.count_static = count_static;
     a.track = track;
     a.changed = g.listC[level & 1];
-    a.heavy = g.listH;
     a.err = &g.state->err;
     a.updates = &g.state->updates;
     const bool stop = round_mode == 2;
@@ -1548,26 +1645,26 @@ int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
     a.lvl_changed = g.state->lvl_changed;
     a.stopped = &g.state->stopped;
     int* rc = g.state->rc;
+    int* sub_ctr = nullptr;  // work counter of the parts launch
     if (round_mode == 1) {
         a.n_changed = rc + kRcC + level;
-        a.n_heavy = rc + kRcLevelHeavy + level;
         a.work_ctr = rc + kRcLevelWork + level;
         a.n_sub = rc + kRcSub + level;
+        sub_ctr = rc + kRcSubWork + level;
     } else if (round_mode == 2) {
         a.n_changed = rc + kRcC + 0;  // unused: the refine does not track changes
-        a.n_heavy = rc + kRcRefineHeavy;
         a.work_ctr = rc + kRcRefineWork;
         a.n_sub = rc + kRcSub + 0;
+        sub_ctr = rc + kRcSubWork + 0;
     } else {
         a.n_changed = &g.state->nC[level & 1];
-        a.n_heavy = &g.state->nH;
         a.work_ctr = &g.state->work_ctr[1];
         a.n_sub = &g.state->nSub;
+        sub_ctr = &g.state->work_ctr[3];
     }
     a.part_cap = g.part_cap;
     a.part_keys = g.part_keys;
-    a.part_size = g.part_size;
-    a.part_t = g.part_t;
+    a.part_meta = g.part_meta;
     a.part_done = g.part_done;
     a.part_stop = g.part_stop;
     a.part_lb = g.part_lb;
@@ -1585,63 +1682,65 @@ int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
     const bool wantU = round_mode == 2 ? g.hmax >= 2 : level >= 2;
     if (want1) {
         a.bytes = &g.state->bytes[kProfLevel1];
-        if (round_mode == 0) {
-            e = cudaMemsetAsync(a.n_heavy, 0, sizeof(int), s);
-            if (e != cudaSuccess) return check_cuda(g.ctx, e, "memset n_heavy");
-        }
         int64_t grid = (work + (kL1Threads / 32) - 1) / (kL1Threads / 32);
         const int64_t gmax = (int64_t)g.ctx->sm_count * 8;
         if (grid > gmax) grid = gmax;
         if (grid < 1) grid = 1;
         prof_begin(g, kProfLevel1, s);
         k_level1<<<(int)grid, kL1Threads, 0, s>>>(a);
-        k_level1_heavy<<<g.ctx->sm_count * 2, kL1Threads, 0, s>>>(a);
-        count_launch(g, 2);
+        count_launch(g, 1);
         prof_end(g, kProfLevel1, s);
     }
     if (!wantU) return KH_OK;
     a.bytes = &g.state->bytes[kProfLevelU];
-    const int lg = table_lg(g.M);
-    const int scap = levelU_stage_cap(lg, g.M);
-    const size_t dyn = levelU_smem(lg, scap);
-    // free-running lane groups unless another schedule is asked for (grouped
-    // is the fastest, or within 2%, on every measured workload)
-    void (*kern)(LevelArgs, int, int) =
-        g.levelu_mode == KH_LEVELU_STEPPED ? k_levelU<false> : k_levelU<true>;
-    a.group_lists = g.levelu_mode == KH_LEVELU_FREE ? 0 : 1;
-    a.group_div = g.levelu_div > 0 ? g.levelu_div : kGroupDivDefault;
+    a.lg = table_lg(g.M);
+    a.bm_words = positions_aligned(g) ? 1 << a.lg : -1;
+    const size_t dyn = (size_t)4 << a.lg;
+    a.group_lists = g.levelu_mode == KH_VAR_AUTO || g.levelu_mode == KH_LEVELU_GROUPED;
+    a.group_shift = 0;
+    while ((1 << a.group_shift) < g.levelu_div) ++a.group_shift;
+    // the nodes' last level only, stored lists only, or both (whole passes over a
+    // batch of mixed h); with or without split nodes
+    const bool any_last = round_mode == 2 || (!a.skip_last && level >= g.hmin);
+    const bool any_list = round_mode != 2 && level < g.hmax;
+    const bool parts = g.part_cap > 0;
+    void (*kern)(LevelArgs) = any_last && any_list ? k_levelU<true, true, false>
+                              : any_last           ? k_levelU<true, false, false>
+                                                   : k_levelU<false, true, false>;
+    void (*pkern)(LevelArgs) = any_last && any_list ? k_levelU<true, true, true>
+                               : any_last           ? k_levelU<true, false, true>
+                                                    : k_levelU<false, true, true>;
     // the largest table any graph can ask for (M up to kMaxM)
-    const int lg_max = table_lg(kMaxM);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)levelU_smem(lg_max, levelU_stage_cap(lg_max, kMaxM)));
+                             4 << table_lg(kMaxM));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(pkern, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << table_lg(kMaxM));
     if (e != cudaSuccess) return check_cuda(g.ctx, e, "cudaFuncSetAttribute(k_levelU)");
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kLuThreads, dyn);
     if (e != cudaSuccess) return check_cuda(g.ctx, e, "occupancy(k_levelU)");
     if (per_sm < 1) per_sm = 1;
+    if (per_sm > kLuPerSm) per_sm = kLuPerSm;
     int64_t grid = (int64_t)g.ctx->sm_count * per_sm;
     if (work < grid) grid = work;
     if (grid < 1) grid = 1;
     if (round_mode == 0) {
         e = cudaMemsetAsync(a.work_ctr, 0, sizeof(int), s);
         if (e != cudaSuccess) return check_cuda(g.ctx, e, "memset work_ctr");
-        if (g.part_cap > 0) {
+        if (parts) {
             e = cudaMemsetAsync(a.n_sub, 0, sizeof(int), s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(sub_ctr, 0, sizeof(int), s);
             if (e != cudaSuccess) return check_cuda(g.ctx, e, "memset n_sub");
         }
     }
     prof_begin(g, kProfLevelU, s);
-    if (g.part_cap > 0) {
-        k_split_plan<<<g.ctx->sm_count * 2, 256, 0, s>>>(a);
-        count_launch(g, 1);
-        // parts need CTAs of their own beyond the node count
-        const int64_t cap = (int64_t)g.ctx->sm_count * per_sm;
-        grid = cap;
-    } else {
-        a.n_sub = nullptr;
-    }
-    kern<<<(int)grid, kLuThreads, dyn, s>>>(a, lg, scap);
+    kern<<<(int)grid, kLuThreads, dyn, s>>>(a);
     count_launch(g, 1);
+    if (parts) {
+        a.work_ctr = sub_ctr;
+        pkern<<<g.ctx->sm_count * per_sm, kLuThreads, dyn, s>>>(a);
+        count_launch(g, 1);
+    }
     prof_end(g, kProfLevelU, s);
     return KH_OK;
 }
@@ -1653,7 +1752,7 @@ void launch_mark_neighbours(Graph& g, const int* list1, const int* cnt1, const i
     MarkFilter f{};
     if (list2) {
         f.rho = g.rho;
-        f.lk = g.lk + (size_t)(phase - 1) * (size_t)g.n;
+        f.meta = g.meta + (size_t)(phase - 1) * (size_t)g.n;
         f.hv = g.hv;
         f.h = g.h;
         f.fresh = g.fresh;
@@ -1667,20 +1766,20 @@ void launch_mark_neighbours(Graph& g, const int* list1, const int* cnt1, const i
 
 // lvl_out[v] = k[v, h(v)], bs_out[v] = |B[v, h(v)]| (each node's last level)
 __global__ void k_gather_last(int64_t n, int h_all, const uint8_t* __restrict__ hv,
-                              const int32_t* __restrict__ lsz, const uint8_t* __restrict__ lk,
-                              uint8_t* __restrict__ lvl_out, int32_t* __restrict__ bs_out) {
+                              const uint32_t* __restrict__ meta, uint8_t* __restrict__ lvl_out,
+                              int32_t* __restrict__ bs_out) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const int h = hv ? (int)hv[v] : h_all;
-        const size_t at = (size_t)(h - 1) * (size_t)n + (size_t)v;
-        if (lvl_out) lvl_out[v] = lk[at];
-        if (bs_out) bs_out[v] = lsz[at];
+        const uint32_t m = meta[(size_t)(h - 1) * (size_t)n + (size_t)v];
+        if (lvl_out) lvl_out[v] = (uint8_t)meta_k(m);
+        if (bs_out) bs_out[v] = meta_size(m);
     }
 }
 
 void launch_gather_last(Graph& g, uint8_t* lvl_out, int32_t* bs_out, cudaStream_t s) {
     if (g.n == 0) return;
-    k_gather_last<<<g.ctx->sm_count * 4, 256, 0, s>>>(g.n, g.h, g.hv, g.lsz, g.lk, lvl_out, bs_out);
+    k_gather_last<<<g.ctx->sm_count * 4, 256, 0, s>>>(g.n, g.h, g.hv, g.meta, lvl_out, bs_out);
     count_launch(g, 1);
 }
 
@@ -1688,10 +1787,9 @@ void launch_stale_sampled(Graph& g, const int* list, const int* d_count, cudaStr
     if (g.n == 0) return;
     const int grid = g.ctx->sm_count * 8;
     prof_begin(g, kProfFrontier, s);
-    k_stale_sampled<<<grid, kLuThreads, 0, s>>>(g.rowptr, g.col, g.alive, g.rank, g.lsz, g.lk, g.h,
-                                                g.hv, g.M, g.Mv, only_h, list, d_count, g.n,
-                                                g.fresh, g.lb64, &g.state->bytes[kProfFrontier],
-                                                g.bestnb);
+    k_stale_sampled<<<grid, kStaleThreads, 0, s>>>(g.rowptr, g.col, g.alive, g.rank, g.meta, g.h, g.hv,
+                                                   g.M, g.Mv, only_h, list, d_count, g.n, g.fresh,
+                                                   g.lb64, &g.state->bytes[kProfFrontier], g.bestnb);
     count_launch(g, 1);
     prof_end(g, kProfFrontier, s);
 }
