@@ -310,7 +310,7 @@ int kh_hdegree_exact_noalloc(int64_t n, const int64_t *rowptr, const int32_t *co
 /* KH_OP_HDEG2_SWEEP: the whole-graph exact 2-degrees (kh_hdegree_exact at
  * h = 2 with a sliced layout) may hand the sources of largest 2-hop work
  * (sum of their neighbours' degrees) to bit-parallel sweeps: one pass over
- * every row per batch of 128 sources, with 128-bit source masks per node.
+ * every row per batch of 1024 sources, with 1024-bit source masks per node.
  * KH_VAR_AUTO: the tuner decides the threshold; KH_SWEEP_OFF: never;
  * KH_SWEEP_FROM: the sources of work >= 2^slices - 1 (slices in [1, 48)).
  * kh_get_variant with this op reports KH_SWEEP_OFF or KH_SWEEP_FROM and the

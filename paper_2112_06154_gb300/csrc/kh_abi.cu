@@ -282,7 +282,7 @@ static void free_graph_arrays(Graph& g) {
     dfree(&g.degX);
     dfree(&g.lb64);
     dfree(&g.order2);
-    dfree(&g.sw_m1);
+    for (int i = 0; i < 3; ++i) dfree(&g.sw_m[i]);
     dfree(&g.sw_filter);
     dfree(&g.sw_hpos);
     dfree(&g.sw_piece_h);

@@ -21,8 +21,8 @@
 //
 // Two more kernels serve the same pass: sources of small 2-hop work on one
 // warp each with a private hash set (k_hdeg2_small), and, for the sources of
-// the largest 2-hop work, bit-parallel sweeps of 128 sources at a time
-// (k_sweep_*; see the comment above them).
+// the largest 2-hop work, bit-parallel sweeps of 1024 sources at a time
+// (k_sweep_*; see the comment above them), which also serve h >= 3.
 #include <vector>
 
 #include "kh_internal.cuh"
@@ -373,50 +373,80 @@ __global__ void k_init2(const int64_t* __restrict__ rowptr, const uint8_t* __res
     }
 }
 
-// ---- bit-parallel sweeps for the sources of largest 2-hop work ----
-// For a batch of up to 128 sources s_j, m1[u] holds bit j when u is a
-// neighbour of s_j.  A node x lies in N(s_j; 2) exactly when bit j is set in
-// m1[x] | OR_{u in A(x)} m1[u] (x = s_j itself through any neighbour u, as s_j
-// is in A(u)).  One sweep over all rows thus gives the 2-balls of 128 sources:
-// it reads each row once (2m column ids and 2m 16-byte gathers from m1, which
-// stays in L2), where the per-source union reads sum_{w in A(s_j)} deg(w)
-// entries for each source.  It pays off for sources whose 2-hop work exceeds
-// about one pass over the graph per batch.  A filter of one bit per 4 nodes
-// (some of them has source bits), held in shared memory by the count kernel,
-// skips the gathers of entries that cannot contribute: for batches of
-// mid-size sources half of all entries or more.
-constexpr int kSweepSrc = 128;
-constexpr int kSweepHead = 64;     // row entries the count kernel reads itself (8 per lane)
-constexpr int kSweepPiece = 2048;  // entries per tail piece of a longer row
+// ---- bit-parallel searches of 1024 sources at a time ----
+// For a batch of up to 1024 sources s_j, m[u] holds bit j when u is within i
+// hops of s_j (32 words per node).  One pull over all rows, m'[x] = m[x] | OR_{u
+// in A(x)} m[u], adds a hop.  The first hop is set by scattering the sources'
+// rows (without s_j itself: s_j is a neighbour of its neighbours, so it joins
+// at hop 2); the last pull only counts the set bits per source.  A pull reads
+// each row once and gathers 128 bytes per entry, for 1024 sources, where a
+// search per source reads the rows of its (h-1)-ball: it pays for the sources
+// of largest 2-hop work at h = 2 (kh_tune.cu) and for whole graphs at h >= 3
+// whose balls are large (run_hdeg_full).
+//
+// What bounds it: the gathers, from L2 where the masks of the batch fit (128 n
+// bytes).  128-byte masks fill whole sectors and spread the per-row work (row
+// bounds, reduction, counting) over 1024 sources: the 16-byte masks of the
+// first version used half of each sector and took 8 times the row passes.
+// Measured: exact 3-degrees of Chung-Lu n = 200k 128 (a search per source) -> 28
+// ms, 4-degrees of Chung-Lu n = 60k 277 -> 7.4 ms, of R-MAT 15 78 -> 2.4 ms;
+// exact 2-degrees of R-MAT 20 140 -> 101 ms, of R-MAT 18 21.6 -> 13.9 ms.  A
+// batch on Chung-Lu n = 200k: a storing pull 75 us (6.8 TB/s of gathers), long-row
+// pieces 17 us, seeding and clearing 8 us each.
+constexpr int kSweepWords = 32;
+constexpr int kSweepSrc = 32 * kSweepWords;
+constexpr int kSweepHead = 128;    // longer rows are OR'd in pieces by k_sweep_pieces
+constexpr int kSweepPiece = 128;   // entries per piece
 constexpr int kSweepPlanes = 8;    // carry-save counter planes: 255 additions between flushes
+constexpr int kSweepThreads = 256;
+constexpr int kSweepPullSm = 5;    // CTAs per SM of a pull that stores, one that counts
+constexpr int kSweepCountSm = 4;
 
-// Set (clear = 0) or zero (clear = 1) the batch's source bits on the
-// neighbours of its sources, one CTA per source (the largest sources' rows
-// hold up to the maximum degree); the setting pass also counts each source's
-// algorithmic bytes (those of one 2-hop search).
-__global__ void k_sweep_scatter(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                const int32_t* __restrict__ src, int nb, uint32_t* __restrict__ m1,
-                                uint32_t* __restrict__ filter, int clear, unsigned long long* bytes) {
+// Set the batch's source bits on the neighbours of its sources, one CTA per
+// source; with bytes also the algorithmic bytes of one 2-hop search per source.
+__global__ void k_sweep_seed(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                             const int32_t* __restrict__ src, uint32_t* __restrict__ m,
+                             uint32_t* __restrict__ filter, unsigned long long* bytes) {
     const int j = blockIdx.x;
-    if (j >= nb) return;
     const int v = src[j];
     const int64_t b = rowptr[v], e = rowptr[v + 1];
     unsigned long long my = 0;
     for (int64_t k = b + threadIdx.x; k < e; k += blockDim.x) {
         const int32_t u = __ldg(col + k);
-        if (clear) {
-            reinterpret_cast<uint4*>(m1)[u] = make_uint4(0u, 0u, 0u, 0u);
-            filter[u >> 7] = 0u;
-        } else {
-            atomicOr(m1 + 4 * (size_t)u + (j >> 5), 1u << (j & 31));
-            atomicOr(filter + (u >> 7), 1u << ((u >> 2) & 31));
-            my += 8ull + 4ull * (unsigned long long)(rowptr[u + 1] - rowptr[u]);
-        }
+        atomicOr(m + (size_t)u * kSweepWords + (j >> 5), 1u << (j & 31));
+        const uint32_t bit = 1u << (u & 31);
+        if (!(*(volatile uint32_t*)(filter + (u >> 5)) & bit)) atomicOr(filter + (u >> 5), bit);
+        if (bytes) my += 8ull + 4ull * (unsigned long long)(rowptr[u + 1] - rowptr[u]);
     }
-    if (clear) return;
+    if (!bytes) return;
     if (threadIdx.x == 0) my += 8ull + 4ull * (unsigned long long)(e - b) + 4ull;
     for (int off = 16; off > 0; off >>= 1) my += __shfl_down_sync(kFull, my, off);
     if ((threadIdx.x & 31) == 0 && my) atomicAdd(bytes, my);
+}
+
+// End of a batch, one CTA per source: deg_h (the ball holds the source itself),
+// the counter and the source bits back to zero.
+__global__ void k_sweep_finish(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                               const int32_t* __restrict__ src, uint4* __restrict__ m,
+                               uint32_t* __restrict__ filter, unsigned int* __restrict__ cnt,
+                               int32_t* __restrict__ deg, unsigned long long* updates,
+                               unsigned long long* bytes, unsigned long long batch_bytes) {
+    const int j = blockIdx.x;
+    const int v = src[j];
+    const int64_t b = rowptr[v], e = rowptr[v + 1];
+    for (int64_t k = b + (threadIdx.x >> 3); k < e; k += blockDim.x >> 3) {
+        const int32_t u = __ldg(col + k);
+        m[(size_t)u * 8 + (threadIdx.x & 7)] = make_uint4(0u, 0u, 0u, 0u);
+        if ((threadIdx.x & 7) == 0) filter[u >> 5] = 0u;
+    }
+    if (threadIdx.x != 0) return;
+    const int at = 32 * (j & 31) + (j >> 5);  // flush_planes' order
+    deg[v] = (int32_t)cnt[at] - 1;
+    cnt[at] = 0u;
+    if (j == 0) {
+        atomicAdd(updates, (unsigned long long)gridDim.x);
+        if (batch_bytes) atomicAdd(bytes, batch_bytes);
+    }
 }
 
 __device__ __forceinline__ void or4(uint4& a, const uint4 b) {
@@ -426,13 +456,63 @@ __device__ __forceinline__ void or4(uint4& a, const uint4 b) {
     a.w |= b.w;
 }
 
-// Rows longer than kSweepHead: the OR of m1 over each tail piece of
-// kSweepPiece entries, into that row's partial word bh (zeroed per sweep).
-__global__ void k_sweep_tails(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                              const int32_t* __restrict__ hnode, const int32_t* __restrict__ piece_h,
-                              const int32_t* __restrict__ piece_off, int64_t npieces,
-                              const uint4* __restrict__ m1, const uint32_t* __restrict__ filter,
-                              uint32_t* __restrict__ bh) {
+// The mask word a lane holds after or_row: lane = 8 sub + l8 reads the l8-th 16
+// bytes of a mask and keeps one of their four words.
+__device__ __forceinline__ int or_row_word(int lane) {
+    const int sub = lane >> 3;
+    return (lane & 7) * 4 + (sub & 2) + (sub & 1);
+}
+
+// OR of the masks of one warp's row entries [b, e), entry b + lane already in c:
+// four entries per load (8 lanes of 16 bytes each), four loads in flight.
+// FILTER: entries whose node has no bits are dropped first (buf: 32 ints of
+// shared memory per warp).
+template <bool FILTER>
+__device__ __forceinline__ uint32_t or_row(const int32_t* __restrict__ col, int64_t b, int64_t e, int32_t c,
+                                           const uint4* __restrict__ m, const uint32_t* __restrict__ filter,
+                                           int32_t* buf, int lane) {
+    const int sub = lane >> 3, l8 = lane & 7;
+    uint4 acc = make_uint4(0u, 0u, 0u, 0u);
+    while (b < e) {
+        const int32_t cn = b + 32 + lane < e ? __ldg(col + b + 32 + lane) : 0;  // the next 32
+        int cnt = (int)(e - b < 32 ? e - b : 32);
+        if (FILTER) {
+            const bool live = lane < cnt && ((__ldg(filter + (c >> 5)) >> (c & 31)) & 1u);
+            const uint32_t lm = __ballot_sync(kFull, live);
+            cnt = __popc(lm);
+            if (live) buf[__popc(lm & ((1u << lane) - 1u))] = c;
+            __syncwarp();
+            c = buf[lane];
+            __syncwarp();
+        }
+#pragma unroll 1
+        for (int j0 = 0; j0 < cnt; j0 += 16) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+                const int32_t u = __shfl_sync(kFull, c, j0 + j + sub);
+                if (j0 + j + sub < cnt) or4(acc, __ldg(m + (size_t)u * 8 + l8));
+            }
+        }
+        b += 32;
+        c = cn;
+    }
+    // OR over the four subgroups; each lane keeps one of its chunk's four words
+    const bool hi = sub & 2, odd = sub & 1;
+    uint32_t k0 = hi ? acc.z : acc.x, k1 = hi ? acc.w : acc.y;
+    k0 |= __shfl_xor_sync(kFull, hi ? acc.x : acc.z, 16);
+    k1 |= __shfl_xor_sync(kFull, hi ? acc.y : acc.w, 16);
+    return (odd ? k1 : k0) | __shfl_xor_sync(kFull, odd ? k0 : k1, 8);
+}
+
+// Rows longer than kSweepHead: the OR over each piece of kSweepPiece entries
+// into the row's words of bh (zero before).  One warp per piece.
+template <bool FILTER>
+__global__ void __launch_bounds__(kSweepThreads)
+    k_sweep_pieces(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                   const int32_t* __restrict__ hnode, const int32_t* __restrict__ piece_h,
+                   const int32_t* __restrict__ piece_off, int64_t npieces, const uint4* __restrict__ m,
+                   const uint32_t* __restrict__ filter, uint32_t* __restrict__ bh) {
+    __shared__ int32_t s_buf[kSweepThreads / 32][32];
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < npieces; p += nw) {
@@ -441,121 +521,108 @@ __global__ void k_sweep_tails(const int64_t* __restrict__ rowptr, const int32_t*
         const int64_t b = rowptr[x] + piece_off[p];
         const int64_t re = rowptr[x + 1];
         const int64_t e = b + kSweepPiece < re ? b + kSweepPiece : re;
-        uint4 acc = make_uint4(0u, 0u, 0u, 0u);
-        for (int64_t k = b + lane; k < e; k += 32) {
-            const int32_t u = __ldg(col + k);
-            if ((__ldg(filter + (u >> 7)) >> ((u >> 2) & 31)) & 1u) or4(acc, __ldg(m1 + u));
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            acc.x |= __shfl_xor_sync(kFull, acc.x, off);
-            acc.y |= __shfl_xor_sync(kFull, acc.y, off);
-            acc.z |= __shfl_xor_sync(kFull, acc.z, off);
-            acc.w |= __shfl_xor_sync(kFull, acc.w, off);
-        }
-        if (lane < 4) {
-            const uint32_t w = lane == 0 ? acc.x : lane == 1 ? acc.y : lane == 2 ? acc.z : acc.w;
-            if (w) atomicOr(bh + 4 * (size_t)h + lane, w);
-        }
+        const uint32_t r = or_row<FILTER>(col, b, e, b + lane < e ? __ldg(col + b + lane) : 0, m, filter,
+                                          s_buf[threadIdx.x >> 5], lane);
+        if (r) atomicOr(bh + (size_t)h * kSweepWords + or_row_word(lane), r);
     }
 }
 
-// Add the counts held in carry-save planes (bit `bit` of plane p is worth
-// 2^p) to the block's per-source counters; lane gl of a group owns bits
-// [16 gl, 16 gl + 16) of the ball word.
-__device__ __forceinline__ void sweep_flush(uint32_t (&c)[kSweepPlanes], unsigned int* s_cnt, int gl) {
+// Add the counts held in a lane's carry-save planes (bit `bit` of plane p is
+// worth 2^p, for source 32 word + bit) to s_cnt[32 bit + word] (the lanes' words
+// are all different: no bank conflicts), four bits at a time as bytes.
+__device__ __forceinline__ void flush_planes(uint32_t (&c)[kSweepPlanes], unsigned int* s_cnt, int word) {
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i) {
+        uint32_t t = 0;
 #pragma unroll
-    for (int bit = 0; bit < 16; ++bit) {
-        unsigned int v = 0;
+        for (int p = 0; p < kSweepPlanes; ++p) t |= ((c[p] >> i) & 0x01010101u) << p;
 #pragma unroll
-        for (int p = 0; p < kSweepPlanes; ++p) v |= ((c[p] >> bit) & 1u) << p;
-        if (v) atomicAdd(&s_cnt[16 * gl + bit], v);
+        for (int q = 0; q < 4; ++q) {
+            const unsigned int v = (t >> (8 * q)) & 255u;
+            if (v) atomicAdd(&s_cnt[32 * (i + 8 * q) + word], v);
+        }
     }
 #pragma unroll
     for (int p = 0; p < kSweepPlanes; ++p) c[p] = 0u;
 }
 
-// Ball words of every node (groups of 8 lanes per node, four nodes per warp
-// step; a row's first kSweepHead entries here, the rest from bh) and the
-// number of nodes in each source's ball (per-lane carry-save counters of 16
-// source bits, flushed every 255 nodes).  With use_filter the filter's
-// fwords words are first copied to shared memory.
-__global__ void __launch_bounds__(1024) k_sweep_count(const int64_t* __restrict__ rowptr,
-                                                      const int32_t* __restrict__ col, int64_t n,
-                                                      const uint4* __restrict__ m1,
-                                                      const uint32_t* __restrict__ filter,
-                                                      int use_filter, int fwords,
-                                                      const int32_t* __restrict__ hpos,
-                                                      const uint4* __restrict__ bh,
-                                                      unsigned int* __restrict__ cnt) {
-    extern __shared__ __align__(16) uint32_t s_filter[];
-    __shared__ unsigned int s_cnt[kSweepSrc];
-    for (int i = threadIdx.x; i < kSweepSrc; i += blockDim.x) s_cnt[i] = 0u;
-    if (use_filter) {
-        const uint4* f4 = reinterpret_cast<const uint4*>(filter);
-        uint4* s4 = reinterpret_cast<uint4*>(s_filter);
-        for (int i = threadIdx.x; i < (fwords >> 2); i += blockDim.x) s4[i] = f4[i];
+// One pull over every row, a warp per row.  STORE: m'[x] to out; COUNT: the
+// number of nodes with bit 32 w + b into cnt[32 b + w] (carry-save counters, a
+// mask word per lane).
+template <bool FILTER, bool STORE, bool COUNT>
+__global__ void __launch_bounds__(kSweepThreads, COUNT ? kSweepCountSm : kSweepPullSm)
+    k_sweep_pull(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n,
+                 const uint32_t* __restrict__ m, const uint32_t* __restrict__ filter,
+                 const int32_t* __restrict__ hpos, uint32_t* __restrict__ bh, uint32_t* __restrict__ out, unsigned int* __restrict__ cnt) {
+    __shared__ int32_t s_buf[kSweepThreads / 32][32];
+    __shared__ unsigned int s_cnt[COUNT ? kSweepSrc : 1];
+    const int lane = threadIdx.x & 31;
+    if (COUNT) {
+        for (int i = threadIdx.x; i < kSweepSrc; i += blockDim.x) s_cnt[i] = 0u;
+        __syncthreads();
     }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, g = lane >> 3, gl = lane & 7;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     uint32_t c[kSweepPlanes];
 #pragma unroll
     for (int p = 0; p < kSweepPlanes; ++p) c[p] = 0u;
+    const int word = or_row_word(lane);
     int adds = 0;
-    // the loop bound is the same for the whole warp (the shuffles need every lane)
-    for (int64_t x0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; x0 < n; x0 += nw * 4) {
-        const int64_t x = x0 + g;
-        uint4 acc = make_uint4(0u, 0u, 0u, 0u);
-        if (x < n) {
-            const int64_t b = rowptr[x], e = rowptr[x + 1];
-            if (e > b) {
-                if (gl == 0) acc = m1[x];
-                const int64_t he = e - b > kSweepHead ? b + kSweepHead : e;
-                if (use_filter) {
-                    for (int64_t k = b + gl; k < he; k += 8) {
-                        const int32_t u = __ldg(col + k);
-                        if ((s_filter[u >> 7] >> ((u >> 2) & 31)) & 1u) or4(acc, __ldg(m1 + u));
-                    }
-                } else {
-                    for (int64_t k = b + gl; k < he; k += 8) or4(acc, __ldg(m1 + __ldg(col + k)));
-                }
-                if (gl == 1 && e - b > kSweepHead) or4(acc, bh[hpos[x]]);
-            }
+    // a row is a chain of three loads (bounds, columns, masks): the bounds are
+    // loaded two rows ahead and the first columns one row ahead
+    int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    int64_t b1 = 0, e1 = 0, b2 = 0, e2 = 0;
+    int32_t c1 = 0;
+    if (x < n) {
+        b1 = rowptr[x];
+        e1 = rowptr[x + 1];
+        if (b1 + lane < e1) c1 = __ldg(col + b1 + lane);
+    }
+    if (x + nw < n) {
+        b2 = rowptr[x + nw];
+        e2 = rowptr[x + nw + 1];
+    }
+    for (; x < n; x += nw) {
+        const int64_t b = b1, e = e1;
+        const int32_t c0 = c1;
+        b1 = b2;
+        e1 = e2;
+        c1 = b1 + lane < e1 ? __ldg(col + b1 + lane) : 0;
+        b2 = e2 = 0;
+        if (x + 2 * nw < n) {
+            b2 = rowptr[x + 2 * nw];
+            e2 = rowptr[x + 2 * nw + 1];
         }
-        for (int off = 1; off < 8; off <<= 1) {
-            acc.x |= __shfl_xor_sync(kFull, acc.x, off);
-            acc.y |= __shfl_xor_sync(kFull, acc.y, off);
-            acc.z |= __shfl_xor_sync(kFull, acc.z, off);
-            acc.w |= __shfl_xor_sync(kFull, acc.w, off);
+        if (e == b) continue;  // never reached (its words stay zero)
+        const uint32_t own = m[(size_t)x * kSweepWords + word];
+        const bool longrow = e - b > kSweepHead;
+        uint32_t r = or_row<FILTER>(col, b, longrow ? b : e, c0, reinterpret_cast<const uint4*>(m), filter,
+                                    s_buf[threadIdx.x >> 5], lane);
+        if (longrow) {  // its pieces' words, left zero for the next pull
+            uint32_t* w = bh + (size_t)hpos[x] * kSweepWords + word;
+            r = *w;
+            *w = 0u;
         }
-        const int wi = gl >> 1;
-        const uint32_t word = wi == 0 ? acc.x : wi == 1 ? acc.y : wi == 2 ? acc.z : acc.w;
-        uint32_t carry = (gl & 1) ? (word >> 16) : (word & 0xffffu);
+        r |= own;
+        if (STORE) out[(size_t)x * kSweepWords + word] = r;
+        if (COUNT) {
 #pragma unroll
-        for (int p = 0; p < kSweepPlanes; ++p) {
-            const uint32_t t = c[p] & carry;
-            c[p] ^= carry;
-            carry = t;
+            for (int p = 0; p < kSweepPlanes; ++p) {
+                const uint32_t t = c[p] & r;
+                c[p] ^= r;
+                r = t;
+            }
+            ++adds;
         }
-        if (++adds == (1 << kSweepPlanes) - 1) {
-            sweep_flush(c, s_cnt, gl);
+        if (COUNT && adds == (1 << kSweepPlanes) - 1) {
+            flush_planes(c, s_cnt, word);
             adds = 0;
         }
     }
-    sweep_flush(c, s_cnt, gl);
+    if (!COUNT) return;
+    if (adds) flush_planes(c, s_cnt, word);
     __syncthreads();
     for (int i = threadIdx.x; i < kSweepSrc; i += blockDim.x)
         if (s_cnt[i]) atomicAdd(cnt + i, s_cnt[i]);
-}
-
-// deg_2 of the batch's sources (the ball holds the source itself); the
-// counters are zeroed for the next sweep.
-__global__ void k_sweep_finish(const int32_t* __restrict__ src, int nb, unsigned int* __restrict__ cnt,
-                               int32_t* __restrict__ deg, unsigned long long* updates) {
-    const int j = threadIdx.x;
-    if (j < nb) deg[src[j]] = (int32_t)cnt[j] - 1;
-    if (j < kSweepSrc) cnt[j] = 0u;
-    if (j == 0) atomicAdd(updates, (unsigned long long)nb);
 }
 
 }  // namespace
@@ -656,11 +723,18 @@ int64_t hdeg2_sources_from_bin(const Graph& g, int bin) {
     return c;
 }
 
-// The sweep's per-graph arrays: m1 (zeroed), the rows longer than kSweepHead
-// and their tail pieces, the counters.
-static int ensure_sweep(Graph& g, cudaStream_t s) {
-    if (g.sw_m1) return KH_OK;
+// The arrays of the bit-parallel searches at h: mask buffers (zeroed), the
+// node filter, the rows longer than kSweepHead and their pieces, the counters.
+int ensure_sweep(Graph& g, int h, cudaStream_t s) {
+    const int bufs = h == 2 ? 1 : h == 3 ? 2 : 3;
     const size_t n = (size_t)(g.n > 0 ? g.n : 1);
+    int rc;
+    for (int i = 0; i < bufs; ++i) {
+        if (g.sw_m[i]) continue;
+        if ((rc = alloc_bytes(g.ctx, (void**)&g.sw_m[i], 4 * kSweepWords * n, "sweep source bits"))) return rc;
+        KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.sw_m[i], 0, 4 * kSweepWords * n, s));
+    }
+    if (g.sw_ready) return KH_OK;
     std::vector<int64_t> rp((size_t)g.n + 1);
     KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(rp.data(), g.rowptr, sizeof(int64_t) * rp.size(),
                                        cudaMemcpyDeviceToHost, s));
@@ -672,32 +746,26 @@ static int ensure_sweep(Graph& g, cudaStream_t s) {
         const int h = (int)hnode.size();
         hpos[(size_t)x] = h;
         hnode.push_back((int32_t)x);
-        for (int64_t off = kSweepHead; off < d; off += kSweepPiece) {
+        for (int64_t off = 0; off < d; off += kSweepPiece) {
             piece_h.push_back(h);
             piece_off.push_back((int32_t)off);
         }
     }
     const size_t nh = hnode.size() > 0 ? hnode.size() : 1;
     const size_t np = piece_h.size() > 0 ? piece_h.size() : 1;
-    int rc;
-    const size_t fw = ((n + 127) / 128 + 3) & ~(size_t)3;  // filter words, a multiple of 4
-    if ((rc = alloc_bytes(g.ctx, (void**)&g.sw_m1, 16 * n, "sweep source bits")) ||
-        (rc = alloc_bytes(g.ctx, (void**)&g.sw_filter, 4 * fw, "sweep filter")) ||
-        (rc = alloc_bytes(g.ctx, (void**)&g.sw_hpos, 4 * n, "sweep row index")) ||
-        (rc = alloc_bytes(g.ctx, (void**)&g.sw_hnode, 4 * nh, "sweep long rows")) ||
-        (rc = alloc_bytes(g.ctx, (void**)&g.sw_bh, 16 * nh, "sweep tail words")) ||
-        (rc = alloc_bytes(g.ctx, (void**)&g.sw_piece_h, 4 * np, "sweep pieces")) ||
-        (rc = alloc_bytes(g.ctx, (void**)&g.sw_piece_off, 4 * np, "sweep pieces")) ||
-        (rc = alloc_bytes(g.ctx, (void**)&g.sw_cnt, 4 * kSweepSrc, "sweep counts"))) {
-        cudaFree(g.sw_m1); cudaFree(g.sw_filter); cudaFree(g.sw_hpos); cudaFree(g.sw_hnode); cudaFree(g.sw_bh);
-        cudaFree(g.sw_piece_h); cudaFree(g.sw_piece_off); cudaFree(g.sw_cnt);
-        g.sw_m1 = nullptr; g.sw_filter = nullptr; g.sw_hpos = nullptr; g.sw_hnode = nullptr; g.sw_bh = nullptr;
-        g.sw_piece_h = nullptr; g.sw_piece_off = nullptr; g.sw_cnt = nullptr;
+    const size_t fw = (n + 31) / 32;
+    // (an array kept from a call that failed half-way is used as it is)
+    if ((!g.sw_filter && (rc = alloc_bytes(g.ctx, (void**)&g.sw_filter, 4 * fw, "sweep filter"))) ||
+        (!g.sw_hpos && (rc = alloc_bytes(g.ctx, (void**)&g.sw_hpos, 4 * n, "sweep row index"))) ||
+        (!g.sw_hnode && (rc = alloc_bytes(g.ctx, (void**)&g.sw_hnode, 4 * nh, "sweep long rows"))) ||
+        (!g.sw_bh && (rc = alloc_bytes(g.ctx, (void**)&g.sw_bh, 4 * kSweepWords * nh, "sweep long-row words"))) ||
+        (!g.sw_piece_h && (rc = alloc_bytes(g.ctx, (void**)&g.sw_piece_h, 4 * np, "sweep pieces"))) ||
+        (!g.sw_piece_off && (rc = alloc_bytes(g.ctx, (void**)&g.sw_piece_off, 4 * np, "sweep pieces"))) ||
+        (!g.sw_cnt && (rc = alloc_bytes(g.ctx, (void**)&g.sw_cnt, 4 * kSweepSrc, "sweep counts"))))
         return rc;
-    }
-    KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.sw_m1, 0, 16 * n, s));
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.sw_filter, 0, 4 * fw, s));
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.sw_cnt, 0, 4 * kSweepSrc, s));
+    KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.sw_bh, 0, 4 * kSweepWords * nh, s));
     KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(g.sw_hpos, hpos.data(), 4 * n, cudaMemcpyHostToDevice, s));
     if (!hnode.empty()) {
         KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(g.sw_hnode, hnode.data(), 4 * hnode.size(),
@@ -710,50 +778,57 @@ static int ensure_sweep(Graph& g, cudaStream_t s) {
     KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));  // host vectors go out of scope
     g.sw_nheavy = (int64_t)hnode.size();
     g.sw_npieces = (int64_t)piece_h.size();
+    g.sw_ready = true;
     return KH_OK;
 }
 
-int run_sweeps(Graph& g, int32_t* deg, const int32_t* src, int64_t count, cudaStream_t s) {
+int run_sweeps(Graph& g, int32_t* deg, const int32_t* src, int64_t count, int h, cudaStream_t s) {
     if (count <= 0) return KH_OK;
-    int rc = ensure_sweep(g, s);
+    int rc = ensure_sweep(g, h, s);
     if (rc) return rc;
-    // the filter in shared memory while it fits (n up to 7.2M nodes)
-    const size_t n1 = (size_t)(g.n > 0 ? g.n : 1);
-    const int fwords = (int)(((n1 + 127) / 128 + 3) & ~(size_t)3);
-    const size_t fsm = (size_t)fwords * 4;
-    const int use_filter = fsm <= (size_t)kSmem2Max ? 1 : 0;
-    const size_t dyn = use_filter ? fsm : 0;
-    KH_CUDA_TRY(g.ctx, cudaFuncSetAttribute(k_sweep_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)kSmem2Max));
-    int per_sm = 0;
-    KH_CUDA_TRY(g.ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_count, 1024, dyn));
-    if (per_sm < 1) return set_error(g.ctx, KH_EINVAL, "sweep kernel does not fit on an SM");
-    const int cgrid = g.ctx->sm_count * per_sm;
     int64_t tgrid = (g.sw_npieces + 7) / 8;
-    if (tgrid > (int64_t)g.ctx->sm_count * 8) tgrid = (int64_t)g.ctx->sm_count * 8;
-    if (tgrid < 1) tgrid = 1;
+    if (tgrid > g.ctx->sm_count * 8) tgrid = g.ctx->sm_count * 8;
+    // at h = 2 the bytes of one search per source (counted by the scatter); the
+    // longer searches count the rows that their pulls read
+    const unsigned long long batch_bytes =
+        h == 2 ? 0ull : (unsigned long long)(h - 1) * (8ull * g.n + 4ull * g.nnz);
     prof_begin(g, kProfBfs, s);
-    int64_t sweeps = 0;
-    for (int64_t b0 = 0; b0 < count; b0 += kSweepSrc, ++sweeps) {
+    int64_t launches = 0;
+    for (int64_t b0 = 0; b0 < count; b0 += kSweepSrc) {
         const int nb = (int)(count - b0 < kSweepSrc ? count - b0 : kSweepSrc);
-        const int sgrid = nb;
-        k_sweep_scatter<<<sgrid, 256, 0, s>>>(g.rowptr, g.col, src + b0, nb, g.sw_m1, g.sw_filter, 0,
-                                              &g.state->bytes[kProfBfs]);
-        if (g.sw_npieces > 0) {
-            KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.sw_bh, 0, 16 * (size_t)g.sw_nheavy, s));
-            k_sweep_tails<<<(int)tgrid, 256, 0, s>>>(g.rowptr, g.col, g.sw_hnode, g.sw_piece_h,
-                                                     g.sw_piece_off, g.sw_npieces,
-                                                     reinterpret_cast<const uint4*>(g.sw_m1), g.sw_filter,
-                                                     g.sw_bh);
+        k_sweep_seed<<<nb, 256, 0, s>>>(g.rowptr, g.col, src + b0, g.sw_m[0], g.sw_filter,
+                                        h == 2 ? &g.state->bytes[kProfBfs] : nullptr);
+        for (int hop = 2; hop <= h; ++hop) {
+            const bool first = hop == 2, last = hop == h;
+            const uint32_t* in = g.sw_m[first ? 0 : 1 + ((hop - 3) & 1)];
+            uint32_t* out = last ? nullptr : g.sw_m[1 + ((hop - 2) & 1)];
+            const uint4* in4 = reinterpret_cast<const uint4*>(in);
+            if (g.sw_npieces > 0) {
+                if (first)
+                    k_sweep_pieces<true><<<(int)tgrid, kSweepThreads, 0, s>>>(
+                        g.rowptr, g.col, g.sw_hnode, g.sw_piece_h, g.sw_piece_off, g.sw_npieces, in4,
+                        g.sw_filter, g.sw_bh);
+                else
+                    k_sweep_pieces<false><<<(int)tgrid, kSweepThreads, 0, s>>>(
+                        g.rowptr, g.col, g.sw_hnode, g.sw_piece_h, g.sw_piece_off, g.sw_npieces, in4,
+                        g.sw_filter, g.sw_bh);
+                ++launches;
+            }
+            void (*pull)(const int64_t*, const int32_t*, int64_t, const uint32_t*, const uint32_t*,
+                         const int32_t*, uint32_t*, uint32_t*, unsigned int*) =
+                first ? (last ? k_sweep_pull<true, false, true> : k_sweep_pull<true, true, false>)
+                      : (last ? k_sweep_pull<false, false, true> : k_sweep_pull<false, true, false>);
+            // one wave: a second, partial one costs a whole row loop
+            pull<<<g.ctx->sm_count * (last ? kSweepCountSm : kSweepPullSm), kSweepThreads, 0, s>>>(g.rowptr, g.col, g.n, in, g.sw_filter, g.sw_hpos, g.sw_bh,
+                                                 out, g.sw_cnt);
+            ++launches;
         }
-        k_sweep_count<<<cgrid, 1024, dyn, s>>>(g.rowptr, g.col, g.n, reinterpret_cast<const uint4*>(g.sw_m1),
-                                               g.sw_filter, use_filter, fwords, g.sw_hpos,
-                                               reinterpret_cast<const uint4*>(g.sw_bh), g.sw_cnt);
-        k_sweep_finish<<<1, kSweepSrc, 0, s>>>(src + b0, nb, g.sw_cnt, deg, &g.state->updates);
-        k_sweep_scatter<<<sgrid, 256, 0, s>>>(g.rowptr, g.col, src + b0, nb, g.sw_m1, g.sw_filter, 1,
-                                              nullptr);
+        k_sweep_finish<<<nb, 256, 0, s>>>(g.rowptr, g.col, src + b0, reinterpret_cast<uint4*>(g.sw_m[0]),
+                                          g.sw_filter, g.sw_cnt, deg, &g.state->updates,
+                                          &g.state->bytes[kProfBfs], batch_bytes);
+        launches += 2;
     }
-    count_launch(g, sweeps * (g.sw_npieces > 0 ? 5 : 4));
+    count_launch(g, launches);
     prof_end(g, kProfBfs, s);
     KH_CUDA_TRY(g.ctx, cudaGetLastError());
     return KH_OK;

@@ -178,8 +178,11 @@ size_t hdeg2_smem(int64_t width);
 int64_t hdeg2_small_split(const Graph& g);
 // sources of order2 whose 2-hop work is at least 2^bin (they come first)
 int64_t hdeg2_sources_from_bin(const Graph& g, int bin);
-// exact 2-degrees of `count` sources by bit-parallel sweeps of 128 sources
-int run_sweeps(Graph& g, int32_t* deg, const int32_t* src, int64_t count, cudaStream_t s);
+// exact h-degrees (h >= 2) of `count` non-isolated sources by bit-parallel
+// searches of kSweepBatch sources
+constexpr int64_t kSweepBatch = 1024;
+int run_sweeps(Graph& g, int32_t* deg, const int32_t* src, int64_t count, int h, cudaStream_t s);
+int ensure_sweep(Graph& g, int h, cudaStream_t s);
 int launch_hdeg2_small(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s,
                        const int32_t* order, int64_t count);
 // kh_tune.cu: the layout of the 2-degree pass for this graph (tuned once), and
@@ -373,11 +376,12 @@ struct Graph {
     int32_t *order2;
     int64_t nsrc2;
     int64_t order2_hist[48];  // sources per log2 bin of 2-hop work (order2 is by descending bin)
-    // bit-parallel 2-degree sweeps: source bits of the batch per node (128 per
-    // node), node index among the rows longer than the sweep's head (or -1),
-    // those rows' tail pieces and their partial ORs, per-bit ball counts
-    uint32_t* sw_m1;
-    uint32_t* sw_filter;      // one bit per 4 nodes: some of them has source bits in m1
+    // bit-parallel searches (kh_hdeg2.cu): mask buffers (32 words per node; the
+    // first holds a batch's source bits and is zero between batches), node
+    // filter, index of each long row (or -1), the long rows, their pieces and
+    // partial ORs, per-source counts
+    uint32_t* sw_m[3];
+    uint32_t* sw_filter;
     int32_t* sw_hpos;
     int32_t* sw_piece_h;
     int32_t* sw_piece_off;
@@ -385,6 +389,9 @@ struct Graph {
     uint32_t* sw_bh;
     unsigned int* sw_cnt;
     int64_t sw_nheavy, sw_npieces;
+    bool sw_ready;
+    // h >= 3: per-source search or bit-parallel batches (0: not decided yet)
+    int hdeg_deep[kMaxH + 1];
     int sw_force;             // forced sweep threshold bin (0: tuner; -1: no sweeps)
     // each node's neighbour of largest degree (-1: none), for cheap stale bounds
     int32_t *bestnb;

@@ -13,7 +13,7 @@
 // The sliced kernel has two launch parameters: the number of slices S (at
 // least what shared memory requires) and the CTA size.  With a sliced layout
 // the sources of the largest 2-hop work may go to the bit-parallel sweeps
-// (k_sweep_*: 128 sources per pass over the rows), from a work threshold.
+// (k_sweep_*: 1024 sources per pass over the rows), from a work threshold.
 // The tuner times every layout candidate on the same sample of sources (every
 // k-th source of the longest-first order, so every size class is represented)
 // with CUDA events on the context stream, keeps the fastest, then prices the
@@ -257,7 +257,7 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
             if (cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess) {
                 for (int rep = 0; rep < 2; ++rep) {  // the first run also builds the sweep arrays
                     cudaEventRecord(e0, s);
-                    const int rc2 = run_sweeps(g, scratch, g.order2 + first, nb, s);
+                    const int rc2 = run_sweeps(g, scratch, g.order2 + first, nb, 2, s);
                     cudaEventRecord(e1, s);
                     float ms = 0.f;
                     if (rc2 != KH_OK || cudaEventSynchronize(e1) != cudaSuccess ||
@@ -275,7 +275,7 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
             if (e1) cudaEventDestroy(e1);
             return t;
         };
-        const double t_warm = time_sweep(0, std::min<int64_t>(g.nsrc2, 128));  // builds the arrays
+        const double t_warm = time_sweep(0, std::min<int64_t>(g.nsrc2, kSweepBatch));  // builds the arrays
         const double t_none = best.ms * (double)stride;
         double t_best = 0.95 * t_none;
         for (int bin = kOrderBinsMax - 1; t_warm >= 0.0 && bin >= kSweepMinBin; --bin) {
@@ -284,15 +284,15 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
             if (nsw >= g.nsrc2) break;
             const int64_t sbig = (nsw + stride - 1) / stride;  // sample entries that are swept
             if (sbig >= m) break;
-            const int64_t nb_mid = std::min<int64_t>(nsw, 128);
-            const int64_t mid = ((nsw / 2) / 128) * 128;
+            const int64_t nb_mid = std::min<int64_t>(nsw, kSweepBatch);
+            const int64_t mid = ((nsw / 2) / kSweepBatch) * kSweepBatch;
             const double t_mid = time_sweep(mid + nb_mid <= nsw ? mid : nsw - nb_mid, nb_mid);
             if (t_mid < 0.0) break;
             TuneChoice rest = best;
             const double t_rest = time_candidate(g, rest, sample + sbig, d_count, m - sbig, scratch, s,
                                                  sample_big > sbig ? sample_big - sbig : 0);
             if (t_rest < 0.0) break;
-            const double t = (double)((nsw + 127) / 128) * t_mid + t_rest * (double)stride;
+            const double t = (double)((nsw + kSweepBatch - 1) / kSweepBatch) * t_mid + t_rest * (double)stride;
             if (t < t_best) {
                 t_best = t;
                 best.sweep_bin = bin;
@@ -303,6 +303,57 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
     g.tuned_hdeg2 = best;
     table_add(key, best);
     *out = best;
+    return KH_OK;
+}
+
+// h >= 3: bit-parallel batches or a search per source, decided once per graph
+// and h.  The searches' cost per source comes from a probe of a few sources
+// spread over the longest-first order (the device byte counter: 4 bytes a row
+// entry); the batches' cost is known: h - 1 pulls over all rows per 1024 sources.
+// A pull entry (a 128-byte gather, from L2 or, once the masks outgrow it, from
+// HBM) costs about kPullCost search entries (a 4-byte read and a bitmap test):
+// measured 16 ps against 2 ps on Chung-Lu n = 200k.
+constexpr int kProbe = 152;
+constexpr double kPullCost = 8.0;
+constexpr double kBatchOverhead = 1.0e7;  // a batch's launches, in search entries
+
+static int choose_deep(Graph& g, cudaStream_t s, bool* batches) {
+    *batches = false;
+    if (g.nnz == 0) return KH_OK;
+    auto pulls = [&](double sources) {
+        return std::ceil(sources / (double)kSweepBatch) *
+               ((double)(g.h - 1) * (double)(g.nnz + g.n) * kPullCost + kBatchOverhead);
+    };
+    // a search reads at most every row entry: no probe where even that is less
+    if ((double)g.n * (double)g.nnz <= pulls((double)g.n)) return KH_OK;
+    if (g.hdeg_deep[g.h] == 0) {
+        int rc = ensure_order2(g, s);
+        if (rc) return rc;
+        const int64_t stride = (g.nsrc2 + kProbe - 1) / kProbe;
+        const int64_t m = (g.nsrc2 + stride - 1) / stride;
+        const int64_t launches_before = g.launches;
+        k_stride_sample<<<1, 256, 0, s>>>(g.order2, g.nsrc2, stride, g.listB, &g.state->tune_count);
+        unsigned long long b0 = 0, b1 = 0;
+        unsigned long long* ctr = &g.state->bytes[kProfBfs];
+        unsigned long long upd = 0;
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&b0, ctr, sizeof(b0), cudaMemcpyDeviceToHost, s));
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&upd, &g.state->updates, sizeof(upd), cudaMemcpyDeviceToHost, s));
+        const bool prof = g.prof_on;
+        g.prof_on = false;  // the probe is not the caller's work
+        rc = launch_hdeg(g, g.listB, &g.state->tune_count, 0, g.listA, nullptr, 0, 0, s);
+        g.prof_on = prof;
+        if (rc) return rc;
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&b1, ctr, sizeof(b1), cudaMemcpyDeviceToHost, s));
+        KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(ctr, &b0, sizeof(b0), cudaMemcpyHostToDevice, s));
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&g.state->updates, &upd, sizeof(upd), cudaMemcpyHostToDevice, s));
+        KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));  // b0 and upd are host locals
+        g.launches = launches_before;
+        const double search = (double)(b1 - b0) / 4.0 / (double)m * (double)g.nsrc2;
+        g.hdeg_deep[g.h] = search > pulls((double)g.nsrc2) ? 2 : 1;
+    }
+    // (without memory for the masks: a search per source)
+    *batches = g.hdeg_deep[g.h] == 2 && ensure_sweep(g, g.h, s) == KH_OK;
     return KH_OK;
 }
 
@@ -318,12 +369,21 @@ int run_hdeg_full(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStr
             // (2-degrees only: the fixed-level counts stay with the sliced kernel)
             int bin = g.sw_force != 0 ? g.sw_force : c.sweep_bin;
             if (cnt || bin < 0) bin = 0;
-            int64_t nsw = bin > 0 ? hdeg2_sources_from_bin(g, bin) : 0;
+            int64_t nsw = bin > 0 && ensure_sweep(g, 2, s) == KH_OK ? hdeg2_sources_from_bin(g, bin) : 0;
             const int64_t big = hdeg2_small_split(g);
             rc = run_sliced(g, c, deg, cnt, jlo, nj, s, g.order2 + nsw, g.nsrc2 - nsw,
                             big > nsw ? big - nsw : 0);
             if (rc || nsw == 0) return rc;
-            return run_sweeps(g, deg, g.order2, nsw, s);
+            return run_sweeps(g, deg, g.order2, nsw, 2, s);
+        }
+    }
+    if (g.h >= 3 && !g.gid && !cnt && g.n > 0) {
+        bool batches = false;
+        int rc = choose_deep(g, s, &batches);
+        if (rc) return rc;
+        if (batches) {
+            KH_CUDA_TRY(g.ctx, cudaMemsetAsync(deg, 0, sizeof(int32_t) * (size_t)g.n, s));  // isolated nodes
+            return run_sweeps(g, deg, g.order2, g.nsrc2, g.h, s);
         }
     }
     return launch_hdeg(g, nullptr, nullptr, g.n, deg, cnt, jlo, nj, s);
