@@ -236,6 +236,7 @@ static void free_graph_arrays(Graph& g) {
     dfree(&g.rowptr);
     dfree(&g.col);
     dfree(&g.rank);
+    dfree(&g.crank);
     dfree(&g.alive);
     dfree(&g.keys);
     dfree(&g.meta);
@@ -384,10 +385,16 @@ int kh_ctx_create(kh_ctx** out, int device, void* cuda_stream) {
             c->own_stream = false;
         } else {
             e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
-            c->own_stream = true;
+            c->own_stream = e == cudaSuccess;
         }
     }
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming);
     if (e != cudaSuccess) {
+        if (c->fork) cudaEventDestroy(c->fork);
+        if (c->side) cudaStreamDestroy(c->side);
+        if (c->own_stream) cudaStreamDestroy(c->stream);
         free(c);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? KH_ENOMEM : KH_ECUDA;
@@ -399,6 +406,9 @@ int kh_ctx_create(kh_ctx** out, int device, void* cuda_stream) {
 int kh_ctx_destroy(kh_ctx* ctx) {
     if (!ctx) return KH_EINVAL;
     cudaSetDevice(ctx->device);
+    cudaEventDestroy(ctx->fork);
+    cudaEventDestroy(ctx->join);
+    cudaStreamDestroy(ctx->side);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     free(ctx);
     return KH_OK;
@@ -682,6 +692,7 @@ int kh_set_sampling(kh_graph* G, uint64_t seed, int64_t M_or_0, double eps, doub
         g.seed = seed;
         g.ranks_valid = false;
         g.pos_valid = false;
+        g.crank_valid = false;
     }
     return KH_OK;
 }

@@ -23,6 +23,7 @@
 // warp each with a private hash set (k_hdeg2_small), and, for the sources of
 // the largest 2-hop work, bit-parallel sweeps of 1024 sources at a time
 // (k_sweep_*; see the comment above them), which also serve h >= 3.
+#include <cmath>
 #include <vector>
 
 #include "kh_internal.cuh"
@@ -313,6 +314,200 @@ __global__ void __launch_bounds__(kSmallWarps * 32)
     for (int off = 16; off > 0; off >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, off);
     if (lane == 0 && my_bytes) atomicAdd(bytes, my_bytes);
     if (lane == 0 && my_upd) atomicAdd(updates, my_upd);
+}
+
+// One CTA per source with a bitmap of all n nodes (KH_VAR_CTA).  N(v; 2) is the
+// union of the rows of v and of its neighbours; a chunk of neighbours' row
+// bounds is read into shared memory, sorted into short (up to 8 entries), middle
+// (up to 32) and long rows, which groups of 2, 8 and 32 lanes claim and read
+// four entries per lane and step; rows of 512 entries or more are read by the
+// whole CTA.
+//
+// What bounds it: latency (a source is a chain of dependent loads) on small
+// graphs, so the CTA is as small as the bitmap allows (kCtaBitmap bytes of
+// shared memory per 128 threads: 8 sources or more in flight per SM), then the
+// shared-memory tests and atomics, one per row entry.  The search kernel of
+// h >= 3 (a queue, 8 barriers a source, the bitmap walked by 256 threads) took
+// 2.4 ms, the sliced kernel with one slice 5.3 ms for the 2-degrees of Chung-Lu
+// n = 200k; this one 1.7 ms (fixed-level counts 4.6 and 7.2 -> 2.1 ms: the ranks
+// are read along the row, not gathered, and counted in registers).  128 threads
+// for a 25 KB bitmap: 256 took the same time for degrees, 20% longer for counts.
+constexpr int kCtaMaxThreads = 512;
+constexpr int64_t kCtaBitmap = 28 * 1024;
+constexpr int kCtaHeavy = 512;
+
+struct Cta2Args {
+    const int64_t* rowptr;
+    const int32_t* col;
+    const uint8_t* rank;   // of the nodes
+    const uint8_t* crank;  // rank of each column entry
+    int words;             // bitmap words, a multiple of 4
+    const int32_t* order;  // sources, longest first
+    int64_t nsrc;
+    int32_t* deg;
+    int32_t* cnt;
+    int jlo, nj;
+    int* work_ctr;
+    unsigned long long* updates;
+    unsigned long long* bytes;
+};
+
+// Mark u (rank r); returns 1 if it is new.
+template <bool RANKS>
+__device__ __forceinline__ int mark_node(uint32_t* bm, int* s_hist, RankCounts& ranks, int32_t u, int r) {
+    uint32_t* w = bm + (u >> 5);
+    const uint32_t bit = 1u << (u & 31);
+    if ((*(volatile uint32_t*)w & bit) || (atomicOr(w, bit) & bit)) return 0;
+    if (RANKS) ranks.add(r, s_hist);
+    return 1;
+}
+
+template <bool RANKS>
+__global__ void __launch_bounds__(kCtaMaxThreads) k_hdeg2_cta(Cta2Args a) {
+    extern __shared__ __align__(16) uint32_t bm[];
+    const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
+    // per row of the chunk: its start and length; the rows of each bucket
+    int64_t* s_b = reinterpret_cast<int64_t*>(bm + a.words);
+    int* s_len = reinterpret_cast<int*>(s_b + T);
+    uint16_t* s_q = reinterpret_cast<uint16_t*>(s_len + T);
+    __shared__ int s_nq[4], s_cq[4];
+    __shared__ int s_hist[32];
+    __shared__ int s_count, s_idx, s_v;
+    unsigned long long my_bytes = 0;
+    for (int i = tid * 4; i < a.words; i += T * 4)
+        *reinterpret_cast<uint4*>(bm + i) = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+        const int i = atomicAdd(a.work_ctr, 1);
+        s_idx = i;
+        if (i < a.nsrc) s_v = a.order[i];
+    }
+    for (;;) {
+        __syncthreads();
+        if (s_idx >= a.nsrc) break;
+        const int v = s_v;
+        int next = 0;
+        if (tid == 0) next = atomicAdd(a.work_ctr, 1);
+        const int64_t vb = a.rowptr[v];
+        const int deg = (int)(a.rowptr[v + 1] - vb);
+        RankCounts ranks;
+        int my = 0;
+        if (tid == 0) s_count = 0;
+        if (RANKS && tid < 32) s_hist[tid] = 0;
+        for (int c0 = 0; c0 <= deg; c0 += T) {  // rows: each neighbour's, then v's own
+            if (c0) __syncthreads();            // the previous chunk is read
+            if (tid < 4) {
+                s_nq[tid] = 0;
+                s_cq[tid] = 0;
+            }
+            const int i = c0 + tid;
+            int len = 0;
+            if (i <= deg) {
+                const int32_t x = i < deg ? __ldg(a.col + vb + i) : v;
+                const int64_t b = a.rowptr[x];
+                len = (int)(a.rowptr[x + 1] - b);
+                s_b[tid] = b;
+                s_len[tid] = len;
+                my_bytes += 8ull + 4ull * (unsigned long long)len;
+            }
+            const int q = len == 0 ? -1 : len <= 8 ? 0 : len <= 32 ? 1 : len < kCtaHeavy ? 2 : 3;
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t mq = __ballot_sync(kFull, q == k);
+                if (!mq) continue;
+                int base = 0;
+                if (lane == 0) base = atomicAdd(&s_nq[k], __popc(mq));
+                base = __shfl_sync(kFull, base, 0);
+                if (q == k) s_q[k * T + base + __popc(mq & ((1u << lane) - 1u))] = (uint16_t)tid;
+            }
+            __syncthreads();
+            for (int hi = 0; hi < s_nq[3]; ++hi) {
+                const int64_t rb = s_b[s_q[3 * T + hi]];
+                const int n = s_len[s_q[3 * T + hi]];
+                for (int k = tid; k < n; k += 4 * T) {
+                    int32_t u[4];
+                    int r[4];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const bool in = k + p * T < n;
+                        u[p] = in ? __ldg(a.col + rb + k + p * T) : -1;
+                        r[p] = RANKS && in ? __ldg(a.crank + rb + k + p * T) : 0;
+                    }
+                    if (RANKS) ranks.reserve(s_hist);
+#pragma unroll
+                    for (int p = 0; p < 4; ++p)
+                        if (u[p] >= 0) my += mark_node<RANKS>(bm, s_hist, ranks, u[p], r[p]);
+                }
+            }
+            int bk = 2, li = -1, pos = 0, n = 0;
+            int64_t rb = 0;
+            for (;;) {  // as walk_chunk of the level union: groups claim rows
+                const int lgG = bk == 2 ? 5 : bk == 1 ? 3 : 1;
+                const int lead = lane >> lgG << lgG;
+                const uint32_t need = __ballot_sync(kFull, li == -1 && lane == lead);
+                if (need) {
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(&s_cq[bk], __popc(need));
+                    base = __shfl_sync(kFull, base, 0);
+                    if (li == -1) {
+                        const int j = base + __popc(need & ((1u << lead) - 1u));
+                        li = -2;
+                        if (j < s_nq[bk]) {
+                            li = s_q[bk * T + j];
+                            rb = s_b[li];
+                            n = s_len[li];
+                            pos = 0;
+                        }
+                    }
+                }
+                if (__all_sync(kFull, li == -2)) {
+                    do --bk;
+                    while (bk >= 0 && s_nq[bk] == 0);
+                    if (bk < 0) break;
+                    li = -1;
+                    continue;
+                }
+                if (li >= 0) {
+                    int32_t u[4];
+                    int r[4];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const int k = pos + (p << lgG) + lane - lead;
+                        u[p] = k < n ? __ldg(a.col + rb + k) : -1;
+                        r[p] = RANKS && k < n ? __ldg(a.crank + rb + k) : 0;
+                    }
+                    if (RANKS) ranks.reserve(s_hist);
+#pragma unroll
+                    for (int p = 0; p < 4; ++p)
+                        if (u[p] >= 0) my += mark_node<RANKS>(bm, s_hist, ranks, u[p], r[p]);
+                    pos += 4 << lgG;
+                    if (pos >= n) li = -1;
+                }
+            }
+        }
+        int nv = 0;
+        if (tid == 0 && next < a.nsrc) nv = a.order[next];
+        my = __reduce_add_sync(kFull, my);
+        if (lane == 0 && my) atomicAdd(&s_count, my);
+        if (RANKS) ranks.finish(s_hist, lane);
+        __syncthreads();
+        if (tid == 0) {
+            a.deg[v] = s_count - 1;  // the ball holds v itself (by symmetry, in each neighbour's row)
+            atomicAdd(a.updates, 1ull);
+            my_bytes += 4ull + (RANKS ? 4ull * (unsigned long long)a.nj : 0ull);
+            s_idx = next;
+            s_v = nv;
+        }
+        if (RANKS && tid < a.nj) {
+            int c = a.rank[v] >= a.jlo + tid ? -1 : 0;
+            for (int j = a.jlo + tid; j < 32; ++j) c += s_hist[j];
+            a.cnt[(size_t)v * a.nj + tid] = c;
+        }
+        for (int i = tid * 4; i < a.words; i += T * 4)
+            *reinterpret_cast<uint4*>(bm + i) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    for (int off = 16; off > 0; off >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, off);
+    if (lane == 0 && my_bytes) atomicAdd(a.bytes, my_bytes);
 }
 
 // 2-hop work of each node and its log2 bin (isolated nodes: bin -1).
@@ -717,6 +912,19 @@ int launch_hdeg2_small(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cu
     return KH_OK;
 }
 
+// A source of half of a CTA slot's share of the work or more (8 slots per SM) is
+// the tail of the launch when one small CTA reads it: 2-degrees of R-MAT 15 / 16
+// 1.45 / 2.7 ms without large CTAs, 0.75 / 1.75 ms so; from a quarter of the
+// share on the large CTAs take the small ones' place (counts of Chung-Lu n = 200k
+// 2.14 -> 2.5 ms).
+int hdeg2_large_bin(const Graph& g) {
+    double total = 0.0;
+    for (int b = 0; b < kOrderBins; ++b) total += 1.5 * std::ldexp((double)g.order2_hist[b], b);
+    int bin = kCtaSmallBin + 1;
+    while (bin < kOrderBins - 1 && std::ldexp(1.0, bin) < total / (2.0 * 8.0 * g.ctx->sm_count)) ++bin;
+    return bin < 14 ? 14 : bin;
+}
+
 int64_t hdeg2_sources_from_bin(const Graph& g, int bin) {
     int64_t c = 0;
     for (int b = bin < 0 ? 0 : bin; b < kOrderBins; ++b) c += g.order2_hist[b];
@@ -831,6 +1039,69 @@ int run_sweeps(Graph& g, int32_t* deg, const int32_t* src, int64_t count, int h,
     count_launch(g, launches);
     prof_end(g, kProfBfs, s);
     KH_CUDA_TRY(g.ctx, cudaGetLastError());
+    return KH_OK;
+}
+
+int launch_hdeg2_cta(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s,
+                     const int32_t* order, int64_t nsrc, bool large) {
+    if (nsrc <= 0) return KH_OK;
+    Cta2Args a{};
+    a.words = (int)(((g.n + 31) / 32 + 3) & ~(int64_t)3);
+    const int64_t bitmap = (int64_t)a.words * 4;
+    const int threads = large                    ? kCtaMaxThreads
+                        : bitmap <= kCtaBitmap     ? 128
+                        : bitmap <= 2 * kCtaBitmap ? 256
+                                                   : kCtaMaxThreads;
+    const size_t dyn = (size_t)bitmap + (size_t)threads * 20;
+    void (*kern)(Cta2Args) = cnt ? k_hdeg2_cta<true> : k_hdeg2_cta<false>;
+    KH_CUDA_TRY(g.ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)kSmemBitmapMax + 20 * kCtaMaxThreads));
+    int per_sm = 0;
+    KH_CUDA_TRY(g.ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, dyn));
+    if (per_sm < 1) return set_error(g.ctx, KH_EINVAL, "2-degree kernel does not fit on an SM");
+    KH_CUDA_TRY(g.ctx, cudaMemsetAsync(&g.state->work_ctr[large ? 3 : 2], 0, sizeof(int), s));
+    int64_t grid = (int64_t)g.ctx->sm_count * per_sm;
+    if (grid > nsrc) grid = nsrc;
+    a.rowptr = g.rowptr;
+    a.col = g.col;
+    a.rank = g.rank;
+    a.crank = g.crank;
+    a.order = order;
+    a.nsrc = nsrc;
+    a.deg = deg;
+    a.cnt = cnt;
+    a.jlo = jlo;
+    a.nj = nj;
+    a.work_ctr = &g.state->work_ctr[large ? 3 : 2];
+    a.updates = &g.state->updates;
+    a.bytes = &g.state->bytes[kProfBfs];
+    prof_begin(g, kProfBfs, s);
+    kern<<<(int)grid, threads, dyn, s>>>(a);
+    count_launch(g, 1);
+    prof_end(g, kProfBfs, s);
+    return KH_OK;
+}
+
+int launch_init2(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s) {
+    k_init2<<<g.ctx->sm_count * 4, 256, 0, s>>>(g.rowptr, g.rank, g.n, deg, cnt, jlo, nj);
+    count_launch(g, 1);
+    return KH_OK;
+}
+
+__global__ void k_crank(const int32_t* __restrict__ col, const uint8_t* __restrict__ rank, int64_t nnz,
+                        uint8_t* __restrict__ crank) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += stride)
+        crank[k] = rank[col[k]];
+}
+
+int ensure_crank(Graph& g, cudaStream_t s) {
+    if (g.crank_valid || g.nnz == 0) return KH_OK;
+    int rc;
+    if (!g.crank && (rc = alloc_bytes(g.ctx, (void**)&g.crank, (size_t)g.nnz, "column ranks"))) return rc;
+    k_crank<<<g.ctx->sm_count * 8, 256, 0, s>>>(g.col, g.rank, g.nnz, g.crank);
+    count_launch(g, 1);
+    g.crank_valid = true;
     return KH_OK;
 }
 

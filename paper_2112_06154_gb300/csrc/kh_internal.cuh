@@ -170,6 +170,18 @@ void launch_stale_exact(Graph& g, const int* list, const int* d_count, cudaStrea
 // their starting values first (every node); otherwise they must hold them.
 int launch_hdeg2_slice(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s,
                        int slices, int threads, const int32_t* order, int64_t nsrc, bool init);
+// the same with one CTA per source and a bitmap of all n nodes (n <= 819200)
+int launch_hdeg2_cta(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s,
+                     const int32_t* order, int64_t nsrc, bool large);
+int launch_init2(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s);
+// in that layout the sources of `order2` from a bin of 2-hop work on take a large
+// CTA each (hdeg2_large_bin), those below kCtaSmallBin a warp each: below 127
+// entries a warp's hash set costs less than a CTA's barriers (grid of 160k
+// nodes: 0.36 -> 0.16 ms)
+int hdeg2_large_bin(const Graph& g);
+constexpr int kCtaSmallBin = 7;
+// crank: the rank of each column entry (kept until the ranks change)
+int ensure_crank(Graph& g, cudaStream_t s);
 // the sources of the sliced kernel, longest 2-hop work first (cached per graph)
 int ensure_order2(Graph& g, cudaStream_t s);
 size_t hdeg2_smem(int64_t width);
@@ -230,11 +242,72 @@ struct kh_ctx {
     bool own_stream;
     int sm_count;
     char err[512];
+    // a second stream for work beside a launch's own (forked from and joined to
+    // `stream` by the two events)
+    cudaStream_t side;
+    cudaEvent_t fork, join;
     // fault injection on the host: the fail_alloc_at-th device allocation from
     // the arming call fails with KH_ENOMEM (0: off)
     int64_t fail_alloc_at;
     int64_t alloc_count;
 };
+
+#ifdef __CUDACC__
+namespace kh {
+// Lane j adds #{lanes : r >= j} to its count (r = -1: no key; all 32 lanes call
+// it).  Ranks are geometric, so a warp's 32 keys need about 7 ballots (no
+// shared-memory atomics: half the keys of a histogram would fall on one address).
+__device__ __forceinline__ void add_rank_counts(int r, int lane, int& S) {
+#pragma unroll 1
+    for (int j = 0; j < 32; ++j) {
+        const uint32_t b = __ballot_sync(0xffffffffu, r >= j);
+        if (!b) break;
+        if (lane == j) S += __popc(b);
+    }
+}
+
+// A lane's counts of nodes by rank: ranks 0..7 as the bytes of one word, the
+// others (1 node in 256) straight into the shared histogram.  A histogram
+// atomic per node would fall on one address for every second node.
+struct RankCounts {
+    unsigned long long r8 = 0;
+    int since = 0;  // nodes since the last flush; a byte holds 255
+    __device__ __forceinline__ void add(int r, int* s_hist) {
+        if (r < 8) {
+            r8 += 1ull << (8 * r);
+            ++since;
+        } else {
+            atomicAdd(&s_hist[r], 1);
+        }
+    }
+    // before a step that adds up to 5 nodes
+    __device__ __forceinline__ void reserve(int* s_hist) {
+        if (since <= 250) return;
+#pragma unroll 1
+        for (int r = 0; r < 8; ++r) {
+            const int c = (int)(r8 >> (8 * r)) & 255;
+            if (c) atomicAdd(&s_hist[r], c);
+        }
+        r8 = 0;
+        since = 0;
+    }
+    // the warp's counts into the histogram (all 32 lanes): two ranks per sum (32
+    // bytes fit 16 bits), lane r adds rank r
+    __device__ __forceinline__ void finish(int* s_hist, int lane) {
+        const uint32_t lo = (uint32_t)r8, hi = (uint32_t)(r8 >> 32);
+        const uint32_t a = __reduce_add_sync(0xffffffffu, lo & 0x00ff00ffu);
+        const uint32_t b = __reduce_add_sync(0xffffffffu, (lo >> 8) & 0x00ff00ffu);
+        const uint32_t c = __reduce_add_sync(0xffffffffu, hi & 0x00ff00ffu);
+        const uint32_t d = __reduce_add_sync(0xffffffffu, (hi >> 8) & 0x00ff00ffu);
+        const uint32_t w = lane & 4 ? (lane & 1 ? d : c) : (lane & 1 ? b : a);
+        const int n = (int)(lane & 2 ? w >> 16 : w & 0xffffu);
+        if (lane < 8 && n) atomicAdd(&s_hist[lane], n);
+        r8 = 0;
+        since = 0;
+    }
+};
+}  // namespace kh
+#endif
 
 namespace kh {
 struct Graph {
@@ -250,6 +323,8 @@ struct Graph {
     int64_t *rowptr;
     int32_t *col;
     uint8_t *rank;
+    uint8_t *crank;         // rank of each column entry (fixed-level counts)
+    bool crank_valid;
     uint8_t *alive;
     uint32_t *keys;
     int64_t keys_levels;    // allocated levels in keys

@@ -214,18 +214,6 @@ __device__ __forceinline__ unsigned long long level1_bytes(int64_t deg, int S, i
     return 8ull + 5ull * (unsigned long long)deg + (last ? 8ull : 4ull * (unsigned long long)S) + 5ull;
 }
 
-// Lane j adds #{lanes : r >= j} to its count (r = -1: no key).  Ranks are
-// geometric, so a warp's 32 keys need about 7 ballots (no shared-memory
-// atomics: half the keys of a histogram would fall on one address).
-__device__ __forceinline__ void add_rank_counts(int r, int lane, int& S) {
-#pragma unroll 1
-    for (int j = 0; j < 32; ++j) {
-        const uint32_t b = __ballot_sync(kFull, r >= j);
-        if (!b) break;
-        if (lane == j) S += __popc(b);
-    }
-}
-
 // kappa, the list size at kappa and the highest rank present from the counts
 // S_j held by lane j.
 __device__ __forceinline__ void level_of_counts(int S, int M, int& kappa, int& Skap, int& top) {

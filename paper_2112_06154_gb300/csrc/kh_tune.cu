@@ -3,8 +3,9 @@
 //
 // Three kernels compute deg_2 of every node (Sec. 2) with different visited-set
 // layouts:
-//   KH_VAR_CTA     k_hdeg: one CTA per source, a visited bitmap of all n nodes
-//                  in shared memory (only while n bits fit), cleared per source;
+//   KH_VAR_CTA     k_hdeg2_cta: one CTA per source, a visited bitmap of all n
+//                  nodes in shared memory (only while n bits fit), cleared per
+//                  source;
 //   KH_VAR_SLICED  k_hdeg2_slice: (source, slice) items, a bitmap of one slice
 //                  of the id range, cleared through the words the item set;
 //   KH_VAR_SLICED_SMALL  the same for sources of large 2-hop work, and
@@ -26,6 +27,7 @@
 // every candidate computes the same degrees.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -125,21 +127,62 @@ __global__ void k_stride_sample(const int32_t* __restrict__ order, int64_t nsrc,
     if (blockIdx.x == 0 && threadIdx.x == 0) *count = (int)m;
 }
 
-// The sliced layout over `order` (nsrc sources, the first nbig of them too
-// large for the warp-per-source kernel): KH_VAR_SLICED_SMALL hands the rest
-// to that kernel.
-int run_sliced(Graph& g, const TuneChoice& c, int32_t* deg, int32_t* cnt, int jlo, int nj,
-               cudaStream_t s, const int32_t* order, int64_t nsrc, int64_t nbig) {
+// Where the work classes end in a longest-first list of sources: too large for a
+// warp (KH_VAR_SLICED_SMALL); a CTA, a large CTA each (KH_VAR_CTA).
+struct Split {
+    int64_t big, cta, large;
+    // the split of every `stride`-th source, of the list without its first `k`
+    Split sample(int64_t stride) const {
+        auto f = [&](int64_t x) { return (x + stride - 1) / stride; };
+        return {f(big), f(cta), f(large)};
+    }
+    Split drop(int64_t k) const {
+        auto f = [&](int64_t x) { return x > k ? x - k : 0; };
+        return {f(big), f(cta), f(large)};
+    }
+};
+
+Split work_split(const Graph& g) {
+    return {hdeg2_small_split(g), hdeg2_sources_from_bin(g, kCtaSmallBin),
+            hdeg2_sources_from_bin(g, hdeg2_large_bin(g))};
+}
+
+// A layout over `order` (nsrc sources, longest first).
+int run_layout(Graph& g, const TuneChoice& c, int32_t* deg, int32_t* cnt, int jlo, int nj,
+               cudaStream_t s, const int32_t* order, int64_t nsrc, const Split& split) {
+    if (c.variant == KH_VAR_CTA) {
+        // a large CTA for each of the sources of largest work, a warp for each of
+        // the small ones, a CTA as small as the bitmap allows for the rest
+        int rc = cnt ? ensure_crank(g, s) : KH_OK;
+        if (rc) return rc;
+        if ((rc = launch_init2(g, deg, cnt, jlo, nj, s))) return rc;
+        if (split.large > 0) {
+            // beside the others: alone, the few large sources leave most SMs idle
+            // (Chung-Lu n = 200k: 1.70 -> 1.9 ms in line)
+            KH_CUDA_TRY(g.ctx, cudaEventRecord(g.ctx->fork, s));
+            KH_CUDA_TRY(g.ctx, cudaStreamWaitEvent(g.ctx->side, g.ctx->fork, 0));
+            rc = launch_hdeg2_cta(g, deg, cnt, jlo, nj, g.ctx->side, order, split.large, true);
+            KH_CUDA_TRY(g.ctx, cudaEventRecord(g.ctx->join, g.ctx->side));
+            if (rc) {
+                cudaStreamWaitEvent(s, g.ctx->join, 0);
+                return rc;
+            }
+        }
+        rc = launch_hdeg2_cta(g, deg, cnt, jlo, nj, s, order + split.large, split.cta - split.large, false);
+        if (split.large > 0) KH_CUDA_TRY(g.ctx, cudaStreamWaitEvent(s, g.ctx->join, 0));
+        if (rc) return rc;
+        return launch_hdeg2_small(g, deg, cnt, jlo, nj, s, order + split.cta, nsrc - split.cta);
+    }
     if (c.variant != KH_VAR_SLICED_SMALL)
         return launch_hdeg2_slice(g, deg, cnt, jlo, nj, s, c.slices, c.threads, order, nsrc, true);
-    int rc = launch_hdeg2_slice(g, deg, cnt, jlo, nj, s, c.slices, c.threads, order, nbig, true);
+    int rc = launch_hdeg2_slice(g, deg, cnt, jlo, nj, s, c.slices, c.threads, order, split.big, true);
     if (rc) return rc;
-    return launch_hdeg2_small(g, deg, cnt, jlo, nj, s, order + nbig, nsrc - nbig);
+    return launch_hdeg2_small(g, deg, cnt, jlo, nj, s, order + split.big, nsrc - split.big);
 }
 
 // One candidate on the sample; returns its event time in ms (negative: failed).
-double time_candidate(Graph& g, const TuneChoice& c, const int32_t* sample, const int* d_count,
-                      int64_t m, int32_t* scratch, cudaStream_t s, int64_t sample_big) {
+double time_candidate(Graph& g, const TuneChoice& c, const int32_t* sample, int64_t m,
+                      int32_t* scratch, cudaStream_t s, const Split& split, int reps = 2) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
         cudaGetLastError();
@@ -147,13 +190,9 @@ double time_candidate(Graph& g, const TuneChoice& c, const int32_t* sample, cons
         return -1.0;
     }
     double best = -1.0;
-    for (int rep = 0; rep < 2; ++rep) {  // the first run warms caches and loads the module
+    for (int rep = 0; rep < reps; ++rep) {  // the first run warms caches and loads the module
         cudaEventRecord(e0, s);
-        int rc;
-        if (c.variant == KH_VAR_CTA)
-            rc = launch_hdeg(g, sample, d_count, 0, scratch, nullptr, 0, 0, s);
-        else
-            rc = run_sliced(g, c, scratch, nullptr, 0, 0, s, sample, m, sample_big);
+        const int rc = run_layout(g, c, scratch, nullptr, 0, 0, s, sample, m, split);
         cudaEventRecord(e1, s);
         if (rc != KH_OK || cudaEventSynchronize(e1) != cudaSuccess) {
             cudaGetLastError();
@@ -206,6 +245,7 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
         if (si > 0 && slist[si] == slist[si - 1]) continue;
         if (slist[si] > 64) continue;
         for (int t : {256, 512, 1024}) {
+            if (t == 512 && cta_fits(g)) continue;
             cand.push_back({KH_VAR_SLICED, slist[si], t, 0.0});
             cand.push_back({KH_VAR_SLICED_SMALL, slist[si], t, 0.0});
         }
@@ -213,9 +253,7 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
     // sample: every stride-th source of the longest-first order
     const int64_t stride = g.nsrc2 > 65536 ? 32 : 1;
     const int64_t m = (g.nsrc2 + stride - 1) / stride;
-    // the stride sample keeps order2's order: its first sample_big sources are big
-    const int64_t big = hdeg2_small_split(g);
-    const int64_t sample_big = (big + stride - 1) / stride;
+    const Split split = work_split(g), sample_split = split.sample(stride);
     int32_t* sample = g.listB;   // scratch (ensure_work holds n entries)
     int32_t* scratch = g.listA;
     int* d_count = &g.state->tune_count;
@@ -226,13 +264,26 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.alive, 1, (size_t)g.n, s));
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.deadbm, 0, ((size_t)(g.n + 127) / 128) * 16, s));
     const int64_t launches_before = g.launches;
-    TuneChoice best{};
-    best.ms = 1e30;
+    TuneChoice best{}, cta{};
+    best.ms = cta.ms = 1e30;
     for (TuneChoice& t : cand) {
         if (m == 0) break;
-        const double ms = time_candidate(g, t, sample, d_count, m, scratch, s, sample_big);
+        const double ms = time_candidate(g, t, sample, m, scratch, s, sample_split);
         t.ms = ms;
+        if (ms >= 0.0 && t.variant == KH_VAR_CTA) cta = t;
         if (ms >= 0.0 && ms < best.ms) best = t;
+    }
+    // A short pass is ranked by itself where one CTA per source is possible: on a
+    // sample the search of the largest sources by one CTA is most of the time, in
+    // the whole pass it is hidden (2-degrees of Chung-Lu n = 200k: the sample put
+    // the sliced layout first, which then took twice as long).
+    const double predicted = best.ms * (double)stride;
+    if (cta.variant == KH_VAR_CTA && best.variant != KH_VAR_AUTO && best.variant != KH_VAR_CTA &&
+        predicted < 100.0) {
+        const double full_cta = time_candidate(g, cta, g.order2, g.nsrc2, scratch, s, split, 1);
+        if (full_cta >= 0.0 && (full_cta < 0.5 * predicted ||
+                                full_cta < time_candidate(g, best, g.order2, g.nsrc2, scratch, s, split, 1)))
+            best = cta;
     }
     if (best.variant == KH_VAR_AUTO) {
         // nothing measured (no sources): any valid layout does
@@ -249,7 +300,7 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
     // (only where the whole pass takes 20 ms or more, and only for a predicted
     // gain of 5%: on small graphs the sample times are too short to rank them)
     best.sweep_bin = 0;
-    if (best.variant != KH_VAR_CTA && m > 0 && hdeg2_sources_from_bin(g, kSweepMinBin) > 0 &&
+    if (m > 0 && hdeg2_sources_from_bin(g, kSweepMinBin) > 0 &&
         best.ms * (double)stride >= 20.0) {
         auto time_sweep = [&](int64_t first, int64_t nb) -> double {
             cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -289,8 +340,8 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
             const double t_mid = time_sweep(mid + nb_mid <= nsw ? mid : nsw - nb_mid, nb_mid);
             if (t_mid < 0.0) break;
             TuneChoice rest = best;
-            const double t_rest = time_candidate(g, rest, sample + sbig, d_count, m - sbig, scratch, s,
-                                                 sample_big > sbig ? sample_big - sbig : 0);
+            const double t_rest = time_candidate(g, rest, sample + sbig, m - sbig, scratch, s,
+                                                 sample_split.drop(sbig));
             if (t_rest < 0.0) break;
             const double t = (double)((nsw + kSweepBatch - 1) / kSweepBatch) * t_mid + t_rest * (double)stride;
             if (t < t_best) {
@@ -307,15 +358,21 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
 }
 
 // h >= 3: bit-parallel batches or a search per source, decided once per graph
-// and h.  The searches' cost per source comes from a probe of a few sources
-// spread over the longest-first order (the device byte counter: 4 bytes a row
-// entry); the batches' cost is known: h - 1 pulls over all rows per 1024 sources.
-// A pull entry (a 128-byte gather, from L2 or, once the masks outgrow it, from
-// HBM) costs about kPullCost search entries (a 4-byte read and a bitmap test):
-// measured 16 ps against 2 ps on Chung-Lu n = 200k.
+// and h.  The searches' cost per source comes from a probe of every n/152-th node
+// (the device byte counter: 4 bytes a row entry); the batches' cost is known: h - 1
+// pulls over all rows per 1024 sources.  A pull entry (a 128-byte gather, from L2
+// or, once the masks outgrow it, from HBM) costs about kPullCost search entries (a
+// 4-byte read and a bitmap test): measured 16 ps against 2 ps on Chung-Lu n = 200k.
 constexpr int kProbe = 152;
 constexpr double kPullCost = 8.0;
 constexpr double kBatchOverhead = 1.0e7;  // a batch's launches, in search entries
+constexpr double kProbeMin = 1.0e8;       // below this many entries a probe costs more than it saves
+
+__global__ void k_stride_ids(int64_t n, int64_t stride, int32_t* __restrict__ out, int* count) {
+    const int64_t m = (n + stride - 1) / stride;
+    for (int64_t i = threadIdx.x; i < m; i += blockDim.x) out[i] = (int32_t)(i * stride);
+    if (threadIdx.x == 0) *count = (int)m;
+}
 
 static int choose_deep(Graph& g, cudaStream_t s, bool* batches) {
     *batches = false;
@@ -325,54 +382,57 @@ static int choose_deep(Graph& g, cudaStream_t s, bool* batches) {
                ((double)(g.h - 1) * (double)(g.nnz + g.n) * kPullCost + kBatchOverhead);
     };
     // a search reads at most every row entry: no probe where even that is less
-    if ((double)g.n * (double)g.nnz <= pulls((double)g.n)) return KH_OK;
+    const double most = (double)g.n * (double)g.nnz;
+    if (most <= kProbeMin || most <= pulls((double)g.n)) return KH_OK;
+    int rc;
     if (g.hdeg_deep[g.h] == 0) {
-        int rc = ensure_order2(g, s);
-        if (rc) return rc;
-        const int64_t stride = (g.nsrc2 + kProbe - 1) / kProbe;
-        const int64_t m = (g.nsrc2 + stride - 1) / stride;
+        const int64_t stride = (g.n + kProbe - 1) / kProbe;
+        const int64_t m = (g.n + stride - 1) / stride;
         const int64_t launches_before = g.launches;
-        k_stride_sample<<<1, 256, 0, s>>>(g.order2, g.nsrc2, stride, g.listB, &g.state->tune_count);
-        unsigned long long b0 = 0, b1 = 0;
-        unsigned long long* ctr = &g.state->bytes[kProfBfs];
-        unsigned long long upd = 0;
-        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&b0, ctr, sizeof(b0), cudaMemcpyDeviceToHost, s));
-        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&upd, &g.state->updates, sizeof(upd), cudaMemcpyDeviceToHost, s));
+        // the probe is not the caller's work: its counters are put back
+        struct {
+            unsigned long long updates, bytes[kProfKinds];
+        } before, after;
+        static_assert(offsetof(DevState, bytes) == offsetof(DevState, updates) + sizeof(unsigned long long),
+                      "the counters are copied as one block");
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&before, &g.state->updates, sizeof(before), cudaMemcpyDeviceToHost, s));
+        k_stride_ids<<<1, 256, 0, s>>>(g.n, stride, g.listB, &g.state->tune_count);
         const bool prof = g.prof_on;
-        g.prof_on = false;  // the probe is not the caller's work
+        g.prof_on = false;
         rc = launch_hdeg(g, g.listB, &g.state->tune_count, 0, g.listA, nullptr, 0, 0, s);
         g.prof_on = prof;
         if (rc) return rc;
-        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&b1, ctr, sizeof(b1), cudaMemcpyDeviceToHost, s));
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&after, &g.state->updates, sizeof(after), cudaMemcpyDeviceToHost, s));
         KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
-        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(ctr, &b0, sizeof(b0), cudaMemcpyHostToDevice, s));
-        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&g.state->updates, &upd, sizeof(upd), cudaMemcpyHostToDevice, s));
-        KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));  // b0 and upd are host locals
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&g.state->updates, &before, sizeof(before), cudaMemcpyHostToDevice, s));
+        KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));  // `before` is a host local
         g.launches = launches_before;
-        const double search = (double)(b1 - b0) / 4.0 / (double)m * (double)g.nsrc2;
-        g.hdeg_deep[g.h] = search > pulls((double)g.nsrc2) ? 2 : 1;
+        const double per = (double)(after.bytes[kProfBfs] - before.bytes[kProfBfs]) / 4.0 / (double)m;
+        g.hdeg_deep[g.h] = per * (double)g.n > pulls((double)g.n) ? 2 : 1;
     }
-    // (without memory for the masks: a search per source)
-    *batches = g.hdeg_deep[g.h] == 2 && ensure_sweep(g, g.h, s) == KH_OK;
+    if (g.hdeg_deep[g.h] != 2) return KH_OK;
+    if ((rc = ensure_order2(g, s))) return rc;
+    *batches = ensure_sweep(g, g.h, s) == KH_OK;  // (no memory for the masks: a search per source)
     return KH_OK;
 }
 
 int run_hdeg_full(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s) {
     if (g.h == 2 && !g.gid && g.n > 0) {
-        TuneChoice c{};
-        int rc = choose_hdeg2(g, s, &c);
+        // the counts take one CTA per source where its bitmap fits (counts of R-MAT
+        // 18 / 19: 16.6 / 44 ms against 34 / 78 with the layout tuned for degrees)
+        TuneChoice c{KH_VAR_CTA, 0, 256, 0.0, 0};
+        int rc = KH_OK;
+        if (!cnt || !cta_fits(g) || g.force_hdeg2.variant != KH_VAR_AUTO) rc = choose_hdeg2(g, s, &c);
         if (rc) return rc;
-        if (c.variant == KH_VAR_SLICED || c.variant == KH_VAR_SLICED_SMALL) {
+        {
             rc = ensure_order2(g, s);
             if (rc) return rc;
             // the sources of largest 2-hop work go to the bit-parallel sweeps
-            // (2-degrees only: the fixed-level counts stay with the sliced kernel)
+            // (2-degrees only: the sweeps do not count by rank)
             int bin = g.sw_force != 0 ? g.sw_force : c.sweep_bin;
             if (cnt || bin < 0) bin = 0;
             int64_t nsw = bin > 0 && ensure_sweep(g, 2, s) == KH_OK ? hdeg2_sources_from_bin(g, bin) : 0;
-            const int64_t big = hdeg2_small_split(g);
-            rc = run_sliced(g, c, deg, cnt, jlo, nj, s, g.order2 + nsw, g.nsrc2 - nsw,
-                            big > nsw ? big - nsw : 0);
+            rc = run_layout(g, c, deg, cnt, jlo, nj, s, g.order2 + nsw, g.nsrc2 - nsw, work_split(g).drop(nsw));
             if (rc || nsw == 0) return rc;
             return run_sweeps(g, deg, g.order2, nsw, 2, s);
         }
