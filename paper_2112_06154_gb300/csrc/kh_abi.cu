@@ -365,6 +365,14 @@ static int finish_check(Graph& g) {
     return KH_OK;
 }
 
+static void free_ctx_objects(kh_ctx* c) {
+    for (cudaEvent_t ev : {c->fork, c->join, c->peel_done[0], c->peel_done[1]})
+        if (ev) cudaEventDestroy(ev);
+    if (c->side) cudaStreamDestroy(c->side);
+    if (c->own_stream) cudaStreamDestroy(c->stream);
+    if (c->peel_state) cudaFreeHost(c->peel_state);
+}
+
 }  // namespace kh
 
 using kh::Graph;
@@ -389,12 +397,11 @@ int kh_ctx_create(kh_ctx** out, int device, void* cuda_stream) {
         }
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming);
+    for (cudaEvent_t* ev : {&c->fork, &c->join, &c->peel_done[0], &c->peel_done[1]})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaMallocHost(&c->peel_state, 2 * sizeof(kh::DevState));
     if (e != cudaSuccess) {
-        if (c->fork) cudaEventDestroy(c->fork);
-        if (c->side) cudaStreamDestroy(c->side);
-        if (c->own_stream) cudaStreamDestroy(c->stream);
+        kh::free_ctx_objects(c);
         free(c);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? KH_ENOMEM : KH_ECUDA;
@@ -406,10 +413,7 @@ int kh_ctx_create(kh_ctx** out, int device, void* cuda_stream) {
 int kh_ctx_destroy(kh_ctx* ctx) {
     if (!ctx) return KH_EINVAL;
     cudaSetDevice(ctx->device);
-    cudaEventDestroy(ctx->fork);
-    cudaEventDestroy(ctx->join);
-    cudaStreamDestroy(ctx->side);
-    if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
+    kh::free_ctx_objects(ctx);
     free(ctx);
     return KH_OK;
 }

@@ -105,7 +105,6 @@ struct BfsArgs {
     int* err;
     unsigned long long* updates;
     unsigned long long* bytes;  // algorithmic bytes: 8 + 4 deg per expanded vertex, 4 per result
-    const int* skip;            // nonzero: the exact early stop fired, nothing to do
     const uint32_t* deadbm;     // removed-node bitmap (shared-memory mode): seeds the visited set
     // batches: graph of each node, first node of each graph, per-node h; the
     // visited bitmap is indexed by the id inside the source's graph
@@ -228,8 +227,10 @@ __global__ void __launch_bounds__(kBfsThreads) k_hdeg(BfsArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     uint32_t* bm = SMEM ? s_bm_dyn : a.gbitmaps + (size_t)blockIdx.x * (size_t)a.words;
     int32_t* q = a.queues + (size_t)blockIdx.x * (size_t)a.qcap;
-    const int64_t total = (a.skip && *a.skip) ? 0 : (a.worklist ? (int64_t)(*a.d_count) : a.count_static);
-    if (total == 0) return;
+    const int64_t total = a.worklist ? (int64_t)(*a.d_count) : a.count_static;
+    // the first source of each block goes by its index: with a short list the other
+    // blocks touch nothing
+    if (blockIdx.x >= total) return;
     unsigned long long my_bytes = 0;
 
     const bool seeded = SMEM && a.deadbm != nullptr && a.gid == nullptr;
@@ -238,8 +239,8 @@ __global__ void __launch_bounds__(kBfsThreads) k_hdeg(BfsArgs a) {
         __syncthreads();
     }
 
-    for (;;) {
-        if (tid == 0) s_src = atomicAdd(a.work_ctr, 1);
+    for (bool first = true;; first = false) {
+        if (tid == 0) s_src = first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(a.work_ctr, 1);
         __syncthreads();
         const int64_t idx = s_src;
         if (idx >= total) break;
@@ -451,8 +452,8 @@ __global__ void k_ball_hop(const int64_t* __restrict__ rowptr, const int32_t* __
                            int32_t* __restrict__ fout, int* nfout, int32_t* __restrict__ wl, int* nwl,
                            const DevState* __restrict__ st, int h_all, int64_t cap,
                            unsigned long long* bytes, int32_t* __restrict__ degX,
-                           const uint8_t* __restrict__ hv, int hop) {
-    if (st->early) return;
+                           const uint8_t* __restrict__ hv, int hop, RoundEnd end) {
+    if (blockIdx.x == 0) end_round(end);
     __shared__ int s_heavy[kBlockHeavyX];
     __shared__ int s_nheavy;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -505,10 +506,8 @@ __global__ void k_stale_exact(const int64_t* __restrict__ rowptr, const int32_t*
                               const uint8_t* __restrict__ alive, const int32_t* __restrict__ degX,
                               const int32_t* __restrict__ list, const int* __restrict__ nlist,
                               int64_t n, uint8_t* __restrict__ fresh,
-                              unsigned long long* __restrict__ lb, const DevState* __restrict__ st,
-                              unsigned long long* bytes, int h_all, const uint8_t* __restrict__ hv,
+                              unsigned long long* __restrict__ lb, unsigned long long* bytes, int h_all, const uint8_t* __restrict__ hv,
                               const int32_t* __restrict__ bestnb) {
-    if (st->early) return;
     __shared__ int s_max[kBfsThreads / 32];
     __shared__ int s_heavy[kBlockHeavyX];
     __shared__ int s_nheavy;
@@ -587,7 +586,6 @@ __global__ void k_apply_loss(const int32_t* __restrict__ list, const int* __rest
                              int32_t* __restrict__ loss, int32_t* __restrict__ d,
                              const uint8_t* __restrict__ fresh, unsigned long long* __restrict__ lb,
                              DevState* __restrict__ st, int64_t cap) {
-    if (st->early) return;
     const int cnt = (int)min((int64_t)*nlist, cap);
     if (blockIdx.x == 0 && threadIdx.x == 0 && cnt > 0) {
         atomicAdd(&st->updates, (unsigned long long)cnt);
@@ -708,7 +706,6 @@ int launch_hdeg(Graph& g, const int* worklist, const int* d_count, int64_t count
     a.err = &g.state->err;
     a.updates = &g.state->updates;
     a.bytes = &g.state->bytes[kProfBfs];
-    a.skip = worklist ? &g.state->early : nullptr;
     a.deadbm = g.deadbm;
     a.gid = g.gid;
     a.vtx_off = g.vtx_off;
@@ -749,7 +746,7 @@ void launch_ball_hop(Graph& g, int hop, cudaStream_t s) {
     k_ball_hop<<<grid, 256, 0, s>>>(g.rowptr, g.col, g.alive, g.seen, fin, nfin, fout, nfout,
                                     g.listW, &g.state->rc[kRcW], g.state, g.h, g.n,
                                     &g.state->bytes[kProfFrontier], hop == 1 ? g.degX : nullptr,
-                                    g.hv, hop);
+                                    g.hv, hop, hop == 1 ? round_end(g) : RoundEnd{});
     count_launch(g, 1);
     prof_end(g, kProfFrontier, s);
 }
@@ -768,8 +765,8 @@ void launch_stale_exact(Graph& g, const int* list, const int* d_count, cudaStrea
     const int grid = g.ctx->sm_count * 8;
     prof_begin(g, kProfFrontier, s);
     k_stale_exact<<<grid, kBfsThreads, 0, s>>>(g.rowptr, g.col, g.alive, g.degX, list, d_count, g.n,
-                                       g.fresh, g.lb64, g.state, &g.state->bytes[kProfFrontier],
-                                       g.h, g.hv, g.bestnb);
+                                       g.fresh, g.lb64, &g.state->bytes[kProfFrontier], g.h, g.hv,
+                                       g.bestnb);
     count_launch(g, 1);
     prof_end(g, kProfFrontier, s);
 }

@@ -66,9 +66,8 @@ constexpr int kProfFrontier = 3;  // removed-set ball hops, neighbour marking
 constexpr int kProfPeel = 4;      // min, select, finish, advance
 constexpr int kProfKinds = 5;
 
-// Per-round counters: every launch inside a peeling round has its own slot,
-// and the last block of the round's final kernel zeroes them all, so a round
-// needs no memset nodes.
+// Per-round counters: every launch inside a peeling round has its own slot, and
+// the next round's first kernel zeroes them all, so a round needs no memset nodes.
 constexpr int kRcBfs = 0;          // refine BFS work counter
 constexpr int kRcRefineWork = 1;   // refine last-level list work counter
 constexpr int kRcLevelWork = 3;    // + i: refresh level i work counter, i = 1..kMaxH
@@ -93,11 +92,9 @@ struct DevState {
     unsigned long long updates;  // node recomputations
     unsigned long long bytes[kProfKinds];  // algorithmic bytes per kernel class
     int err;                     // kErr* bits
-    int early;                   // exact early stop taken this round
     int nQ;                      // refine list size (stale nodes due this round)
     unsigned long long minU;     // min of the upper bounds d over alive nodes
     int rc[kRcCount];            // per-round counters (kRc*)
-    int done;                    // blocks of the round's final kernel that finished
     // peel work statistics: list recomputations and changes per level in the
     // rounds' refresh passes, refines stopped early
     unsigned long long lvl_work[kMaxH + 1];
@@ -108,6 +105,27 @@ struct DevState {
 };
 
 struct Graph;
+
+// After a round's removal set is chosen: c = max(c, the round's minimum) of every
+// graph, the minima back to none.  Done by one block of the first refresh kernel
+// (nothing else reads them before the next round).
+struct RoundEnd {
+    unsigned long long *c, *mn, *mr, *mu;  // c nullptr: nothing to do
+    int64_t ngraphs;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ void end_round(const RoundEnd& r) {
+    if (!r.c) return;
+    for (int64_t q = threadIdx.x; q < r.ngraphs; q += blockDim.x) {
+        const unsigned long long m = r.mn[q] < r.mr[q] ? r.mn[q] : r.mr[q];
+        if (m != ~0ull && m > r.c[q]) r.c[q] = m;
+        r.mn[q] = ~0ull;
+        r.mr[q] = ~0ull;
+        r.mu[q] = ~0ull;
+    }
+}
+#endif
+RoundEnd round_end(const Graph& g);
 
 // The lazy refine decides whether d(v) <= T = max(c, U) and may stop once a
 // partial value (a lower bound of d(v)) exceeds it.  It runs on until the
@@ -213,16 +231,16 @@ int hdeg2_min_slices(int64_t n);
 int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
                  int64_t count_static, int track, cudaStream_t s, int round_mode = 0,
                  int skip_last = -1);
-// alive neighbours of the nodes in list1 and list2 (may be nullptr) join the
-// work list listW (count *out_count), deduplicated by stamp phase
-// A(list1) and the part of A(list2) whose level `phase` can have changed
-// (rank filter on rho) join the work list.
+// A(list1) and the part of A(list2) (may be nullptr) whose level `phase` can have
+// changed (rank filter on rho), deduplicated by stamp phase: nodes whose last
+// level it is become stale, the others join the work list listW (count
+// *out_count).  Phase 1 also ends the round's selection (end_round).
 void launch_mark_neighbours(Graph& g, const int* list1, const int* cnt1, const int* list2,
                             const int* cnt2, int phase, int* out_count, cudaStream_t s);
-// sampled mode: mark the nodes of `list` (nullptr: all) stale at the last
-// level with a lower bound of their estimate
-void launch_stale_sampled(Graph& g, const int* list, const int* d_count, cudaStream_t s,
-                          int only_h = 0);
+// start of a sampled peel: every alive node stale with a lower bound
+void launch_stale_all(Graph& g, cudaStream_t s);
+// start of a peel: meta words of no lists, alive nodes stale at their last level
+int launch_init_meta(Graph& g, cudaStream_t s);
 // each node's last-level k and |B| into device arrays (either may be nullptr)
 void launch_gather_last(Graph& g, uint8_t* lvl_out, int32_t* bs_out, cudaStream_t s);
 
@@ -246,6 +264,8 @@ struct kh_ctx {
     // `stream` by the two events)
     cudaStream_t side;
     cudaEvent_t fork, join;
+    void* peel_state;          // pinned: the device state after the last two replays of a peel
+    cudaEvent_t peel_done[2];
     // fault injection on the host: the fail_alloc_at-th device allocation from
     // the arming call fails with KH_ENOMEM (0: off)
     int64_t fail_alloc_at;

@@ -1,7 +1,7 @@
 // kh_peel.cu -- bucket-synchronous peeling (ExactCore of Sec. 2; Core, Alg. 4).
 //
 // Round r on the alive set X (all device-resident):
-//   1. minval = min_{v in X} d[v]                         (k_min_alive)
+//   1. minval = min_{v in X} d[v]                         (k_begin)
 //   2. c = max(c, minval); R = {v in X : d[v] <= c};
 //      core[v] = c, alive[v] = 2 for v in R               (k_select)
 //   3. refresh d on X \ R where it can have changed:
@@ -9,7 +9,7 @@
 //               then a bounded BFS per such node;
 //      sampled: level i = 1..h recomputes the alive neighbours of R and of the
 //               nodes whose (|B|, k) changed at level i-1 (Alg. 3).
-//   4. alive[R] = 0; the last block advances the state          (k_finish)
+//   4. alive[R] = 0 and the next round's minimum                 (k_begin)
 // Removing every node with d <= c at once gives the same core map as Alg. 4's
 // one-at-a-time loop because d(v; X) never grows as X shrinks (deg_h by
 // inclusion of neighbourhoods; the estimate by Prop. 4.2): every node of R
@@ -17,7 +17,16 @@
 //
 // Exact mode applies the paper's early stop (Sec. 5): once c >= |X| - 1 every
 // remaining node has deg_h <= |X| - 1 <= c, so all get core c in the next
-// round; the refresh of this round is then skipped.
+// round (k_begin).
+//
+// A round of a small graph, or of a late peel, is a chain of kernels with little
+// work each: about 4 us per kernel in the replayed graph.  So the phases that
+// need no grid-wide result of each other share a kernel: the end of a round and
+// the next one's minima (k_begin), the state's advance and the refine list
+// (k_collect), marking and the stale bounds (k_mark_nbrs).  7 kernels a round at
+// h = 2 (9 before), 8 exact (10 before): the (k,2)-core of Chung-Lu n = 50k 122 ->
+// 74 us a round (with the marking spread over all warps), exact 77 -> 69 us, the
+// (k,3)-core of R-MAT 18 142 -> 109 us.
 //
 // Lazy last level.  A node whose h-neighbourhood may have changed is only
 // marked stale: its last value stays as an upper bound (d never grows as X
@@ -88,34 +97,85 @@ __device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigne
     return a < b ? a : b;
 }
 
-// Round start: the minimum of d over the alive nodes into mu[graph] and over
-// the fresh ones into mn[graph].  A single graph reduces per block; a batch
-// takes one atomic per node that improves its graph's current minimum (read
-// first, so most nodes need none).
+// Sec. 5: with c >= |X| - 1 every remaining node has deg_h <= |X| - 1 <= c.
+__device__ __forceinline__ bool early_stop(unsigned long long c, int left) {
+    return left > 0 && c + 1 >= (unsigned long long)left;
+}
+
+// Round start.  The previous round ends: its removed nodes leave (alive = 0, dead
+// bitmap bit set), the per-round counters go back to zero, and, in exact peels,
+// the nodes of a graph with c >= |X| - 1 get core c in the round after that one
+// (the paper's early stop, Sec. 5: every remaining deg_h <= |X| - 1 <= c).  Then,
+// unless the removal order is given, the minimum of d over the alive nodes into
+// mu[graph] and over the fresh ones into mn[graph]: a single graph reduces per
+// block; a batch takes one atomic per node that improves its graph's current
+// minimum (read first, so most nodes need none).
+struct BeginArgs {
+    uint8_t* alive;
+    const uint8_t* fresh;
+    int64_t n;
+    const int32_t* vl;
+    DevState* st;
+    PeelState p;
+    const int32_t* R;
+    uint32_t* deadbm;
+    int32_t* core;      // exact: the early stop writes here (nullptr: none)
+    int32_t* round_of;
+    int want_min;
+};
+
 template <typename T>
-__global__ void k_min_alive(const uint8_t* __restrict__ alive, const uint8_t* __restrict__ fresh,
-                            const T* __restrict__ d, int64_t n, const int32_t* __restrict__ vl,
-                            DevState* st, unsigned long long* mu, unsigned long long* mn,
-                            const int32_t* __restrict__ gid) {
-    if (st->n_alive == 0) return;
-    unsigned long long m = ~0ull, mf = ~0ull;
+__global__ void k_begin(BeginArgs a, const T* __restrict__ d) {
+    DevState* st = a.st;
+    if (blockIdx.x == 0) {
+        for (int i = threadIdx.x; i < kRcCount; i += blockDim.x) st->rc[i] = 0;
+        if (threadIdx.x == 0) st->nQ = 0;
+    }
+    if (st->n_alive == 0) return;  // the peel is over
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int64_t v = vl ? vl[i] : i;
-        if (alive[v] == 1) {
-            const unsigned long long x = (unsigned long long)d[v];
-            const bool fr = fresh[v] != 0;
-            if (gid) {
-                const int g = gid[v];
-                if (x < *(volatile unsigned long long*)(mu + g)) atomicMin(mu + g, x);
-                if (fr && x < *(volatile unsigned long long*)(mn + g)) atomicMin(mn + g, x);
-            } else {
-                m = umin(m, x);
-                if (fr) mf = umin(mf, x);
-            }
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int nR = st->nR;
+    for (int64_t i = first; i < nR; i += stride) {
+        const int v = a.R[i];
+        a.alive[v] = 0;
+        atomicOr(a.deadbm + (v >> 5), 1u << (v & 31));
+    }
+    const int round = st->round;
+    const bool stop = a.core && round >= 0;
+    const bool one = stop && !a.p.gid && early_stop(a.p.c[0], st->n_alive_next);
+    if (!a.want_min && !stop) return;
+    unsigned long long m = ~0ull, mf = ~0ull;
+    int gone = 0;
+    for (int64_t i = first; i < a.n; i += stride) {
+        const int64_t v = a.vl ? a.vl[i] : i;
+        if (a.alive[v] != 1) continue;
+        const int g = graph_of(a.p, v);
+        if (one || (stop && a.p.gid && early_stop(a.p.c[g], a.p.left[g]))) {
+            a.core[v] = (int32_t)a.p.c[g];
+            a.round_of[v] = round + 1;
+            a.alive[v] = 0;
+            ++gone;
+            continue;
+        }
+        if (!a.want_min) continue;
+        const unsigned long long x = (unsigned long long)d[v];
+        const bool fr = a.fresh[v] != 0;
+        if (a.p.gid) {
+            if (x < *(volatile unsigned long long*)(a.p.mu + g)) atomicMin(a.p.mu + g, x);
+            if (fr && x < *(volatile unsigned long long*)(a.p.mn + g)) atomicMin(a.p.mn + g, x);
+        } else {
+            m = umin(m, x);
+            if (fr) mf = umin(mf, x);
         }
     }
-    if (gid) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        atomicAdd(&st->bytes[kProfPeel], (unsigned long long)a.n * (2 + sizeof(T)));
+    if (a.p.gid) {
+        // (a single graph's early stop is seen by the next kernel from c and the count)
+        for (int off = 16; off > 0; off >>= 1) gone += __shfl_down_sync(kFull, gone, off);
+        if ((threadIdx.x & 31) == 0 && gone) atomicSub(&st->n_alive_next, gone);
+        return;
+    }
     for (int off = 16; off > 0; off >>= 1) {
         m = umin(m, __shfl_down_sync(kFull, m, off));
         mf = umin(mf, __shfl_down_sync(kFull, mf, off));
@@ -132,9 +192,8 @@ __global__ void k_min_alive(const uint8_t* __restrict__ alive, const uint8_t* __
             m = umin(m, s_m[w]);
             mf = umin(mf, s_f[w]);
         }
-        if (m != ~0ull) atomicMin(mu, m);
-        if (mf != ~0ull) atomicMin(mn, mf);
-        if (blockIdx.x == 0) atomicAdd(&st->bytes[kProfPeel], (unsigned long long)n * (2 + sizeof(T)));
+        if (m != ~0ull) atomicMin(a.p.mu, m);
+        if (mf != ~0ull) atomicMin(a.p.mn, mf);
     }
 }
 
@@ -174,11 +233,23 @@ __global__ void k_min_lb(const uint8_t* __restrict__ alive, const uint8_t* __res
 // bound joins the round minimum (mr), which keeps that minimum <= c and so
 // c' = c, as the exact values would (the true minimum is <= its bound <= c).
 // The replay of a given order (dense) needs every value and skips nothing.
+// advance: one thread also moves the state to this round (0: the first refine,
+// before round 0); stop: exact, the early stop of a single graph ends the peel.
 template <typename T>
 __global__ void k_collect(const uint8_t* __restrict__ alive, uint8_t* __restrict__ fresh, int64_t n,
                           const int32_t* __restrict__ vl, LbArgs a, const T* __restrict__ d,
-                          int keep_all, DevState* st, PeelState p, int32_t* __restrict__ out) {
-    if (st->n_alive == 0) return;
+                          int keep_all, DevState* st, PeelState p, int32_t* __restrict__ out, int advance,
+                          int stop) {
+    if (advance && blockIdx.x == 0 && threadIdx.x == 0) {
+        if (st->n_alive != 0) {
+            const int left = st->n_alive_next;
+            const bool over = stop && st->round >= 0 && !p.gid && early_stop(p.c[0], left);
+            if (left > 0) st->round += 1;  // (the early stop's nodes left in a round of their own)
+            st->n_alive = over ? 0 : left;
+            st->n_alive_next = 0;
+        }
+        st->nR = 0;
+    }
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t nround = (n + 31) & ~(int64_t)31;
@@ -278,105 +349,6 @@ __global__ void k_select(uint8_t* __restrict__ alive, const T* __restrict__ d, i
     if (lane == 0 && keep) atomicAdd(&st->n_alive_next, keep);
     if (blockIdx.x == 0 && threadIdx.x == 0)
         atomicAdd(&st->bytes[kProfPeel], (unsigned long long)n * (1 + sizeof(T)));
-}
-
-// Exact mode early stop: when c >= |X_new| - 1 every remaining node gets core
-// c in round `round + 1`.  Every block evaluates the condition; block 0
-// records it for the kernels that follow (they skip the refresh).
-template <typename C>
-__global__ void k_assign_rest(uint8_t* __restrict__ alive, int64_t n, const int32_t* __restrict__ vl,
-                              DevState* st, PeelState p, C* __restrict__ core,
-                              int32_t* __restrict__ round_of) {
-    if (st->n_alive == 0) return;
-    // single graphs only (a batch has no global early stop)
-    const unsigned long long m = round_min(p, 0);
-    const unsigned long long c = p.c[0] > m ? p.c[0] : m;
-    const int left = st->n_alive_next;
-    const bool early = left > 0 && c + 1 >= (unsigned long long)left;
-    if (blockIdx.x == 0 && threadIdx.x == 0) st->early = early ? 1 : 0;
-    if (!early) return;
-    const int round = st->round + 1;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int64_t v = vl ? vl[i] : i;
-        if (alive[v] == 1) {
-            core[v] = (C)c;
-            round_of[v] = round;
-            alive[v] = 0;
-        }
-    }
-}
-
-// Batches: the early stop of each graph on its own (c_g >= |X_g| - 1 after
-// this round's removal).  Finished graphs' nodes leave at once, so the
-// refresh that follows never reaches them.
-template <typename C>
-__global__ void k_assign_rest_batch(uint8_t* __restrict__ alive, int64_t n,
-                                    const int32_t* __restrict__ vl, DevState* st, PeelState p,
-                                    C* __restrict__ core, int32_t* __restrict__ round_of) {
-    if (st->n_alive == 0) return;
-    const int round = st->round + 1;
-    int gone = 0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int64_t v = vl ? vl[i] : i;
-        if (alive[v] == 1) {
-            const int g = p.gid[v];
-            const unsigned long long m = round_min(p, g);
-            const unsigned long long c = p.c[g] > m ? p.c[g] : m;
-            const int left = *(volatile int32_t*)(p.left + g);
-            if (left > 0 && c + 1 >= (unsigned long long)left) {
-                core[v] = (C)c;
-                round_of[v] = round;
-                alive[v] = 0;
-                ++gone;
-            }
-        }
-    }
-    for (int off = 16; off > 0; off >>= 1) gone += __shfl_down_sync(kFull, gone, off);
-    if ((threadIdx.x & 31) == 0 && gone) atomicSub(&st->n_alive_next, gone);
-}
-
-// Ends a round: removed nodes leave (alive = 0, dead bitmap bit set); the
-// last block to finish advances the state and zeroes the per-round counters.
-__global__ void k_finish(uint8_t* __restrict__ alive, const int32_t* __restrict__ R, DevState* st,
-                         uint32_t* __restrict__ deadbm, PeelState p, int64_t ngraphs) {
-    __shared__ int s_last;
-    const int nR = st->nR;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nR; i += stride) {
-        const int v = R[i];
-        alive[v] = 0;
-        atomicOr(deadbm + (v >> 5), 1u << (v & 31));
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(&st->done, 1) == (int)gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    for (int i = threadIdx.x; i < kRcCount; i += blockDim.x) st->rc[i] = 0;
-    // every graph: c = max(c, this round's minimum); minima reset
-    for (int64_t q = threadIdx.x; q < ngraphs; q += blockDim.x) {
-        const unsigned long long m = round_min(p, (int)q);
-        if (m != ~0ull && m > p.c[q]) p.c[q] = m;
-        p.mn[q] = ~0ull;
-        p.mr[q] = ~0ull;
-        p.mu[q] = ~0ull;
-    }
-    if (threadIdx.x == 0) {
-        if (st->n_alive != 0) {
-            st->round += st->early ? 2 : 1;
-            st->n_alive = st->early ? 0 : st->n_alive_next;
-        }
-        st->n_alive_next = 0;
-        st->nR = 0;
-        st->nQ = 0;
-        st->early = 0;
-        st->done = 0;
-    }
 }
 
 // EstDense: the round's candidate set X is the alive set with every value
@@ -651,19 +623,21 @@ PeelState peel_state(const Graph& g, bool sampled) {
 
 int64_t peel_graphs(const Graph& g) { return g.gid ? g.ngraphs : 1; }
 
+
 // Recompute the last level of the refine list (stale nodes with lb <= T).
-int refine(Graph& g, bool sampled, cudaStream_t s) {
+int refine(Graph& g, bool sampled, cudaStream_t s, bool advance) {
     const int grid = peel_grid(g);
     const LbArgs la = lb_args(g);
     prof_begin(g, kProfPeel, s);
     if (sampled)
         k_collect<unsigned long long><<<grid, kPeelThreads, 0, s>>>(
-            g.alive, g.fresh, g.vcount, g.vlist, la, g.d64, g.dense ? 1 : 0, g.state, peel_state(g, sampled),
-            g.listB);
+            g.alive, g.fresh, g.vcount, g.vlist, la, g.d64, g.dense ? 1 : 0, g.state, peel_state(g, sampled), g.listB,
+            advance ? 1 : 0, 0);
     else
         k_collect<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.fresh, g.vcount, g.vlist, la,
                                                          g.d32, g.dense ? 1 : 0, g.state,
-                                                         peel_state(g, sampled), g.listB);
+                                                         peel_state(g, sampled), g.listB,
+            advance ? 1 : 0, g.dense ? 0 : 1);
     count_launch(g, 1);
     prof_end(g, kProfPeel, s);
     if (sampled) return launch_level(g, g.h, g.listB, &g.state->nQ, 0, 0, s, 2);
@@ -678,12 +652,12 @@ int start_peel(Graph& g, bool sampled, cudaStream_t s) {
     int rc = KH_OK;
     if (sampled) {
         // every list below each node's last level; the last level itself stays lazy
-        KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.meta, 0, sizeof(uint32_t) * (size_t)g.hmax * (size_t)g.n, s));
+        if ((rc = launch_init_meta(g, s))) return rc;
         for (int i = 1; i < g.hmax && rc == KH_OK; ++i)
             rc = launch_level(g, i, nullptr, nullptr, g.n, 0, s, 0, 1);
         if (rc) return rc;
         KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.d64, 0xff, sizeof(unsigned long long) * (size_t)g.n, s));
-        launch_stale_sampled(g, nullptr, nullptr, s);
+        launch_stale_all(g, s);
     } else {
         k_init_exact<<<grid, kPeelThreads, 0, s>>>(g.rowptr, g.col, g.alive, g.start_keep ? 1 : 0,
                                                    g.n, g.degX, g.d32);
@@ -693,7 +667,7 @@ int start_peel(Graph& g, bool sampled, cudaStream_t s) {
     const LbArgs la = lb_args(g);
     k_min_lb<<<grid, kPeelThreads, 0, s>>>(g.alive, g.fresh, g.n, la, g.state, peel_state(g, sampled));
     count_launch(g, 1);
-    rc = refine(g, sampled, s);
+    rc = refine(g, sampled, s, false);
     if (rc) return rc;
     // the bootstrap used the per-round counters: zero them for round 0
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.state->rc, 0, sizeof(int) * kRcCount, s));
@@ -705,10 +679,8 @@ int start_peel(Graph& g, bool sampled, cudaStream_t s) {
 }
 
 // The second half of a round: the refresh of the nodes the removal set R
-// affects, then the end of the round.
-int refresh_and_finish(Graph& g, bool sampled, cudaStream_t s) {
-    const int grid = peel_grid(g);
-    const PeelState ps = peel_state(g, sampled);
+// affects.  Its first kernel also ends the selection (end_round).
+int refresh(Graph& g, bool sampled, cudaStream_t s) {
     int rc = KH_OK;
     if (!sampled) {
         // the ball of R in the old graph: alive degrees drop (hop 1), the
@@ -725,61 +697,47 @@ int refresh_and_finish(Graph& g, bool sampled, cudaStream_t s) {
     } else {
         int* rcs = g.state->rc;
         for (int i = 1; i <= g.hmax && rc == KH_OK; ++i) {
-            // level i candidates: A(R), plus A(nodes whose level i-1 changed)
+            // level i candidates: A(R), plus A(nodes whose level i-1 changed);
+            // nodes whose last level is i become stale (lazy refine) ...
             launch_mark_neighbours(g, g.listR, &g.state->nR, i >= 2 ? g.listC[(i - 1) & 1] : nullptr,
                                    rcs + kRcC + i - 1, i, rcs + kRcW + i, s);
-            // nodes with more levels recompute level i (tracking changes) ...
+            // ... those with more levels recompute level i (tracking changes)
             if (i < g.hmax) rc = launch_level(g, i, g.listW, rcs + kRcW + i, 0, 1, s, 1);
-            // ... nodes whose last level is i become stale (lazy refine)
-            if (i >= g.hmin) launch_stale_sampled(g, g.listW, rcs + kRcW + i, s, i);
         }
-        if (rc) return rc;
     }
-    prof_begin(g, kProfPeel, s);
-    k_finish<<<grid, kPeelThreads, 0, s>>>(g.alive, g.listR, g.state, g.deadbm, ps, peel_graphs(g));
-    count_launch(g, 1);
-    prof_end(g, kProfPeel, s);
-    return KH_OK;
+    return rc;
 }
 
 // One peeling round, entirely stream-ordered (capturable).
 int launch_round(Graph& g, bool sampled, cudaStream_t s) {
     const int grid = peel_grid(g);
+    const PeelState ps = peel_state(g, sampled);
     int rc = KH_OK;
+    // end of the previous round; U = min of the upper bounds (and of the fresh
+    // values); refine stale nodes with lb <= max(c, U) (folds its results into mr).
+    // EstDense: the threshold stays infinite (no round minimum is taken), so
+    // every stale node is recomputed in full before the sum is taken.
+    BeginArgs ba{g.alive, g.fresh, g.vcount, g.vlist, g.state, ps, g.listR, g.deadbm,
+                 sampled || g.dense ? nullptr : g.core32, g.round_of, g.dense ? 0 : 1};
+    prof_begin(g, kProfPeel, s);
+    if (sampled) k_begin<unsigned long long><<<grid, kPeelThreads, 0, s>>>(ba, g.d64);
+    else k_begin<int32_t><<<grid, kPeelThreads, 0, s>>>(ba, g.d32);
+    count_launch(g, 1);
+    prof_end(g, kProfPeel, s);
+    rc = refine(g, sampled, s, true);
+    if (rc) return rc;
+    prof_begin(g, kProfPeel, s);
     if (g.dense) {
-        // EstDense: the threshold stays infinite (no round minimum is taken),
-        // so every stale node is recomputed in full before the sum is taken
-        rc = refine(g, sampled, s);
-        if (rc) return rc;
-        prof_begin(g, kProfPeel, s);
         if (sampled)
             k_dense_sum<unsigned long long><<<grid, kPeelThreads, 0, s>>>(
                 g.alive, g.d64, g.vcount, g.vlist, g.state, g.dsum, g.n + 1);
         else
             k_dense_sum<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.d32, g.vcount, g.vlist,
                                                                g.state, g.dsum, g.n + 1);
-        k_select_sched<<<grid, kPeelThreads, 0, s>>>(g.alive, g.sched, g.vcount, g.vlist, g.state,
-                                                     peel_state(g, sampled), g.listR, g.seen, g.round_of);
+        k_select_sched<<<grid, kPeelThreads, 0, s>>>(g.alive, g.sched, g.vcount, g.vlist, g.state, ps,
+                                                     g.listR, g.seen, g.round_of);
         count_launch(g, 2);
-        prof_end(g, kProfPeel, s);
-        return refresh_and_finish(g, sampled, s);
-    }
-    // U = min of the upper bounds (and of the fresh values); refine stale
-    // nodes with lb <= max(c, U); the refine folds its results into mr
-    prof_begin(g, kProfPeel, s);
-    if (sampled)
-        k_min_alive<unsigned long long><<<grid, kPeelThreads, 0, s>>>(
-            g.alive, g.fresh, g.d64, g.vcount, g.vlist, g.state, g.pmu, g.pmn, g.gid);
-    else
-        k_min_alive<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.fresh, g.d32, g.vcount, g.vlist,
-                                                           g.state, g.pmu, g.pmn, g.gid);
-    count_launch(g, 1);
-    prof_end(g, kProfPeel, s);
-    rc = refine(g, sampled, s);
-    if (rc) return rc;
-    prof_begin(g, kProfPeel, s);
-    const PeelState ps = peel_state(g, sampled);
-    if (sampled) {
+    } else if (sampled) {
         k_select<unsigned long long, unsigned long long><<<grid, kPeelThreads, 0, s>>>(
             g.alive, g.d64, g.vcount, g.vlist, g.state, ps, g.core64, g.round_of, g.listR, g.seen);
         count_launch(g, 1);
@@ -787,17 +745,9 @@ int launch_round(Graph& g, bool sampled, cudaStream_t s) {
         k_select<int32_t, int32_t><<<grid, kPeelThreads, 0, s>>>(
             g.alive, g.d32, g.vcount, g.vlist, g.state, ps, g.core32, g.round_of, g.listR, g.seen);
         count_launch(g, 1);
-        if (!g.gid)  // the early stop of Sec. 5
-            k_assign_rest<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.vcount, g.vlist, g.state,
-                                                                 ps, g.core32, g.round_of);
-        else  // the same, graph by graph
-            k_assign_rest_batch<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.vcount, g.vlist,
-                                                                       g.state, ps, g.core32,
-                                                                       g.round_of);
-        count_launch(g, 1);
     }
     prof_end(g, kProfPeel, s);
-    return refresh_and_finish(g, sampled, s);
+    return refresh(g, sampled, s);
 }
 
 int check_state_err(Graph& g, const DevState& hs) {
@@ -866,6 +816,8 @@ int run_estimate_all(Graph& g) {
     return KH_OK;
 }
 
+RoundEnd round_end(const Graph& g) { return {g.pc, g.pmn, g.pmr, g.pmu, peel_graphs(g)}; }
+
 // The peel's CSR and node list are the graph's own outside a peel.
 struct PeelView {
     Graph& g;
@@ -913,7 +865,8 @@ int run_core(Graph& g, bool sampled, void* out_core, int32_t* round_of_host, boo
     memcpy(init.bytes, keep_bytes, sizeof(keep_bytes));  // profiling counters accumulate
     init.minval = ~0ull;
     init.minU = ~0ull;
-    init.n_alive = (int)(g.start_keep ? g.start_alive : g.n);
+    init.n_alive = init.n_alive_next = (int)(g.start_keep ? g.start_alive : g.n);
+    init.round = -1;  // the first round's k_collect makes it 0
     KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(g.state, &init, sizeof(init), cudaMemcpyHostToDevice, s));
     KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));  // `init` is a host stack object
     const size_t pbytes = sizeof(unsigned long long) * (size_t)peel_graphs(g);
@@ -933,7 +886,6 @@ int run_core(Graph& g, bool sampled, void* out_core, int32_t* round_of_host, boo
     rc = start_peel(g, sampled, s);
     if (rc) return rc;
     // the BFS scratch must exist before capture (its allocation may synchronize)
-    DevState hs;
     int64_t launches = 0;
     cudaGraphExec_t exec = nullptr;
     const bool use_graph = !g.prof_on;
@@ -941,40 +893,58 @@ int run_core(Graph& g, bool sampled, void* out_core, int32_t* round_of_host, boo
         rc = round_graph(g, sampled, s, &exec);
         if (rc) return rc;
     }
-    int64_t compact_at = g.start_keep ? g.start_alive : g.n;  // alive count at the last compaction
-    for (;;) {
+    // Each replay's state comes back to pinned memory; the next replay is sent off
+    // before it is looked at, so that the device does not wait for the host (12 to
+    // 20 us per 8 rounds), unless the replay looked at last says that this one
+    // ends the peel (an idle replay costs about as much).
+    DevState* states = static_cast<DevState*>(g.ctx->peel_state);
+    auto replay = [&](int slot) -> int {
         NvtxRange nvtx_range(use_graph ? "peel rounds (graph replay)" : "peel round");
         if (use_graph) {
             KH_CUDA_TRY(g.ctx, cudaGraphLaunch(exec, s));
             launches += kRoundsPerGraph;
             count_launch(g, g.round_exec_kernels);
         } else {
-            rc = launch_round(g, sampled, s);
-            if (rc) return rc;
+            const int rc2 = launch_round(g, sampled, s);
+            if (rc2) return rc2;
             launches += 1;
         }
         KH_CUDA_TRY(g.ctx, cudaGetLastError());
-        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&hs, g.state, sizeof(DevState), cudaMemcpyDeviceToHost, s));
-        KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&states[slot], g.state, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+        KH_CUDA_TRY(g.ctx, cudaEventRecord(g.ctx->peel_done[slot], s));
+        return KH_OK;
+    };
+    DevState hs;
+    int64_t compact_at = g.start_keep ? g.start_alive : g.n;  // alive count at the last compaction
+    int64_t alive_before = compact_at, removed = 0;           // of the replay looked at last
+    bool ahead = false;                                       // the next replay is under way
+    for (int slot = 0;; slot ^= 1) {
+        if (!ahead && (rc = replay(slot))) return rc;
+        ahead = use_graph && alive_before > 2 * removed && launches <= g.n + 2;
+        if (ahead && (rc = replay(slot ^ 1))) return rc;
+        KH_CUDA_TRY(g.ctx, cudaEventSynchronize(g.ctx->peel_done[slot]));
+        hs = states[slot];
         rc = check_state_err(g, hs);
         if (rc) return rc;
-        if (hs.n_alive == 0) break;
+        if (hs.n_alive == 0 || hs.n_alive_next == 0) break;
+        removed = alive_before - hs.n_alive_next;
+        alive_before = hs.n_alive_next;
         const bool may = g.compact_mode == KH_COMPACT_ALWAYS ||
                          (g.compact_mode == KH_VAR_AUTO && compact_at >= kCompactMinAlive);
-        if (may && 2 * (int64_t)hs.n_alive <= compact_at) {
+        if (may && 2 * (int64_t)hs.n_alive_next <= compact_at) {
             NvtxRange nvtx_compact("peel compaction");
-            rc = compact_peel(g, s);
+            rc = compact_peel(g, s);  // (waits for the replay under way)
             if (rc) return rc;
-            compact_at = hs.n_alive;
+            compact_at = hs.n_alive_next;
             if (use_graph) {
                 rc = round_graph(g, sampled, s, &exec);  // the launches changed: capture again
                 if (rc) return rc;
             }
         }
-        if (launches > g.n + 2 + kRoundsPerGraph)
+        if (launches > g.n + 2 + 3 * kRoundsPerGraph)
             return set_error(g.ctx, KH_ETIMEOUT, "peeling did not finish within n+1 rounds");
     }
-    g.last_rounds = hs.round;
+    g.last_rounds = hs.round + 1;
     g.last_updates = (int64_t)hs.updates;
     for (int i = 0; i <= kMaxH; ++i) {
         g.last_lvl_work[i] = (int64_t)hs.lvl_work[i];

@@ -45,9 +45,11 @@ constexpr int kLuPerSm = 12;  // CTAs per SM of k_levelU
 
 // Meta word of a list (one per level and node): |B| in bits 0-13, k in bits
 // 14-19, the highest rank present in bits 20-24, the dense-form flag, and a
-// flag that is set while the node is alive (a removed node's word is zero).
+// flag that is set while the node is alive (a removed node's word is zero; in
+// a peel the last level's word has it from the start).
 constexpr uint32_t kMetaAlive = 1u << 31;
 constexpr uint32_t kMetaDense = 1u << 30;
+constexpr uint32_t kMetaFresh = 1u << 29;  // last level: (|B|, k) are those of the current alive set
 __device__ __forceinline__ int meta_size(uint32_t m) { return (int)(m & 0x3fffu); }
 __device__ __forceinline__ int meta_k(uint32_t m) { return (int)((m >> 14) & 63u); }
 __device__ __forceinline__ int meta_top(uint32_t m) { return (int)((m >> 20) & 31u); }
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(kL1Threads) k_level1(LevelArgs a) {
                 const unsigned long long est = estimate_of(Skap, kappa, rv, nl.M);
                 a.est[v] = est;
                 if (a.min_done) atomicMin(a.min_done + (a.gid ? a.gid[v] : 0), est);
-                record_change(a, nl, v, meta_pack(Skap, kappa, top, false));
+                record_change(a, nl, v, meta_pack(Skap, kappa, top, false) | kMetaFresh);
                 atomicAdd(a.updates, 1ull);
             }
             continue;
@@ -364,7 +366,7 @@ __global__ void __launch_bounds__(kL1Threads) k_level1(LevelArgs a) {
                 const unsigned long long est = estimate_of(Skap, kappa, rv, nl.M);
                 a.est[v] = est;
                 if (a.min_done) atomicMin(a.min_done + (a.gid ? a.gid[v] : 0), est);
-                record_change(a, nl, v, meta_pack(Skap, kappa, s_top, false));
+                record_change(a, nl, v, meta_pack(Skap, kappa, s_top, false) | kMetaFresh);
                 atomicAdd(a.updates, 1ull);
                 my_bytes += level1_bytes(e - b, Skap, 1);
             }
@@ -866,7 +868,9 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
     const int64_t total = PARTS        ? min((int64_t)(*a.n_sub), a.part_cap)
                           : a.worklist ? (int64_t)(*a.d_count)
                                        : a.count_static;
-    if (total == 0) return;
+    // the first items go by block index, so that a short list costs the other
+    // blocks neither a counter nor a table
+    if (blockIdx.x >= total) return;
     unsigned long long my_bytes = 0;
     // the table starts empty once per launch; every node leaves it empty again
 #pragma unroll 1
@@ -875,9 +879,8 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
     // the CTA's next item: a node, or (PARTS) a part of a split node
     const int* items = PARTS ? a.sub_v : a.worklist;
     if (tid == 0) {
-        const int i = atomicAdd(a.work_ctr, 1);
-        sh.idx = i;
-        if (i < total) sh.v = items ? items[i] : i;
+        sh.idx = blockIdx.x;
+        sh.v = items ? items[blockIdx.x] : (int)blockIdx.x;
     }
     int cls_graph = -1;
     for (;;) {
@@ -888,7 +891,7 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
         int mode = PARTS ? 1 : 0;
         const int v = sh.v, part = PARTS ? a.sub_j[idx] : 0;
         int next = 0;
-        if (tid == 0) next = atomicAdd(a.work_ctr, 1);
+        if (tid == 0) next = (int)gridDim.x + atomicAdd(a.work_ctr, 1);
         bool skip = PARTS && v < 0;  // a part the plan could not place
         NodeLevel nl{};
         int64_t b = 0;
@@ -1141,7 +1144,7 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
                     const unsigned long long est = estimate_of(S, kappa, rv, nl.M);
                     a.est[v] = est;
                     if (a.min_done) atomicMin(a.min_done + g, est);
-                    record_change(a, nl, v, meta_pack(S, kappa, top, false));
+                    record_change(a, nl, v, meta_pack(S, kappa, top, false) | kMetaFresh);
                     atomicAdd(a.updates, 1ull);
                     my_bytes += 21ull + (!PARTS || mode == 0 ? lists_bytes : 0);
                 }
@@ -1181,108 +1184,44 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
 // j >= k[u,i] - 1, the level and the members are all unchanged.  The test needs
 // k[u,i] for the current node set: intermediate levels always have it, a last
 // level only while u is fresh.
-struct MarkFilter {
-    const int8_t* rho;    // nullptr: no filter
-    const uint32_t* meta; // meta words of level `phase`
-    const uint8_t* hv;    // per-node h (batches) or nullptr
+struct MarkArgs {
+    const int64_t* rowptr;
+    const int32_t* col;
+    const uint32_t* meta;  // meta words of level `phase`
+    int32_t* seen;
+    const int32_t* list1;
+    const int* nlist1;
+    const int32_t* list2;  // may be nullptr; rank-filtered by rho
+    const int* nlist2;
+    const int8_t* rho;
+    const uint8_t* hv;     // per-node h (batches) or nullptr
     int h;
-    const uint8_t* fresh;
+    int phase;
+    int32_t* wl;
+    int* nwl;
+    int64_t cap;
+    const DevState* st;
+    unsigned long long* bytes;
+    RoundEnd end;          // phase 1: the round's c and minima advance here
+    // STALE: nodes whose last level is `phase` become stale instead of listed
+    uint32_t* meta_last;   // = meta, writable
+    const uint32_t* prev;  // meta words of level phase - 1 (nullptr at phase 1)
+    const uint32_t* key32;
+    const int32_t* bestnb;
+    const int32_t* Mv;
+    int64_t M;
+    uint8_t* fresh;
+    unsigned long long* lb;
 };
 
-__device__ __forceinline__ bool level_may_change(const MarkFilter& f, int u, int rw, int level) {
-    const int hu = f.hv ? (int)f.hv[u] : f.h;
-    const bool known = level < hu || (level == hu && f.fresh[u]);
-    return !known || rw >= meta_k(f.meta[u]) - 1;
-}
-
-// Alive neighbours of the listed nodes (two lists, the second optional and
-// rank-filtered) join the work list once per stamp (round, phase).  One CTA
-// per listed node.
 // (The CTA-wide path of the row kernels below: rows longer than kWarpRow are
 // gathered per block and done by all its warps after the warp-per-node pass.)
 constexpr int kWarpRow = 2048;
 constexpr int kBlockHeavy = 64;
+constexpr int kMarkWarps = 32;  // most warps on one listed node
 
 __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
     return a > b ? a : b;
-}
-
-// Visit entries [k0 + lane, ...) of a listed node's row: mark each alive
-// neighbour that passes the filter once per stamp and append it to wl.
-__device__ __forceinline__ void mark_entry(const int32_t* __restrict__ col,
-                                           const uint8_t* __restrict__ alive,
-                                           int32_t* __restrict__ seen, int32_t* __restrict__ wl,
-                                           int* nwl, int64_t cap, const MarkFilter& f, bool filt,
-                                           int rw, int phase, int stamp, int64_t k, int64_t e,
-                                           int lane) {
-    bool isnew = false;
-    int32_t u = 0;
-    if (k < e) {
-        u = col[k];
-        if (alive[u] == 1 && (!filt || level_may_change(f, u, rw, phase)) &&
-            *(volatile int32_t*)(seen + u) != stamp)
-            isnew = atomicExch(seen + u, stamp) != stamp;
-    }
-    const uint32_t m = __ballot_sync(kFull, isnew);
-    if (!m) return;
-    int base = 0;
-    if (lane == 0) base = atomicAdd(nwl, __popc(m));
-    base = __shfl_sync(kFull, base, 0);
-    if (isnew) {
-        const int p = base + __popc(m & ((1u << lane) - 1u));
-        if (p < cap) wl[p] = u;
-    }
-}
-
-__global__ void k_mark_nbrs(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                            const uint8_t* __restrict__ alive, int32_t* __restrict__ seen,
-                            const int32_t* __restrict__ list1, const int* __restrict__ nlist1,
-                            const int32_t* __restrict__ list2, const int* __restrict__ nlist2,
-                            int32_t* __restrict__ wl, int* nwl, const DevState* __restrict__ st,
-                            int phase, int64_t cap, unsigned long long* bytes, MarkFilter f) {
-    __shared__ int s_heavy[kBlockHeavy];
-    __shared__ int s_nheavy;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n1 = *nlist1;
-    const int nin = n1 + (list2 ? *nlist2 : 0);
-    const int stamp = st->round * kPhaseStride + phase;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long my_bytes = 0;
-    if (threadIdx.x == 0) s_nheavy = 0;
-    __syncthreads();
-    // one warp per listed node; rows longer than kWarpRow go to the block afterwards
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nin; i += nw) {
-        const int w = i < n1 ? list1[i] : list2[i - n1];
-        const int64_t b = rowptr[w], e = rowptr[w + 1];
-        if (e - b > kWarpRow) {
-            int slot = 0;
-            if (lane == 0) slot = atomicAdd(&s_nheavy, 1);
-            slot = __shfl_sync(kFull, slot, 0);
-            if (slot < kBlockHeavy) {
-                if (lane == 0) s_heavy[slot] = (int)i;
-                continue;
-            }
-        }
-        const bool filt = f.rho != nullptr && i >= n1;
-        const int rw = filt ? (int)f.rho[w] : 0;
-        if (lane == 0) my_bytes += 12ull + 4ull * (unsigned long long)(e - b);
-        for (int64_t k0 = b; k0 < e; k0 += 32)
-            mark_entry(col, alive, seen, wl, nwl, cap, f, filt, rw, phase, stamp, k0 + lane, e, lane);
-    }
-    __syncthreads();
-    const int nh = min(s_nheavy, kBlockHeavy);
-    for (int j = 0; j < nh; ++j) {
-        const int i = s_heavy[j];
-        const int w = i < n1 ? list1[i] : list2[i - n1];
-        const bool filt = f.rho != nullptr && i >= n1;
-        const int rw = filt ? (int)f.rho[w] : 0;
-        const int64_t b = rowptr[w], e = rowptr[w + 1];
-        if (threadIdx.x == 0) my_bytes += 12ull + 4ull * (unsigned long long)(e - b);
-        for (int64_t k0 = b + warp * 32; k0 < e; k0 += blockDim.x)
-            mark_entry(col, alive, seen, wl, nwl, cap, f, filt, rw, phase, stamp, k0 + lane, e, lane);
-    }
-    for (int off = 16; off > 0; off >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, off);
-    if (lane == 0 && my_bytes) atomicAdd(bytes, my_bytes);
 }
 
 // Alg. 1 on a list (its meta word), with the node of rank r_first counted
@@ -1291,119 +1230,156 @@ __device__ __forceinline__ unsigned long long est_first(uint32_t m, int r_first,
     return estimate_of(meta_size(m), meta_k(m), r_first, M);
 }
 
-// Mark nodes stale at the last level h and give each a lower bound of its
-// estimate: N(v; h-1) and, for every alive neighbour w, N(w; h-1) (which
-// contains v) are inside N(v; h); Alg. 1 on either with v's rank first is at
-// most the estimate of N(v; h) (Prop. 4.2).  Only the level-(h-1) sizes and
-// levels are read.  One CTA per node.
-// Batches: a node's h and M come from its graph, and only nodes whose last
-// level is `only_h` (when nonzero) are marked.
-// A row longer than kStaleScan takes its neighbour term from the neighbour
-// of largest degree alone (bestnb) while that neighbour is alive: any alive
-// neighbour w gives a sub-multiset N(w; h-1) of N(v; h) led by v, so one
-// neighbour's term is still a lower bound, at O(1) cost instead of O(deg).
+// Mark u (alive, its last level is the phase; m: that level's meta word) stale
+// and give it a lower bound of its estimate: N(u; h-1) and, for an alive
+// neighbour w, N(w; h-1) (which contains u) are inside N(u; h); Alg. 1 on either
+// with u's rank first is at most the estimate of N(u; h) (Prop. 4.2).  Only
+// the level-(h-1) meta words are read.  The neighbour term comes from the
+// neighbour of largest degree (bestnb) while that is alive, else from the first
+// kStaleScan entries of the row: any alive neighbours give a lower bound
+// (scanning rows of up to 64 entries each time gave no fewer refines that count:
+// 577 -> 569 ms without on Chung-Lu n = 200k, h = 3).
 constexpr int kStaleScan = 64;
-constexpr int kStaleThreads = 256;
+__device__ __forceinline__ void make_stale(const MarkArgs& a, int32_t u, uint32_t m) {
+    unsigned long long lb = 0;
+    if (a.prev) {
+        const int64_t M = a.Mv ? (int64_t)a.Mv[u] : a.M;
+        const int ru = (int)(a.key32[u] >> kIdBits);
+        const int32_t w = a.bestnb[u];
+        lb = est_first(a.prev[u], ru, M);
+        const uint32_t mw = w >= 0 ? a.prev[w] : 0u;
+        if (mw & kMetaAlive) {
+            lb = umax64(lb, est_first(mw, ru, M));
+        } else {
+            const int64_t b = a.rowptr[u];
+            const int n = (int)min((int64_t)kStaleScan, a.rowptr[u + 1] - b);
+#pragma unroll 1
+            for (int k = 0; k < n; ++k) {
+                const uint32_t mk = a.prev[a.col[b + k]];
+                if (mk & kMetaAlive) lb = umax64(lb, est_first(mk, ru, M));
+            }
+        }
+    }
+    a.lb[u] = lb;
+    a.fresh[u] = 0;
+    a.meta_last[u] = m & ~kMetaFresh;
+}
 
-__global__ void k_stale_sampled(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                const uint8_t* __restrict__ alive, const uint8_t* __restrict__ rank,
-                                const uint32_t* __restrict__ meta, int h_all, const uint8_t* __restrict__ hv, int64_t M_all,
-                                const int32_t* __restrict__ Mv, int only_h,
-                                const int32_t* __restrict__ list, const int* __restrict__ nlist,
-                                int64_t n, uint8_t* __restrict__ fresh,
-                                unsigned long long* __restrict__ lb, unsigned long long* bytes,
-                                const int32_t* __restrict__ bestnb) {
-    __shared__ unsigned long long s_max[kStaleThreads / 32];
+// Row entries k0 + 32 q + lane, q < 4, of a listed node (rho rw; -128: no
+// filter): each alive neighbour that passes joins wl once per stamp.  The stamp
+// is read first: most entries of a round's rows are repeats.  meta holds the
+// rest: alive, k, and at the last level whether k is current.
+template <bool STALE>
+__device__ __forceinline__ void mark_step(const MarkArgs& a, int rw, int stamp, int64_t k0, int64_t e,
+                                          int lane) {
+    int32_t u[4];
+    bool go[4];
+    uint32_t m[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t k = k0 + 32 * q + lane;
+        u[q] = k < e ? a.col[k] : -1;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) go[q] = u[q] >= 0 && *(volatile int32_t*)(a.seen + u[q]) != stamp;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) m[q] = go[q] ? a.meta[u[q]] : 0u;
+    int n = 0;
+    uint32_t isnew[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        go[q] = (m[q] & kMetaAlive) != 0;
+        if (go[q] && rw > -128) {
+            const int hu = a.hv ? (int)a.hv[u[q]] : a.h;
+            const bool known = a.phase < hu || (m[q] & kMetaFresh);
+            go[q] = !known || rw >= meta_k(m[q]) - 1;
+        }
+        if (go[q]) go[q] = atomicExch(a.seen + u[q], stamp) != stamp;
+        if (STALE && go[q] && (!a.hv || (int)a.hv[u[q]] == a.phase)) {
+            make_stale(a, u[q], m[q]);
+            go[q] = false;
+        }
+        isnew[q] = __ballot_sync(kFull, go[q]);
+        n += __popc(isnew[q]);
+    }
+    if (!n) return;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(a.nwl, n);
+    base = __shfl_sync(kFull, base, 0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (go[q]) {
+            const int p = base + __popc(isnew[q] & ((1u << lane) - 1u));
+            if (p < a.cap) a.wl[p] = u[q];
+        }
+        base += __popc(isnew[q]);
+    }
+}
+
+// Alive neighbours of the listed nodes (two lists, the second optional and
+// rank-filtered) join the work list once per stamp (round, phase).  A short list
+// is spread over all warps, several to a node: one warp walking a row of 1000
+// entries in 40 dependent steps was the length of the launch (52 us a round on
+// the (k,2)-core of Chung-Lu n = 50k under events, 10 us so; that core 538 -> 368
+// ms, the (k,3)-core of R-MAT 18 297 -> 246 ms).
+template <bool STALE>
+__global__ void k_mark_nbrs(MarkArgs a) {
+    if (blockIdx.x == 0) end_round(a.end);
     __shared__ int s_heavy[kBlockHeavy];
     __shared__ int s_nheavy;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t cnt = list ? (int64_t)(*nlist) : n;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int n1 = *a.nlist1;
+    const int nin = n1 + (a.list2 ? *a.nlist2 : 0);
+    const int stamp = a.st->round * kPhaseStride + a.phase;
+    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+    const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int per = nin > 0 ? min(kMarkWarps, max(1, nw / nin)) : 1;  // warps per node
     unsigned long long my_bytes = 0;
     if (threadIdx.x == 0) s_nheavy = 0;
     __syncthreads();
-    // one warp per node; rows longer than kWarpRow go to the block afterwards
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < cnt; i += nw) {
-        const int v = list ? list[i] : (int)i;
-        if (alive[v] != 1) continue;  // warp-uniform
-        const int h = hv ? (int)hv[v] : h_all;
-        if (only_h && h != only_h) continue;
-        const int64_t b = rowptr[v], e = rowptr[v + 1];
-        if (bestnb && h >= 2 && e - b > kStaleScan) {
-            const int w = bestnb[v];
-            if (alive[w] == 1) {  // warp-uniform
-                if (lane == 0) {
-                    const int64_t M = Mv ? (int64_t)Mv[v] : M_all;
-                    const uint32_t* prev = meta + (size_t)(h - 2) * (size_t)n;
-                    const int rv = rank[v];
-                    lb[v] = umax64(est_first(prev[v], rv, M), est_first(prev[w], rv, M));
-                    fresh[v] = 0;
-                    my_bytes += 29ull + 9ull;
-                }
-                continue;
-            }
-        }
-        if (e - b > kWarpRow) {
-            int slot = 0;
-            if (lane == 0) slot = atomicAdd(&s_nheavy, 1);
+    for (int i = wid / per; i < nin; i += nw / per) {
+        if (wid / per >= nw / per) break;  // the warps past the last whole group
+        const int sub = wid % per;
+        const int w = i < n1 ? a.list1[i] : a.list2[i - n1];
+        const int64_t b = a.rowptr[w], e = a.rowptr[w + 1];
+        if (e - b > (int64_t)kWarpRow * per) {
+            int slot = kBlockHeavy;
+            if (lane == 0 && per == 1) slot = atomicAdd(&s_nheavy, 1);
             slot = __shfl_sync(kFull, slot, 0);
             if (slot < kBlockHeavy) {
-                if (lane == 0) s_heavy[slot] = v;
+                if (lane == 0) s_heavy[slot] = i;
                 continue;
             }
         }
-        const int64_t M = Mv ? (int64_t)Mv[v] : M_all;
-        const uint32_t* prev = h >= 2 ? meta + (size_t)(h - 2) * (size_t)n : nullptr;
-        unsigned long long m = 0;
-        if (prev) {
-            const int rv = rank[v];
-            for (int64_t k = b + lane; k < e; k += 32) {
-                const int32_t w = col[k];
-                const uint32_t mw = prev[w];
-                if (mw & kMetaAlive) m = umax64(m, est_first(mw, rv, M));
-            }
-            for (int off = 16; off > 0; off >>= 1) m = umax64(m, __shfl_down_sync(kFull, m, off));
-            m = umax64(m, est_first(prev[v], rv, M));
-        }
-        if (lane == 0) {
-            lb[v] = m;
-            fresh[v] = 0;
-            my_bytes += 29ull + 9ull * (unsigned long long)(e - b);
-        }
+        const int rw = a.rho && i >= n1 ? (int)a.rho[w] : -128;
+        if (lane == 0 && sub == 0) my_bytes += 12ull + 4ull * (unsigned long long)(e - b);
+        for (int64_t k0 = b + sub * 128; k0 < e; k0 += per * 128) mark_step<STALE>(a, rw, stamp, k0, e, lane);
     }
     __syncthreads();
     const int nh = min(s_nheavy, kBlockHeavy);
     for (int j = 0; j < nh; ++j) {
-        const int v = s_heavy[j];
-        const int h = hv ? (int)hv[v] : h_all;
-        const int64_t M = Mv ? (int64_t)Mv[v] : M_all;
-        const uint32_t* prev = h >= 2 ? meta + (size_t)(h - 2) * (size_t)n : nullptr;
-        unsigned long long m = 0;
-        const int64_t b = rowptr[v], e = rowptr[v + 1];
-        if (prev) {
-            const int rv = rank[v];
-            for (int64_t k = b + threadIdx.x; k < e; k += blockDim.x) {
-                const int32_t w = col[k];
-                const uint32_t mw = prev[w];
-                if (mw & kMetaAlive) m = umax64(m, est_first(mw, rv, M));
-            }
-            for (int off = 16; off > 0; off >>= 1) m = umax64(m, __shfl_down_sync(kFull, m, off));
-            if (lane == 0) s_max[warp] = m;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = umax64(m, s_max[w]);
-                m = umax64(m, est_first(prev[v], rv, M));
-            }
-        }
-        if (threadIdx.x == 0) {
-            lb[v] = m;
-            fresh[v] = 0;
-            my_bytes += 29ull + 9ull * (unsigned long long)(e - b);
-        }
-        __syncthreads();
+        const int i = s_heavy[j];
+        const int w = i < n1 ? a.list1[i] : a.list2[i - n1];
+        const int rw = a.rho && i >= n1 ? (int)a.rho[w] : -128;
+        const int64_t b = a.rowptr[w], e = a.rowptr[w + 1];
+        if (threadIdx.x == 0) my_bytes += 12ull + 4ull * (unsigned long long)(e - b);
+        for (int64_t k0 = b + warp * 128; k0 < e; k0 += 4 * blockDim.x) mark_step<STALE>(a, rw, stamp, k0, e, lane);
     }
     for (int off = 16; off > 0; off >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, off);
-    if (lane == 0 && my_bytes) atomicAdd(bytes, my_bytes);
+    if (lane == 0 && my_bytes) atomicAdd(a.bytes, my_bytes);
+}
+
+// Start of a peel: every alive node stale (make_stale), whatever its last level.
+__global__ void k_stale_all(MarkArgs a, int64_t n, const uint8_t* __restrict__ alive, uint32_t* meta) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        if (alive[v] != 1) continue;
+        const int h = a.hv ? (int)a.hv[v] : a.h;
+        a.meta_last = meta + (size_t)(h - 1) * (size_t)n;
+        a.prev = h >= 2 ? meta + (size_t)(h - 2) * (size_t)n : nullptr;
+        make_stale(a, (int32_t)v, a.meta_last[v]);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(a.bytes, 38ull * (unsigned long long)n);
 }
 
 }  // namespace
@@ -1733,21 +1709,51 @@ int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
     return KH_OK;
 }
 
+static MarkArgs mark_args(Graph& g, int phase) {
+    MarkArgs a{};
+    a.rowptr = g.rowptr;
+    a.col = g.col;
+    a.meta = a.meta_last = g.meta + (size_t)(phase - 1) * (size_t)g.n;
+    a.prev = phase >= 2 ? g.meta + (size_t)(phase - 2) * (size_t)g.n : nullptr;
+    a.seen = g.seen;
+    a.hv = g.hv;
+    a.h = g.h;
+    a.phase = phase;
+    a.cap = g.n;
+    a.st = g.state;
+    a.bytes = &g.state->bytes[kProfFrontier];
+    a.key32 = g.key32;
+    a.bestnb = g.bestnb;
+    a.Mv = g.Mv;
+    a.M = g.M;
+    a.fresh = g.fresh;
+    a.lb = g.lb64;
+    return a;
+}
+
 void launch_mark_neighbours(Graph& g, const int* list1, const int* cnt1, const int* list2,
                             const int* cnt2, int phase, int* out_count, cudaStream_t s) {
+    MarkArgs a = mark_args(g, phase);
+    a.list1 = list1;
+    a.nlist1 = cnt1;
+    a.list2 = list2;
+    a.nlist2 = cnt2;
+    a.rho = list2 ? g.rho : nullptr;
+    a.wl = g.listW;
+    a.nwl = out_count;
+    if (phase == 1) a.end = round_end(g);
     const int grid = g.ctx->sm_count * 8;
     prof_begin(g, kProfFrontier, s);
-    MarkFilter f{};
-    if (list2) {
-        f.rho = g.rho;
-        f.meta = g.meta + (size_t)(phase - 1) * (size_t)g.n;
-        f.hv = g.hv;
-        f.h = g.h;
-        f.fresh = g.fresh;
-    }
-    k_mark_nbrs<<<grid, 256, 0, s>>>(g.rowptr, g.col, g.alive, g.seen, list1, cnt1, list2, cnt2,
-                                     g.listW, out_count, g.state, phase, g.n,
-                                     &g.state->bytes[kProfFrontier], f);
+    if (phase >= g.hmin) k_mark_nbrs<true><<<grid, 256, 0, s>>>(a);
+    else k_mark_nbrs<false><<<grid, 256, 0, s>>>(a);
+    count_launch(g, 1);
+    prof_end(g, kProfFrontier, s);
+}
+
+void launch_stale_all(Graph& g, cudaStream_t s) {
+    if (g.n == 0) return;
+    prof_begin(g, kProfFrontier, s);
+    k_stale_all<<<g.ctx->sm_count * 8, 256, 0, s>>>(mark_args(g, 1), g.n, g.alive, g.meta);
     count_launch(g, 1);
     prof_end(g, kProfFrontier, s);
 }
@@ -1765,21 +1771,28 @@ __global__ void k_gather_last(int64_t n, int h_all, const uint8_t* __restrict__ 
     }
 }
 
+// Start of a peel: no lists, every alive node's last-level word alive and stale.
+__global__ void k_init_meta(int64_t n, int h_all, const uint8_t* __restrict__ hv,
+                            const uint8_t* __restrict__ alive, uint32_t* __restrict__ meta) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        const int h = hv ? (int)hv[v] : h_all;
+        if (alive[v] == 1) meta[(size_t)(h - 1) * (size_t)n + (size_t)v] = kMetaAlive;
+    }
+}
+
+int launch_init_meta(Graph& g, cudaStream_t s) {
+    KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.meta, 0, sizeof(uint32_t) * (size_t)g.hmax * (size_t)g.n, s));
+    if (g.n == 0) return KH_OK;
+    k_init_meta<<<g.ctx->sm_count * 4, 256, 0, s>>>(g.n, g.h, g.hv, g.alive, g.meta);
+    count_launch(g, 1);
+    return KH_OK;
+}
+
 void launch_gather_last(Graph& g, uint8_t* lvl_out, int32_t* bs_out, cudaStream_t s) {
     if (g.n == 0) return;
     k_gather_last<<<g.ctx->sm_count * 4, 256, 0, s>>>(g.n, g.h, g.hv, g.meta, lvl_out, bs_out);
     count_launch(g, 1);
-}
-
-void launch_stale_sampled(Graph& g, const int* list, const int* d_count, cudaStream_t s, int only_h) {
-    if (g.n == 0) return;
-    const int grid = g.ctx->sm_count * 8;
-    prof_begin(g, kProfFrontier, s);
-    k_stale_sampled<<<grid, kStaleThreads, 0, s>>>(g.rowptr, g.col, g.alive, g.rank, g.meta, g.h, g.hv,
-                                                   g.M, g.Mv, only_h, list, d_count, g.n, g.fresh,
-                                                   g.lb64, &g.state->bytes[kProfFrontier], g.bestnb);
-    count_launch(g, 1);
-    prof_end(g, kProfFrontier, s);
 }
 
 }  // namespace kh
