@@ -389,6 +389,170 @@ __global__ void __launch_bounds__(kBfsThreads) k_hdeg(BfsArgs a) {
     if (lane == 0 && my_bytes) atomicAdd(a.bytes, my_bytes);
 }
 
+// The peel's refine (LOSS = false) and loss searches at h = 2.  N(v; 2) is the union
+// of the rows of v and of its neighbours (dead nodes are in the bitmap from the
+// start), so there is no queue and no level to wait for: the neighbours' row
+// bounds of a chunk go to shared memory, sorted into short, middle and long
+// rows, and groups of 2, 8 and 32 lanes read them, four entries per lane in
+// flight; rows of kHeavyDeg2 entries or more are read by the whole CTA.
+// A round has a handful of sources, so the chain of one source is the length
+// of the launch: on the exact (k,2)-core of Chung-Lu n = 50k 9 us a refine launch
+// (18 with the search above) and 18 us a loss launch (25), the core 334 -> 262 ms.
+constexpr int kHeavyDeg2 = 512;
+
+template <bool LOSS>
+__global__ void __launch_bounds__(kBfsThreads) k_hdeg2_peel(BfsArgs a) {
+    extern __shared__ __align__(16) uint32_t s_bm_dyn[];
+    __shared__ int64_t s_b[kBfsThreads];
+    __shared__ int s_len[kBfsThreads];
+    __shared__ uint8_t s_q[4][kBfsThreads];
+    __shared__ int s_nq[4], s_cq[4];
+    __shared__ int s_src, s_count;
+    uint32_t* bm = s_bm_dyn;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t total = (int64_t)(*a.d_count);
+    if (blockIdx.x >= total) return;
+    unsigned long long my_bytes = 0;
+    for (int64_t idx = blockIdx.x; idx < total; idx = s_src) {
+        const int v = a.worklist[idx];
+        const int64_t vb = a.rowptr[v];
+        const int deg = (int)(a.rowptr[v + 1] - vb);
+        if (tid == 0) s_count = 0;
+        // visited set := removed nodes (vector copy of the dead bitmap)
+        for (int i = tid; i < (a.words + 3) >> 2; i += kBfsThreads)
+            reinterpret_cast<uint4*>(bm)[i] = __ldcg(reinterpret_cast<const uint4*>(a.deadbm) + i);
+        unsigned long long T = ~0ull;
+        if (!LOSS && a.stop_c) T = stop_level(*a.stop_c > *a.stop_mu ? *a.stop_c : *a.stop_mu);
+        const bool can_stop = T != ~0ull;
+        int my = 0;
+        for (int c0 = 0; c0 <= deg; c0 += kBfsThreads) {  // rows: each neighbour's, then v's own
+            const int i = c0 + tid;
+            int len = 0;
+            if (i <= deg) {
+                const int32_t x = i < deg ? __ldg(a.col + vb + i) : v;
+                const int64_t b = a.rowptr[x];
+                len = (int)(a.rowptr[x + 1] - b);
+                // a neighbour removed in an earlier round is no longer expanded
+                if (i < deg && ((__ldcg(a.deadbm + (x >> 5)) >> (x & 31)) & 1u)) len = 0;
+                s_b[tid] = b;
+                s_len[tid] = len;
+                if (len) my_bytes += 8ull + 4ull * (unsigned long long)len;
+            }
+            const int q = len == 0 ? -1 : len <= 8 ? 0 : len <= 32 ? 1 : len < kHeavyDeg2 ? 2 : 3;
+            if (tid < 4) {
+                s_nq[tid] = 0;
+                s_cq[tid] = 0;
+            }
+            __syncthreads();
+            if (c0 == 0 && tid == 0) bm[v >> 5] |= 1u << (v & 31);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t mq = __ballot_sync(kFull, q == k);
+                if (!mq) continue;
+                int base = 0;
+                if (lane == 0) base = atomicAdd(&s_nq[k], __popc(mq));
+                base = __shfl_sync(kFull, base, 0);
+                if (q == k) s_q[k][base + __popc(mq & ((1u << lane) - 1u))] = (uint8_t)tid;
+            }
+            __syncthreads();
+            auto visit2 = [&](int32_t u) {
+                uint32_t* w = bm + (u >> 5);
+                const uint32_t bit = 1u << (u & 31);
+                if ((*(volatile uint32_t*)w & bit) || (atomicOr(w, bit) & bit)) return;
+                ++my;
+                // (a node within one hop of the removed set is stamped: no loss)
+                if (LOSS) loss_mark(a, u);
+            };
+            for (int hi = 0; hi < s_nq[3]; ++hi) {
+                const int32_t* row = a.col + s_b[s_q[3][hi]];
+                const int n = s_len[s_q[3][hi]];
+                for (int k = tid; k < n; k += 4 * kBfsThreads) {
+                    int32_t u[4];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) u[p] = k + p * kBfsThreads < n ? __ldg(row + k + p * kBfsThreads) : -1;
+#pragma unroll
+                    for (int p = 0; p < 4; ++p)
+                        if (u[p] >= 0) visit2(u[p]);
+                }
+                if (can_stop) fold_count(my, &s_count, lane);
+                if (can_stop && (unsigned long long)*(volatile int*)&s_count > T) break;
+            }
+            int bk = 2, li = -1, pos = 0, n = 0;
+            const int32_t* row = nullptr;
+            for (int step = 0;; ++step) {  // groups claim rows (walk_chunk of the level union)
+                if (can_stop && (step & 3) == 3) {
+                    // the visited set is a subset of the ball: past T the rest is not needed
+                    fold_count(my, &s_count, lane);
+                    int over = 0;
+                    if (lane == 0) over = (unsigned long long)*(volatile int*)&s_count > T;
+                    if (__shfl_sync(kFull, over, 0)) break;
+                }
+                const int lgG = bk == 2 ? 5 : bk == 1 ? 3 : 1;
+                const int lead = lane >> lgG << lgG;
+                const uint32_t need = __ballot_sync(kFull, li == -1 && lane == lead);
+                if (need) {
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(&s_cq[bk], __popc(need));
+                    base = __shfl_sync(kFull, base, 0);
+                    if (li == -1) {
+                        const int j = base + __popc(need & ((1u << lead) - 1u));
+                        li = -2;
+                        if (j < s_nq[bk]) {
+                            li = s_q[bk][j];
+                            row = a.col + s_b[li];
+                            n = s_len[li];
+                            pos = lane - lead;
+                        }
+                    }
+                }
+                if (__all_sync(kFull, li == -2)) {
+                    do --bk;
+                    while (bk >= 0 && s_nq[bk] == 0);
+                    if (bk < 0) break;
+                    li = -1;
+                    continue;
+                }
+                if (li >= 0) {
+                    int32_t u[4];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) u[p] = pos + (p << lgG) < n ? __ldg(row + pos + (p << lgG)) : -1;
+#pragma unroll
+                    for (int p = 0; p < 4; ++p)
+                        if (u[p] >= 0) visit2(u[p]);
+                    pos += 4 << lgG;
+                    if (pos - (lane - lead) >= n) li = -1;
+                }
+            }
+            if (can_stop) fold_count(my, &s_count, lane);
+            __syncthreads();  // the chunk is read
+            if (can_stop && (unsigned long long)s_count > T) break;  // d(v) > T
+        }
+        if (!LOSS) {
+            fold_count(my, &s_count, lane);
+            __syncthreads();
+        }
+        if (tid == 0) {
+            s_src = (int)gridDim.x + atomicAdd(a.work_ctr, 1);
+            if (!LOSS) {
+                if (can_stop && (unsigned long long)s_count > T) {
+                    // v stays stale: its upper bound is kept, its lower bound raised
+                    a.lb[v] = (unsigned long long)s_count;
+                    a.fresh[v] = 0;
+                    atomicAdd(a.stopped, 1ull);
+                } else {
+                    a.deg[v] = s_count;
+                    if (a.min_done) atomicMin(a.min_done, (unsigned long long)s_count);
+                    atomicAdd(a.updates, 1ull);
+                }
+                my_bytes += 4ull;
+            }
+        }
+        __syncthreads();
+    }
+    for (int off = 16; off > 0; off >>= 1) my_bytes += __shfl_down_sync(kFull, my_bytes, off);
+    if (lane == 0 && my_bytes) atomicAdd(a.bytes, my_bytes);
+}
+
 constexpr int kWarpRowX = 2048;   // longer rows are done by the whole block
 constexpr int kBlockHeavyX = 64;
 
@@ -670,6 +834,9 @@ int launch_hdeg(Graph& g, const int* worklist, const int* d_count, int64_t count
     void (*kern)(BfsArgs);
     if (cnt) kern = smem ? k_hdeg<true, true> : k_hdeg<true, false>;
     else kern = smem ? k_hdeg<false, true> : k_hdeg<false, false>;
+    // inside a round at h = 2 (a single graph): the queue-free kernel
+    const bool peel2 = round_ctr && smem && !cnt && !g.gid && g.h == 2;
+    if (peel2) kern = loss ? k_hdeg2_peel<true> : k_hdeg2_peel<false>;
     if (smem) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kSmemBitmapMax);
@@ -682,7 +849,7 @@ int launch_hdeg(Graph& g, const int* worklist, const int* d_count, int64_t count
     if (!smem && per_sm > 2) per_sm = 2;  // global bitmaps: bound the scratch
     int64_t work = worklist ? g.n : count_static;
     const int grid = pick_grid(g.ctx->sm_count, per_sm, work);
-    int rc = ensure_bfs_scratch(g, grid, !smem);
+    int rc = peel2 ? KH_OK : ensure_bfs_scratch(g, grid, !smem);
     if (rc) return rc;
     BfsArgs a{};
     a.rowptr = g.rowptr;
