@@ -346,6 +346,7 @@ static int set_M(Graph& g, int64_t M) {
     return KH_OK;
 }
 
+// A result to the caller (host results are written when this returns).
 static int copy_out(Graph& g, void* dst, const void* src, size_t bytes, uint32_t flags) {
     cudaStream_t s = g.ctx->stream;
     if (bytes == 0) return KH_OK;
@@ -356,12 +357,38 @@ static int copy_out(Graph& g, void* dst, const void* src, size_t bytes, uint32_t
     return KH_OK;
 }
 
-static int finish_check(Graph& g) {
-    int err = 0;
+struct Result {
+    void* dst;  // nullptr: not wanted
+    const void* src;
+    size_t bytes;
+};
+
+// Several results and the device error word with one wait.  Small host results
+// go through the context's pinned memory: a copy to pageable memory waits by
+// itself, 8 us each on a call of 100 us.
+static int copy_out_checked(Graph& g, const Result* r, int count, uint32_t flags) {
     cudaStream_t s = g.ctx->stream;
-    KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&err, &g.state->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    kh_pinned* pin = g.ctx->pinned;
+    size_t total = 0;
+    for (int i = 0; i < count; ++i)
+        if (r[i].dst) total += r[i].bytes;
+    const bool dev = (flags & KH_DEVICE_PTR) != 0, staged = !dev && total <= sizeof(pin->stage);
+    KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&pin->err, &g.state->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    size_t at = 0;
+    for (int i = 0; i < count; ++i) {
+        if (!r[i].dst || r[i].bytes == 0) continue;
+        KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(staged ? pin->stage + at : r[i].dst, r[i].src, r[i].bytes,
+                                           dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+        at += r[i].bytes;
+    }
     KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
-    if (err) return set_error(g.ctx, KH_EINTERNAL, "device check failed (flags 0x%x)", err);
+    if (pin->err) return set_error(g.ctx, KH_EINTERNAL, "device check failed (flags 0x%x)", pin->err);
+    at = 0;
+    for (int i = 0; staged && i < count; ++i) {
+        if (!r[i].dst || r[i].bytes == 0) continue;
+        memcpy(r[i].dst, pin->stage + at, r[i].bytes);
+        at += r[i].bytes;
+    }
     return KH_OK;
 }
 
@@ -370,7 +397,7 @@ static void free_ctx_objects(kh_ctx* c) {
         if (ev) cudaEventDestroy(ev);
     if (c->side) cudaStreamDestroy(c->side);
     if (c->own_stream) cudaStreamDestroy(c->stream);
-    if (c->peel_state) cudaFreeHost(c->peel_state);
+    if (c->pinned) cudaFreeHost(c->pinned);
 }
 
 }  // namespace kh
@@ -399,7 +426,7 @@ int kh_ctx_create(kh_ctx** out, int device, void* cuda_stream) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
     for (cudaEvent_t* ev : {&c->fork, &c->join, &c->peel_done[0], &c->peel_done[1]})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMallocHost(&c->peel_state, 2 * sizeof(kh::DevState));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->pinned, sizeof(kh_pinned));
     if (e != cudaSuccess) {
         kh::free_ctx_objects(c);
         free(c);
@@ -732,9 +759,9 @@ int kh_hdegree_exact(kh_graph* G, int32_t* deg, uint32_t flags) {
     rc = kh::run_hdeg_full(g, g.d32, nullptr, 0, 0, s);
     if (rc) return rc;
     KH_CUDA_TRY(g.ctx, cudaGetLastError());
-    rc = kh::copy_out(g, deg, g.d32, sizeof(int32_t) * (size_t)g.n, flags);
-    if (rc) return rc;
-    return (flags & KH_DEVICE_PTR) ? KH_OK : kh::finish_check(g);
+    if (flags & KH_DEVICE_PTR) return kh::copy_out(g, deg, g.d32, sizeof(int32_t) * (size_t)g.n, flags);
+    const kh::Result out{deg, g.d32, sizeof(int32_t) * (size_t)g.n};
+    return kh::copy_out_checked(g, &out, 1, flags);
 }
 
 int kh_sampled_counts(kh_graph* G, int32_t j_lo, int32_t j_hi, int32_t* cnt, uint32_t flags) {
@@ -761,13 +788,14 @@ int kh_sampled_counts(kh_graph* G, int32_t j_lo, int32_t j_hi, int32_t* cnt, uin
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.alive, 1, (size_t)g.n, s));
     KH_CUDA_TRY(g.ctx, cudaMemsetAsync(g.deadbm, 0, ((size_t)(g.n + 127) / 128) * 16, s));
     rc = kh::run_hdeg_full(g, g.d32, dcnt, j_lo, nj, s);
-    if (rc == KH_OK && !(flags & KH_DEVICE_PTR) && g.n > 0) {
-        rc = kh::copy_out(g, cnt, dcnt, sizeof(int32_t) * (size_t)g.n * nj, 0);
+    if (rc == KH_OK && !(flags & KH_DEVICE_PTR)) {
+        const kh::Result out{cnt, dcnt, sizeof(int32_t) * (size_t)g.n * nj};
+        rc = kh::copy_out_checked(g, &out, 1, 0);
     }
     if (dcnt && !(flags & KH_DEVICE_PTR)) cudaFreeAsync(dcnt, s);
     if (rc) return rc;
     KH_CUDA_TRY(g.ctx, cudaGetLastError());
-    return (flags & KH_DEVICE_PTR) ? KH_OK : kh::finish_check(g);
+    return KH_OK;
 }
 
 int kh_estimate(kh_graph* G, uint64_t* est, uint8_t* level, int32_t* bsize, uint32_t flags) {
@@ -782,10 +810,10 @@ int kh_estimate(kh_graph* G, uint64_t* est, uint8_t* level, int32_t* bsize, uint
     int32_t* bs_tmp = g.listA;
     kh::launch_gather_last(g, lvl_tmp, bs_tmp, g.ctx->stream);
     KH_CUDA_TRY(g.ctx, cudaGetLastError());
-    rc = kh::copy_out(g, est, g.d64, sizeof(uint64_t) * (size_t)g.n, flags);
-    if (!rc && level) rc = kh::copy_out(g, level, lvl_tmp, (size_t)g.n, flags);
-    if (!rc && bsize) rc = kh::copy_out(g, bsize, bs_tmp, sizeof(int32_t) * (size_t)g.n, flags);
-    return rc;
+    const kh::Result out[3] = {{est, g.d64, sizeof(uint64_t) * (size_t)g.n},
+                               {level, lvl_tmp, (size_t)g.n},
+                               {bsize, bs_tmp, sizeof(int32_t) * (size_t)g.n}};
+    return kh::copy_out_checked(g, out, 3, flags);
 }
 
 int kh_core_exact(kh_graph* G, int32_t* core, uint32_t flags) {

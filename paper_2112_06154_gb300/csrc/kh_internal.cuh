@@ -250,9 +250,15 @@ int run_core(Graph& g, bool sampled, void* out_core, int32_t* round_of_host, boo
 // the sum of d over the alive set (host outputs)
 int run_dense(Graph& g, bool sampled, const int32_t* round_of, int32_t rounds, uint64_t* sum,
               int64_t* size, int32_t* best);
-int run_estimate_all(Graph& g);
+int run_estimate_all(Graph& g);  // enqueued; the caller checks state->err
 
 }  // namespace kh
+
+struct kh_pinned {
+    kh::DevState states[2];    // the device state after the last two replays of a peel
+    int err;
+    uint8_t stage[256 * 1024]; // small results on their way to the caller
+};
 
 struct kh_ctx {
     int device;
@@ -264,7 +270,7 @@ struct kh_ctx {
     // `stream` by the two events)
     cudaStream_t side;
     cudaEvent_t fork, join;
-    void* peel_state;          // pinned: the device state after the last two replays of a peel
+    struct kh_pinned* pinned;  // pinned host memory of the context
     cudaEvent_t peel_done[2];
     // fault injection on the host: the fail_alloc_at-th device allocation from
     // the arming call fails with KH_ENOMEM (0: off)

@@ -809,10 +809,6 @@ int run_estimate_all(Graph& g) {
     for (int i = 1; i <= g.hmax && rc == KH_OK; ++i)
         rc = launch_level(g, i, nullptr, nullptr, g.n, 0, s, 0, 0);
     if (rc) return rc;
-    int err = 0;
-    KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&err, &g.state->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
-    if (err) return set_error(g.ctx, KH_EINTERNAL, "device check failed (flags 0x%x)", err);
     return KH_OK;
 }
 
@@ -897,7 +893,7 @@ int run_core(Graph& g, bool sampled, void* out_core, int32_t* round_of_host, boo
     // before it is looked at, so that the device does not wait for the host (12 to
     // 20 us per 8 rounds), unless the replay looked at last says that this one
     // ends the peel (an idle replay costs about as much).
-    DevState* states = static_cast<DevState*>(g.ctx->peel_state);
+    DevState* states = g.ctx->pinned->states;
     auto replay = [&](int slot) -> int {
         NvtxRange nvtx_range(use_graph ? "peel rounds (graph replay)" : "peel round");
         if (use_graph) {
