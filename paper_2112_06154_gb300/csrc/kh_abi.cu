@@ -651,7 +651,7 @@ int kh_footprint(int64_t n, int64_t nnz, int32_t h, int64_t M_or_0, double eps, 
     // level lists 1..h-1 (cap words per node and level), meta words of 1..h,
     // change ranks, positions and their class tables, the union's stage slots
     b += (int64_t)(h - 1) * n * cap * 4 + (int64_t)h * n * 4 + n + 4 * n + n / 32 + 1024 +
-         (int64_t)12 * 160 * cap * 4;
+         (int64_t)2 * 12 * 160 * cap * 4;
     // split parts of heavy nodes: at most nnz / 409 slots (ceil(deg/512) <=
     // deg/409 for deg > 2048), each cap keys plus counters
     const int64_t parts = nnz / 409;

@@ -127,6 +127,47 @@ __device__ __forceinline__ void end_round(const RoundEnd& r) {
 #endif
 RoundEnd round_end(const Graph& g);
 
+// Level unions split nodes of more than kSplitDeg neighbours into parts of
+// kSplitChunk neighbours each.  One CTA reads 2048 lists in about 40 us, as long
+// as a whole launch of a middle round; below that the parts' own set-up costs
+// more than the shorter tail gives (sampled (k,3)-cores of Chung-Lu n = 200k /
+// R-MAT 18: 688 / 311 ms with 4096 and 2048, 659 / 297 ms with 2048 and 512).
+constexpr int kSplitDeg = 2048;
+constexpr int kSplitChunk = 512;
+
+// Part slots and items of one union pass.  Whoever lists the nodes of the pass
+// hands the heavy ones to their parts instead, so that the parts can run beside
+// the other nodes.
+struct PartPlan {
+    int* n_sub;           // items planned
+    int32_t *sub_v, *sub_j;
+    int32_t* split_first; // a heavy node's first slot
+    int64_t cap;          // slots (0: the graph has no heavy node)
+    int* err;
+};
+#ifdef __CUDACC__
+// Plan v's parts if it is heavy (one thread); false: not heavy.
+__device__ __forceinline__ bool plan_parts(const PartPlan& p, int v, int64_t deg) {
+    if (p.cap == 0 || deg <= kSplitDeg) return false;
+    const int P = (int)((deg + kSplitChunk - 1) / kSplitChunk);
+    const int base = atomicAdd(p.n_sub, P);
+    if ((int64_t)base + P <= p.cap) {
+        for (int j = 0; j < P; ++j) {
+            p.sub_v[base + j] = v;
+            p.sub_j[base + j] = j;
+        }
+        p.split_first[v] = base;
+    } else {
+        // cannot happen: cap covers every heavy node of the graph at once
+        for (int64_t j = base; j < p.cap && j < (int64_t)base + P; ++j) p.sub_v[j] = -1;
+        atomicOr(p.err, kErrList);
+    }
+    return true;
+}
+#endif
+// the plan whose items level `level` of a round computes (0: the refine)
+PartPlan round_parts(const Graph& g, int level);
+
 // The lazy refine decides whether d(v) <= T = max(c, U) and may stop once a
 // partial value (a lower bound of d(v)) exceeds it.  It runs on until the
 // partial value exceeds kStopSlack * T instead: the node's new lower bound then

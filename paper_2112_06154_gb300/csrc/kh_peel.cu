@@ -239,7 +239,8 @@ template <typename T>
 __global__ void k_collect(const uint8_t* __restrict__ alive, uint8_t* __restrict__ fresh, int64_t n,
                           const int32_t* __restrict__ vl, LbArgs a, const T* __restrict__ d,
                           int keep_all, DevState* st, PeelState p, int32_t* __restrict__ out, int advance,
-                          int stop) {
+                          int stop, PartPlan plan, const int64_t* __restrict__ rowptr,
+                          const uint8_t* __restrict__ hv) {
     if (advance && blockIdx.x == 0 && threadIdx.x == 0) {
         if (st->n_alive != 0) {
             const int left = st->n_alive_next;
@@ -266,14 +267,15 @@ __global__ void k_collect(const uint8_t* __restrict__ alive, uint8_t* __restrict
                 due = lower_bound(a, (int)v) <= T;
             }
         }
+        if (due) fresh[v] = 1;
+        // a heavy node of a union goes to its parts
+        if (due && plan.cap > 0 && (!hv || hv[v] >= 2))
+            due = !plan_parts(plan, (int)v, rowptr[v + 1] - rowptr[v]);
         const uint32_t m = __ballot_sync(kFull, due);
         int base = 0;
         if (lane == 0 && m) base = atomicAdd(&st->nQ, __popc(m));
         base = __shfl_sync(kFull, base, 0);
-        if (due) {
-            out[base + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
-            fresh[v] = 1;
-        }
+        if (due) out[base + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
     }
 }
 
@@ -632,12 +634,12 @@ int refine(Graph& g, bool sampled, cudaStream_t s, bool advance) {
     if (sampled)
         k_collect<unsigned long long><<<grid, kPeelThreads, 0, s>>>(
             g.alive, g.fresh, g.vcount, g.vlist, la, g.d64, g.dense ? 1 : 0, g.state, peel_state(g, sampled), g.listB,
-            advance ? 1 : 0, 0);
+            advance ? 1 : 0, 0, g.hmax >= 2 ? round_parts(g, 0) : PartPlan{}, g.rowptr, g.hv);
     else
         k_collect<int32_t><<<grid, kPeelThreads, 0, s>>>(g.alive, g.fresh, g.vcount, g.vlist, la,
                                                          g.d32, g.dense ? 1 : 0, g.state,
                                                          peel_state(g, sampled), g.listB,
-            advance ? 1 : 0, g.dense ? 0 : 1);
+            advance ? 1 : 0, g.dense ? 0 : 1, PartPlan{}, g.rowptr, g.hv);
     count_launch(g, 1);
     prof_end(g, kProfPeel, s);
     if (sampled) return launch_level(g, g.h, g.listB, &g.state->nQ, 0, 0, s, 2);

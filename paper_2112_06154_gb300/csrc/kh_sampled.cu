@@ -115,30 +115,17 @@ struct LevelArgs {
     int8_t* rho;  // tracked passes: top rank of each changed list's changes
     unsigned long long* min_done;  // refine: per-graph minimum of the completed values
     // split heavy nodes (k_levelU): partial sets of cap words per part slot,
-    // their meta words, parts finished per split node (at its first slot),
-    // each heavy node's first slot, the part items (part_cap 0: no split)
+    // their meta words, parts finished per split node (at its first slot)
     uint32_t* part_keys;
     uint32_t* part_meta;
     int32_t* part_done;
     int32_t* part_stop;             // per split node: some part stopped early (refine)
     unsigned long long* part_lb;    // per split node: the largest partial estimate above T
-    int32_t* split_first;
-    int32_t* sub_v;
-    int32_t* sub_j;
-    int* n_sub;
-    int64_t part_cap;
+    PartPlan plan;
 };
 
 constexpr int kL1Heavy = 512;
 constexpr int kL1BlockHeavy = 64;
-// k_levelU splits nodes of more than kSplitDeg neighbours into parts of
-// kSplitChunk neighbours each.  One CTA reads 2048 lists in about 40 us, as long
-// as a whole launch of a middle round; below that the parts' own set-up costs
-// more than the shorter tail gives (sampled (k,3)-cores of Chung-Lu n = 200k /
-// R-MAT 18: 688 / 311 ms with 4096 and 2048, 659 / 297 ms with 2048 and 512).
-constexpr int kSplitDeg = 2048;
-constexpr int kSplitChunk = 512;
-
 // What one node computes in this launch: its level, whether that is its last
 // level h(v) (estimate) or an intermediate one (list), its M, and where its
 // inputs (level - 1) and outputs live.
@@ -809,23 +796,6 @@ __device__ __forceinline__ int lost_rank(const LevelArgs& a, const UnionShared& 
     return r;
 }
 
-// Give a heavy node its part slots and part items (one thread).
-__device__ __forceinline__ void plan_parts(const LevelArgs& a, int v, int deg) {
-    const int P = (deg + kSplitChunk - 1) / kSplitChunk;
-    const int base = atomicAdd(a.n_sub, P);
-    if ((int64_t)base + P <= a.part_cap) {
-        for (int j = 0; j < P; ++j) {
-            a.sub_v[base + j] = v;
-            a.sub_j[base + j] = j;
-        }
-        a.split_first[v] = base;
-    } else {
-        // cannot happen: part_cap covers every heavy node of the graph at once
-        for (int64_t j = base; j < a.part_cap && j < (int64_t)base + P; ++j) a.sub_v[j] = -1;
-        atomicOr(a.err, kErrList);
-    }
-}
-
 // Levels >= 2, one CTA of 128 threads per node.
 //
 // The set of distinct members is a bitmap over positions in shared memory
@@ -865,7 +835,7 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
     extern __shared__ __align__(16) uint32_t tab[];
     __shared__ UnionShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t total = PARTS        ? min((int64_t)(*a.n_sub), a.part_cap)
+    const int64_t total = PARTS        ? min((int64_t)(*a.plan.n_sub), a.plan.cap)
                           : a.worklist ? (int64_t)(*a.d_count)
                                        : a.count_static;
     // the first items go by block index, so that a short list costs the other
@@ -877,7 +847,7 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
     for (int i = tid * 4; i < (1 << a.lg); i += kLuThreads * 4)
         *reinterpret_cast<uint4*>(tab + i) = make_uint4(0u, 0u, 0u, 0u);
     // the CTA's next item: a node, or (PARTS) a part of a split node
-    const int* items = PARTS ? a.sub_v : a.worklist;
+    const int* items = PARTS ? a.plan.sub_v : a.worklist;
     if (tid == 0) {
         sh.idx = blockIdx.x;
         sh.v = items ? items[blockIdx.x] : (int)blockIdx.x;
@@ -889,7 +859,7 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
         if (idx >= total) break;
         // mode 0: a whole node; 1: one part of a split node (2: its merge)
         int mode = PARTS ? 1 : 0;
-        const int v = sh.v, part = PARTS ? a.sub_j[idx] : 0;
+        const int v = sh.v, part = PARTS ? a.plan.sub_j[idx] : 0;
         int next = 0;
         if (tid == 0) next = (int)gridDim.x + atomicAdd(a.work_ctr, 1);
         bool skip = PARTS && v < 0;  // a part the plan could not place
@@ -905,10 +875,11 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
             kv = a.key32[v];
             g = a.gid ? a.gid[v] : 0;
             skip = a.alive[v] != 1 || nl.skip || nl.lvl < 2 || (!LIST && !nl.last) || (!LAST && nl.last);
-            if (!PARTS && !skip && a.part_cap > 0 && deg > kSplitDeg) {
-                // a heavy node is done in parts by the launch that follows
+            if (!PARTS && !skip && a.plan.cap > 0 && deg > kSplitDeg) {
+                // a heavy node is done in parts by the launch that follows (a round's
+                // lists hold none)
                 skip = true;
-                if (tid == 0) plan_parts(a, v, deg);
+                if (tid == 0) plan_parts(a.plan, v, deg);
             }
         }
         if (skip) {
@@ -921,7 +892,7 @@ __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
         }
         const int rv = (int)(kv >> kIdBits);
         const bool last = LAST && (!LIST || nl.last);
-        const int first = PARTS && mode ? a.split_first[v] : -1;
+        const int first = PARTS && mode ? a.plan.split_first[v] : -1;
         const int nparts = (deg + kSplitChunk - 1) / kSplitChunk;
         const uint8_t* wrank = a.wrank + (a.gid ? word_base(a.vtx_off[g], g) : 0);
         if (g != cls_graph) {
@@ -1203,6 +1174,7 @@ struct MarkArgs {
     const DevState* st;
     unsigned long long* bytes;
     RoundEnd end;          // phase 1: the round's c and minima advance here
+    PartPlan plan;         // heavy nodes that would be listed
     // STALE: nodes whose last level is `phase` become stale instead of listed
     uint32_t* meta_last;   // = meta, writable
     const uint32_t* prev;  // meta words of level phase - 1 (nullptr at phase 1)
@@ -1299,6 +1271,8 @@ __device__ __forceinline__ void mark_step(const MarkArgs& a, int rw, int stamp, 
             make_stale(a, u[q], m[q]);
             go[q] = false;
         }
+        if (go[q] && a.plan.cap > 0)
+            go[q] = !plan_parts(a.plan, u[q], a.rowptr[u[q] + 1] - a.rowptr[u[q]]);
         isnew[q] = __ballot_sync(kFull, go[q]);
         n += __popc(isnew[q]);
     }
@@ -1539,7 +1513,7 @@ int ensure_positions(Graph& g) {
         return rc;
     if (!g.wrank && (rc = alloc_bytes(g.ctx, (void**)&g.wrank, (size_t)word_base(g.n, ng) + 4, "word ranks")))
         return rc;
-    // compaction stage of the hash form, one slot per CTA of k_levelU
+    // compaction stage of the hash form, one slot per CTA of k_levelU (nodes; parts)
     if (g.lu_stage && g.lu_stage_cap < g.cap) {
         KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
         cudaFree(g.lu_stage);
@@ -1547,7 +1521,7 @@ int ensure_positions(Graph& g) {
     }
     if (!g.lu_stage) {
         if ((rc = alloc_bytes(g.ctx, (void**)&g.lu_stage,
-                              sizeof(uint32_t) * (size_t)g.ctx->sm_count * kLuPerSm * (size_t)g.cap, "union stage")))
+                              sizeof(uint32_t) * 2 * (size_t)g.ctx->sm_count * kLuPerSm * (size_t)g.cap, "union stage")))
             return rc;
         g.lu_stage_cap = g.cap;
     }
@@ -1613,28 +1587,25 @@ int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
     if (round_mode == 1) {
         a.n_changed = rc + kRcC + level;
         a.work_ctr = rc + kRcLevelWork + level;
-        a.n_sub = rc + kRcSub + level;
         sub_ctr = rc + kRcSubWork + level;
+        a.plan = round_parts(g, level);
     } else if (round_mode == 2) {
         a.n_changed = rc + kRcC + 0;  // unused: the refine does not track changes
         a.work_ctr = rc + kRcRefineWork;
-        a.n_sub = rc + kRcSub + 0;
         sub_ctr = rc + kRcSubWork + 0;
+        a.plan = round_parts(g, 0);
     } else {
         a.n_changed = &g.state->nC[level & 1];
         a.work_ctr = &g.state->work_ctr[1];
-        a.n_sub = &g.state->nSub;
+        a.plan = round_parts(g, 0);
+        a.plan.n_sub = &g.state->nSub;
         sub_ctr = &g.state->work_ctr[3];
     }
-    a.part_cap = g.part_cap;
     a.part_keys = g.part_keys;
     a.part_meta = g.part_meta;
     a.part_done = g.part_done;
     a.part_stop = g.part_stop;
     a.part_lb = g.part_lb;
-    a.split_first = g.split_first;
-    a.sub_v = g.sub_v;
-    a.sub_j = g.sub_j;
     cudaError_t e;
     if (track && round_mode == 0) {
         e = cudaMemsetAsync(a.n_changed, 0, sizeof(int), s);
@@ -1692,21 +1663,39 @@ int launch_level(Graph& g, int level, const int* worklist, const int* d_count,
         e = cudaMemsetAsync(a.work_ctr, 0, sizeof(int), s);
         if (e != cudaSuccess) return check_cuda(g.ctx, e, "memset work_ctr");
         if (parts) {
-            e = cudaMemsetAsync(a.n_sub, 0, sizeof(int), s);
+            e = cudaMemsetAsync(a.plan.n_sub, 0, sizeof(int), s);
             if (e == cudaSuccess) e = cudaMemsetAsync(sub_ctr, 0, sizeof(int), s);
             if (e != cudaSuccess) return check_cuda(g.ctx, e, "memset n_sub");
         }
     }
     prof_begin(g, kProfLevelU, s);
+    if (parts && round_mode != 0) {
+        // planned by the kernel that made the list: beside the other nodes
+        LevelArgs pa = a;
+        pa.work_ctr = sub_ctr;
+        pa.stage = g.lu_stage + (size_t)g.ctx->sm_count * kLuPerSm * (size_t)g.cap;
+        KH_CUDA_TRY(g.ctx, cudaEventRecord(g.ctx->fork, s));
+        KH_CUDA_TRY(g.ctx, cudaStreamWaitEvent(g.ctx->side, g.ctx->fork, 0));
+        pkern<<<g.ctx->sm_count * per_sm, kLuThreads, dyn, g.ctx->side>>>(pa);
+        KH_CUDA_TRY(g.ctx, cudaEventRecord(g.ctx->join, g.ctx->side));
+        a.plan.cap = 0;  // no heavy node in the list
+    }
     kern<<<(int)grid, kLuThreads, dyn, s>>>(a);
     count_launch(g, 1);
-    if (parts) {
+    if (parts && round_mode != 0) {
+        KH_CUDA_TRY(g.ctx, cudaStreamWaitEvent(s, g.ctx->join, 0));
+        count_launch(g, 1);
+    } else if (parts) {
         a.work_ctr = sub_ctr;
         pkern<<<g.ctx->sm_count * per_sm, kLuThreads, dyn, s>>>(a);
         count_launch(g, 1);
     }
     prof_end(g, kProfLevelU, s);
     return KH_OK;
+}
+
+PartPlan round_parts(const Graph& g, int level) {
+    return {g.state->rc + kRcSub + level, g.sub_v, g.sub_j, g.split_first, g.part_cap, &g.state->err};
 }
 
 static MarkArgs mark_args(Graph& g, int phase) {
@@ -1742,6 +1731,7 @@ void launch_mark_neighbours(Graph& g, const int* list1, const int* cnt1, const i
     a.wl = g.listW;
     a.nwl = out_count;
     if (phase == 1) a.end = round_end(g);
+    if (phase >= 2) a.plan = round_parts(g, phase);  // (level 1 is not a union)
     const int grid = g.ctx->sm_count * 8;
     prof_begin(g, kProfFrontier, s);
     if (phase >= g.hmin) k_mark_nbrs<true><<<grid, 256, 0, s>>>(a);
