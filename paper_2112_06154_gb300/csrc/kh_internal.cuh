@@ -128,11 +128,15 @@ __device__ __forceinline__ void end_round(const RoundEnd& r) {
 RoundEnd round_end(const Graph& g);
 
 // Level unions split nodes of more than kSplitDeg neighbours into parts of
-// kSplitChunk neighbours each.  One CTA reads 2048 lists in about 40 us, as long
-// as a whole launch of a middle round; below that the parts' own set-up costs
-// more than the shorter tail gives (sampled (k,3)-cores of Chung-Lu n = 200k /
-// R-MAT 18: 688 / 311 ms with 4096 and 2048, 659 / 297 ms with 2048 and 512).
-constexpr int kSplitDeg = 2048;
+// kSplitChunk neighbours each, on graphs with a node of more than kSplitMin.  One
+// CTA reads 1024 lists in about 20 us, as long as a whole launch of a middle
+// round; below that the parts' own set-up costs more than the shorter tail
+// gives (sampled (k,3)-cores of Chung-Lu n = 200k / R-MAT 18: 513 / 216 ms from
+// 2048 on, 502 / 206 from 1024, 497 / 264 from 512 with parts of 256).  Without a
+// really heavy node the launch of the parts costs more than it gives ((k,2)-core
+// of Chung-Lu n = 50k, largest degree 1250: 328 -> 335 ms).
+constexpr int kSplitMin = 2048;
+constexpr int kSplitDeg = 1024;
 constexpr int kSplitChunk = 512;
 
 // Part slots and items of one union pass.  Whoever lists the nodes of the pass

@@ -1360,17 +1360,22 @@ __global__ void k_stale_all(MarkArgs a, int64_t n, const uint8_t* __restrict__ a
 
 namespace {
 // Part slots a whole-graph level pass needs: ceil(deg / kSplitChunk) per node
-// of degree above kSplitDeg.
+// of degree above kSplitDeg (out[0]); the nodes above kSplitMin (out[1]).
 __global__ void k_count_parts(const int64_t* __restrict__ rowptr, int64_t n,
                               unsigned long long* out) {
-    unsigned long long c = 0;
+    unsigned long long c = 0, big = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const int64_t deg = rowptr[v + 1] - rowptr[v];
         if (deg > kSplitDeg) c += (unsigned long long)((deg + kSplitChunk - 1) / kSplitChunk);
+        big += deg > kSplitMin;
     }
-    for (int off = 16; off > 0; off >>= 1) c += __shfl_down_sync(kFull, c, off);
+    for (int off = 16; off > 0; off >>= 1) {
+        c += __shfl_down_sync(kFull, c, off);
+        big += __shfl_down_sync(kFull, big, off);
+    }
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
+    if ((threadIdx.x & 31) == 0 && big) atomicAdd(out + 1, big);
 }
 }  // namespace
 
@@ -1378,18 +1383,18 @@ int ensure_split(Graph& g) {
     cudaStream_t s = g.ctx->stream;
     if (!g.split_planned) {
         unsigned long long* d = nullptr;
-        unsigned long long parts = 0;
-        KH_CUDA_TRY(g.ctx, cudaMallocAsync((void**)&d, sizeof(unsigned long long), s));
-        cudaError_t e = cudaMemsetAsync(d, 0, sizeof(unsigned long long), s);
+        unsigned long long parts[2] = {0, 0};
+        KH_CUDA_TRY(g.ctx, cudaMallocAsync((void**)&d, sizeof(parts), s));
+        cudaError_t e = cudaMemsetAsync(d, 0, sizeof(parts), s);
         if (e == cudaSuccess && g.n > 0) {
             k_count_parts<<<g.ctx->sm_count * 4, 256, 0, s>>>(g.rowptr, g.n, d);
             count_launch(g, 1);
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&parts, d, sizeof(parts), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(parts, d, sizeof(parts), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         cudaFreeAsync(d, s);
         if (e != cudaSuccess) return check_cuda(g.ctx, e, "count split parts");
-        g.part_cap = (int64_t)parts;
+        g.part_cap = parts[1] ? (int64_t)parts[0] : 0;
         g.split_planned = true;
     }
     if (g.part_cap == 0) return KH_OK;
