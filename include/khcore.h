@@ -308,7 +308,7 @@ int kh_hdegree_exact_noalloc(int64_t n, const int64_t *rowptr, const int32_t *co
 #define KH_LEVELU_FREE 2
 #define KH_LEVELU_GROUPED 3
 /* KH_OP_HDEG2_SWEEP: the whole-graph exact 2-degrees (kh_hdegree_exact at
- * h = 2 with a sliced layout) may hand the sources of largest 2-hop work
+ * h = 2, any layout) may hand the sources of largest 2-hop work
  * (sum of their neighbours' degrees) to bit-parallel sweeps: one pass over
  * every row per batch of 1024 sources, with 1024-bit source masks per node.
  * KH_VAR_AUTO: the tuner decides the threshold; KH_SWEEP_OFF: never;

@@ -1,5 +1,7 @@
-// kh_hdeg2.cu -- exact 2-degrees of a whole graph with sliced shared-memory
-// visited sets (graphs whose n-bit visited set does not fit in shared memory).
+// kh_hdeg2.cu -- exact 2-degrees of a whole graph: sliced shared-memory visited
+// sets (k_hdeg2_slice, graphs whose n-bit visited set does not fit in shared
+// memory), one CTA per source where it does (k_hdeg2_cta), and bit-parallel
+// searches of many sources (k_sweep_*).
 //
 // Sec. 2: deg_2(v) = |N(v; 2)| - 1 with N(v; 2) = {v} U A(v) U (U_{w in A(v)} A(w)).
 // For a node with at least one neighbour, v itself lies in A(w) for every w in

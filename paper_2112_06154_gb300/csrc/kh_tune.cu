@@ -12,14 +12,14 @@
 //                  k_hdeg2_small (a warp and a private hash set per source)
 //                  for the rest.
 // The sliced kernel has two launch parameters: the number of slices S (at
-// least what shared memory requires) and the CTA size.  With a sliced layout
+// least what shared memory requires) and the CTA size.  With every layout
 // the sources of the largest 2-hop work may go to the bit-parallel sweeps
 // (k_sweep_*: 1024 sources per pass over the rows), from a work threshold.
 // The tuner times every layout candidate on the same sample of sources (every
 // k-th source of the longest-first order, so every size class is represented)
 // with CUDA events on the context stream, keeps the fastest, then prices the
-// sweep thresholds (sweeps times a measured sweep, plus the sliced layout on
-// the rest of the sample), and records the choice in a table keyed by the
+// sweep thresholds (sweeps times a measured sweep, plus the layout on the
+// rest of the sample), and records the choice in a table keyed by the
 // graph's shape class (device SMs, log2 n, log2 nnz, log2 of max degree / mean
 // degree).  With the environment variable KH_TUNE_FILE set, the table is read
 // from and appended to that text file, so a later process on a graph of the
@@ -411,8 +411,8 @@ static int choose_deep(Graph& g, cudaStream_t s, bool* batches) {
         g.hdeg_deep[g.h] = per * (double)g.n > pulls((double)g.n) ? 2 : 1;
     }
     if (g.hdeg_deep[g.h] != 2) return KH_OK;
-    if ((rc = ensure_order2(g, s))) return rc;
-    *batches = ensure_sweep(g, g.h, s) == KH_OK;  // (no memory for the masks: a search per source)
+    // (no memory for the order or the masks: a search per source)
+    *batches = ensure_order2(g, s) == KH_OK && ensure_sweep(g, g.h, s) == KH_OK;
     return KH_OK;
 }
 
@@ -427,6 +427,9 @@ int run_hdeg_full(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStr
         {
             rc = ensure_order2(g, s);
             if (rc) return rc;
+            // (no memory for the ranks of the row entries: counts by the search kernel)
+            if (cnt && c.variant == KH_VAR_CTA && ensure_crank(g, s) != KH_OK)
+                return launch_hdeg(g, nullptr, nullptr, g.n, deg, cnt, jlo, nj, s);
             // the sources of largest 2-hop work go to the bit-parallel sweeps
             // (2-degrees only: the sweeps do not count by rank)
             int bin = g.sw_force != 0 ? g.sw_force : c.sweep_bin;

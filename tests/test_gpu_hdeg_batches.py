@@ -61,3 +61,26 @@ def test_small_balls_keep_the_search(ctx):
         assert K.kh_launch_count(G) - before == 1
     finally:
         G.close()
+
+
+def test_no_memory_for_masks_or_entry_ranks(ctx):
+    """The passes that need extra arrays fall back on the search per source."""
+    rp, cl = GRAPHS["cl5k"]()
+    G = K.kh_graph_load_csr(ctx, rp, cl)
+    try:
+        for h in (3, 4):
+            K.kh_set_h(G, h)
+            if h == 4:
+                K.kh_debug_fail_alloc(ctx, 1)  # h = 3 has all but the third mask array
+            assert np.array_equal(K.kh_hdegree_exact(G), O.hdegree_exact(rp, cl, h))
+        K.kh_debug_fail_alloc(ctx, 0)
+        assert np.array_equal(K.kh_hdegree_exact(G), O.hdegree_exact(rp, cl, 4))
+        K.kh_set_h(G, 2)
+        want = O.hdegree_exact(rp, cl, 2)
+        K.kh_debug_fail_alloc(ctx, 1)  # the ranks of the row entries
+        assert np.array_equal(K.kh_sampled_counts(G, 0, 3)[:, 0], want)
+        K.kh_debug_fail_alloc(ctx, 0)
+        assert np.array_equal(K.kh_sampled_counts(G, 0, 3)[:, 0], want)
+    finally:
+        K.kh_debug_fail_alloc(ctx, 0)
+        G.close()
