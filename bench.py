@@ -46,11 +46,11 @@ E2E_STEPS = 3  # end-to-end steps (graph upload included), capped to keep the ru
 
 # kernel class -> the kernels it brackets (kh_prof_read kinds)
 CLASS_KERNELS = {
-    "bfs": "k_hdeg, k_hdeg2_slice, k_hdeg2_small, k_sweep_* (exact h-degrees)",
-    "level1": "k_level1, k_level1_heavy (level-1 lists)",
-    "levelU": "k_levelU (level >= 2 lists, hashed union with trim)",
+    "bfs": "k_hdeg, k_hdeg2_peel, k_hdeg2_cta, k_hdeg2_slice, k_hdeg2_small, k_sweep_* (exact h-degrees)",
+    "level1": "k_level1 (level-1 lists)",
+    "levelU": "k_levelU (level >= 2 lists, bitmap or hashed union with trim)",
     "frontier": "k_mark_nbrs, k_ball_hop, k_stale_*, k_apply_loss",
-    "peel": "k_min_alive, k_collect, k_select, k_finish",
+    "peel": "k_begin, k_collect, k_select",
 }
 
 

@@ -825,7 +825,10 @@ __device__ __forceinline__ int lost_rank(const LevelArgs& a, const UnionShared& 
 // would hold a bitmap of all 200k positions, with 8 CTAs.
 // Measured (start: one 256-thread CTA per node, hash set, 27 KB): estimates of
 // R-MAT 22 at h = 3 251 -> 78 ms, (k,3)-core of Chung-Lu n = 200k 1080 -> 659 ms,
-// (k,2)-core of Chung-Lu n = 50k at M = 1200 919 -> 538 ms.
+// (k,2)-core of Chung-Lu n = 50k at M = 1200 919 -> 538 ms (503 and 328 ms since the
+// marking is spread over the warps, rounds have fewer kernels and heavy nodes smaller
+// parts).  A warp per light node with a private quarter of the table gave nothing on
+// the estimates (79.9 ms) and cost 30% in the rounds.
 //
 // LAST: nodes at their last level (estimate, refine); LIST: nodes below it
 // (stored lists); PARTS: the parts of the split nodes, which the launch before
