@@ -20,6 +20,14 @@ namespace kh {
 namespace {
 
 constexpr int kBfsThreads = 256;
+// A peel round has a handful of sources, so at h >= 3 the length of its searches is
+// that of one CTA's: 512 threads where balls are large (mean degree of at least
+// kBfsWideDegree), (k,3)-core of Chung-Lu n = 20k 2103 -> 1554 ms, of R-MAT 13 466 -> 328,
+// (k,4)-core of G(20k, 60k) (mean degree 6) 131 -> 112.  On a grid (mean degree 4, balls of
+// 25 nodes) the wider barriers cost more than they give: 10.6 -> 11.1 ms.  1024 threads:
+// 1400, 283, 112 and 13.1 ms, but 295 against 273 on the (k,4)-core of R-MAT 13.
+constexpr int kBfsRoundThreads = 512;
+constexpr int kBfsWideDegree = 5;
 constexpr int kHeavyDeg = 128;
 constexpr int kMaxHeavy = 64;
 constexpr uint32_t kFull = 0xffffffffu;
@@ -218,7 +226,7 @@ __device__ __forceinline__ void expand_row(const BfsArgs& a, uint32_t* bm, int32
 }
 
 template <bool RANKS, bool SMEM, bool ALLALIVE = false>
-__global__ void __launch_bounds__(kBfsThreads) k_hdeg(BfsArgs a) {
+__global__ void __launch_bounds__(kBfsRoundThreads) k_hdeg(BfsArgs a) {
     extern __shared__ __align__(16) uint32_t s_bm_dyn[];
     __shared__ int s_src, s_qtail, s_count, s_nheavy, s_stop;
     __shared__ unsigned long long s_T;
@@ -842,8 +850,10 @@ int launch_hdeg(Graph& g, const int* worklist, const int* d_count, int64_t count
                                              (int)kSmemBitmapMax);
         if (e != cudaSuccess) return check_cuda(g.ctx, e, "cudaFuncSetAttribute(k_hdeg)");
     }
+    const bool wide = round_ctr && !g.gid && g.h >= 3 && g.nnz >= kBfsWideDegree * g.n;
+    const int threads = wide ? kBfsRoundThreads : kBfsThreads;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBfsThreads, dyn);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, dyn);
     if (e != cudaSuccess) return check_cuda(g.ctx, e, "occupancy(k_hdeg)");
     if (per_sm < 1) per_sm = 1;
     if (!smem && per_sm > 2) per_sm = 2;  // global bitmaps: bound the scratch
@@ -896,7 +906,7 @@ int launch_hdeg(Graph& g, const int* worklist, const int* d_count, int64_t count
         if (e != cudaSuccess) return check_cuda(g.ctx, e, "memset work_ctr");
     }
     prof_begin(g, kProfBfs, s);
-    kern<<<grid, kBfsThreads, dyn, s>>>(a);
+    kern<<<grid, threads, dyn, s>>>(a);
     count_launch(g, 1);
     prof_end(g, kProfBfs, s);
     return KH_OK;

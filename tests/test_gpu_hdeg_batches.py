@@ -84,3 +84,18 @@ def test_no_memory_for_masks_or_entry_ranks(ctx):
     finally:
         K.kh_debug_fail_alloc(ctx, 0)
         G.close()
+
+
+@pytest.mark.parametrize("h", [3, 4])
+@pytest.mark.parametrize("m", [1501, 1506, 3000])  # around a mean degree of 5
+def test_exact_cores_by_wide_searches(ctx, m, h):
+    rp, cl = gg.erdos_renyi(601, m, 8)
+    want, wround, steps = O.core_exact(rp, cl, h)
+    G = K.kh_graph_load_csr(ctx, rp, cl)
+    try:
+        K.kh_set_h(G, h)
+        assert np.array_equal(K.kh_core_exact(G), want)
+        ro, rounds, _ = K.kh_peel_info(G)
+        assert np.array_equal(ro, wround) and rounds == steps
+    finally:
+        G.close()
