@@ -531,7 +531,10 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
             li = -1;
             continue;
         }
-        const int t = *(volatile int*)&sh.t;
+        // the level likewise: other warps raise it, and the whole warp tests it below
+        int t = 0;
+        if (lane == 0) t = *(volatile int*)&sh.t;
+        t = __shfl_sync(kFull, t, 0);
         int ins = 0;
         bool done = false;
         if (li >= 0) {
@@ -608,12 +611,10 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
         const int S = snapshot_counts(sh.hist, lane);
         const uint32_t over = __ballot_sync(kFull, S > c.M);
         const int pmax = over ? 31 - __clz(over) : -1;
-        if (pmax + 1 > t) {
-            const int Sn = __shfl_sync(kFull, S, (pmax + 1) & 31);
-            if (lane == 0) {
-                atomicMax(&sh.t, pmax + 1);
-                *(volatile int*)&sh.tot = pmax < 31 ? Sn : 0;
-            }
+        const int Sn = __shfl_sync(kFull, S, (pmax + 1) & 31);
+        if (lane == 0 && pmax + 1 > t) {
+            atomicMax(&sh.t, pmax + 1);
+            *(volatile int*)&sh.tot = pmax < 31 ? Sn : 0;
         }
         if (LAST && c.can_stop) {
             // Def. 4.1 on the keys inserted so far plus v itself: a subset
