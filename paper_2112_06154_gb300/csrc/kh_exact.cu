@@ -482,8 +482,14 @@ __global__ void __launch_bounds__(kBfsThreads) k_hdeg2_peel(BfsArgs a) {
                     for (int p = 0; p < 4; ++p)
                         if (u[p] >= 0) visit2(u[p]);
                 }
-                if (can_stop) fold_count(my, &s_count, lane);
-                if (can_stop && (unsigned long long)*(volatile int*)&s_count > T) break;
+                if (can_stop) {
+                    fold_count(my, &s_count, lane);
+                    // one read for the whole warp: lanes that saw different counts
+                    // would part ways before the next collective
+                    int over = 0;
+                    if (lane == 0) over = (unsigned long long)*(volatile int*)&s_count > T;
+                    if (__shfl_sync(kFull, over, 0)) break;
+                }
             }
             int bk = 2, li = -1, pos = 0, n = 0;
             const int32_t* row = nullptr;

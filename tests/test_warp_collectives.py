@@ -147,7 +147,7 @@ def test_the_reading_finds_both_forms():
                         "t = *(volatile int*)s; if (__shfl_sync(kFull, t, 0)) break; } }")
 
 
-@pytest.mark.parametrize("name", ["kh_sampled.cu"])
+@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))))
 def test_no_collective_under_a_value_other_warps_change(name):
     with open(os.path.join(CSRC, name)) as f:
         assert findings(f.read()) == []
