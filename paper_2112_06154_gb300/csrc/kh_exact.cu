@@ -494,6 +494,10 @@ __global__ void __launch_bounds__(kBfsThreads) k_hdeg2_peel(BfsArgs a) {
             int bk = 2, li = -1, pos = 0, n = 0;
             const int32_t* row = nullptr;
             for (int step = 0;; ++step) {  // groups claim rows (walk_chunk of the level union)
+                if (step > row_steps(kBfsThreads)) {
+                    if (lane == 0) atomicOr(a.err, kErrLoop);
+                    break;
+                }
                 if (can_stop && (step & 3) == 3) {
                     // the visited set is a subset of the ball: past T the rest is not needed
                     fold_count(my, &s_count, lane);

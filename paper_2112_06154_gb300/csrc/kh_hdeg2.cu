@@ -350,6 +350,7 @@ struct Cta2Args {
     int32_t* cnt;
     int jlo, nj;
     int* work_ctr;
+    int* err;
     unsigned long long* updates;
     unsigned long long* bytes;
 };
@@ -443,7 +444,11 @@ __global__ void __launch_bounds__(kCtaMaxThreads) k_hdeg2_cta(Cta2Args a) {
             }
             int bk = 2, li = -1, pos = 0, n = 0;
             int64_t rb = 0;
-            for (;;) {  // as walk_chunk of the level union: groups claim rows
+            for (int step = 0;; ++step) {  // as walk_chunk of the level union: groups claim rows
+                if (step > row_steps(T)) {
+                    if (lane == 0) atomicOr(a.err, kErrLoop);
+                    break;
+                }
                 const int lgG = bk == 2 ? 5 : bk == 1 ? 3 : 1;
                 const int lead = lane >> lgG << lgG;
                 const uint32_t need = __ballot_sync(kFull, li == -1 && lane == lead);
@@ -1075,6 +1080,7 @@ int launch_hdeg2_cta(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cuda
     a.jlo = jlo;
     a.nj = nj;
     a.work_ctr = &g.state->work_ctr[large ? 3 : 2];
+    a.err = &g.state->err;
     a.updates = &g.state->updates;
     a.bytes = &g.state->bytes[kProfBfs];
     prof_begin(g, kProfBfs, s);

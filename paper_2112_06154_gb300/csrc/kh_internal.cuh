@@ -106,6 +106,12 @@ struct DevState {
 
 struct Graph;
 
+// The row readers of k_hdeg2_cta and k_hdeg2_peel: every step of a warp over a chunk
+// of `rows` rows of up to 511 entries reads one of them on (short and middle rows in
+// one step, the others 128 entries a step) or ends one of three buckets, so no
+// correct loop takes more steps than this; one that does ends with kErrLoop.
+constexpr int row_steps(int rows) { return 4 * rows + 4; }
+
 // After a round's removal set is chosen: c = max(c, the round's minimum) of every
 // graph, the minima back to none.  Done by one block of the first refresh kernel
 // (nothing else reads them before the next round).

@@ -436,6 +436,10 @@ constexpr int kKeysPerLane = 4;  // words one lane loads per step (one 16-byte v
 // ones (up to about 8 keys expected at or above t: 2 lanes a list), middle
 // (up to 64: 8 lanes), long (a warp a list) and dense (8 lanes).
 constexpr int kBuckets = 4;
+// Every step of a warp reads at least one of the chunk's lists on by 8 words (a
+// short one, by 2 lanes) or ends a bucket, so no correct walk takes more steps than
+// this; one that does ends the union with kErrLoop.
+constexpr int kWalkSteps = kLuThreads * (kMaxM / 8 + 2) + kBuckets;
 constexpr int kShort = 0, kMiddle = 1, kDense = 2, kLong = 3;
 
 // Shared state of one node's union.
@@ -499,7 +503,7 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
         sz = sh.sz[li];
     }
 #pragma unroll 1
-    for (;;) {
+    for (int step = 0; step < kWalkSteps; ++step) {
         // one read for the whole warp: lanes that saw a flag at different
         // moments would part ways before the ballots
         int stop = 0;
@@ -634,6 +638,10 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
                     atomicCAS(&sh.exit, 0, 2);
             }
         }
+    }
+    if (lane == 0) {
+        atomicOr(c.err, kErrLoop);
+        atomicCAS(&sh.exit, 0, 2);  // the other warps leave too
     }
 }
 
