@@ -79,6 +79,7 @@ constexpr int kRcLossWork = 88;    // exact refresh: loss-BFS work counter
 constexpr int kRcLossCount = 89;   // exact refresh: nodes with a loss this round
 constexpr int kRcSub = 90;         // + i: split-part items of level i (0: the refine)
 constexpr int kRcCount = 107;
+constexpr int kRoundKey = 21;      // what a captured batch of rounds holds (kh_peel.cu: round_graph)
 
 struct DevState {
     unsigned long long c;        // current core value (max of round minima)
@@ -489,7 +490,7 @@ struct Graph {
     std::vector<unsigned long long>* prof_btrace[kProfKinds];
     // cached CUDA graph of a batch of peeling rounds
     cudaGraphExec_t round_exec;
-    int round_exec_key[10];
+    int64_t round_exec_key[kRoundKey];
     int64_t round_exec_kernels;  // kernels in one replay of round_exec
     // kernels launched on behalf of this graph (graph replays count their nodes)
     int64_t launches;

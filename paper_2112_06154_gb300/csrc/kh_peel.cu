@@ -760,11 +760,14 @@ int check_state_err(Graph& g, const DevState& hs) {
 
 // Capture kRoundsPerGraph rounds into an executable graph (cached per shape).
 int round_graph(Graph& g, bool sampled, cudaStream_t s, cudaGraphExec_t* out) {
-    // everything a captured launch bakes in: mode, h, M, slot size, scratch, batch tables
-    const int key[10] = {(sampled ? 1 : 0) | (g.dense ? 2 : 0), g.h, (int)g.M, (int)g.cap,
-                         (int)g.scratch_ctas, (int)(reinterpret_cast<uintptr_t>(g.hv) >> 4),
-                         (int)(reinterpret_cast<uintptr_t>(g.Mv) >> 4), g.hmin,
-                         (int)(reinterpret_cast<uintptr_t>(g.rowptr) >> 4), (int)g.vcount};
+    // Everything that the captured launches hold and a later call can change: settings
+    // and sizes, and the address of every array that is freed and allocated again in a
+    // graph's life (the others stay where they are; what an array holds is read anew).
+    auto at = [](const void* p) { return (int64_t)reinterpret_cast<uintptr_t>(p); };
+    const int64_t key[kRoundKey] = {
+        (sampled ? 1 : 0) | (g.dense ? 2 : 0), g.h, g.hmin, g.hmax, g.M, g.cap, g.scratch_ctas, g.vcount,
+        g.levelu_mode, g.levelu_div, at(g.rowptr), at(g.col), at(g.vlist), at(g.hv), at(g.Mv), at(g.keys),
+        at(g.meta), at(g.queues), at(g.gbitmaps), at(g.part_keys), at(g.lu_stage)};
     if (g.round_exec && memcmp(key, g.round_exec_key, sizeof(key)) == 0) {
         *out = g.round_exec;
         return KH_OK;
