@@ -86,11 +86,27 @@ void load_table_locked() {
     fclose(f);
 }
 
-bool table_find(const std::string& key, TuneChoice* out) {
+bool cta_fits(const Graph& g) {
+    const int64_t words = (g.n + 31) / 32;
+    return ((words + 3) & ~(int64_t)3) * 4 <= kSmemBitmapMax;
+}
+
+// Whether a row's layout can run on this graph: graphs of one shape class differ in n
+// by up to a factor of two, so slices that fit one may be too wide for another, and a
+// file may hold anything.
+bool row_fits(const Graph& g, const TableRow& r) {
+    if (r.sweep_bin < 0 || r.sweep_bin >= kOrderBinsMax) return false;
+    if (r.variant == KH_VAR_CTA) return cta_fits(g);
+    if (r.variant != KH_VAR_SLICED && r.variant != KH_VAR_SLICED_SMALL) return false;
+    return (r.threads == 128 || r.threads == 256 || r.threads == 512 || r.threads == 1024) &&
+           r.slices >= hdeg2_min_slices(g.n) && r.slices <= 1024;
+}
+
+bool table_find(const Graph& g, const std::string& key, TuneChoice* out) {
     std::lock_guard<std::mutex> lk(g_table_mu);
     load_table_locked();
     for (auto it = g_table->rbegin(); it != g_table->rend(); ++it)
-        if (it->key == key) {
+        if (it->key == key && row_fits(g, *it)) {
             out->variant = it->variant;
             out->slices = it->slices;
             out->threads = it->threads;
@@ -111,11 +127,6 @@ void table_add(const std::string& key, const TuneChoice& c) {
     if (!f) return;
     fprintf(f, "%s | %d %d %d %.4f %d\n", key.c_str(), c.variant, c.slices, c.threads, c.ms, c.sweep_bin);
     fclose(f);
-}
-
-bool cta_fits(const Graph& g) {
-    const int64_t words = (g.n + 31) / 32;
-    return ((words + 3) & ~(int64_t)3) * 4 <= kSmemBitmapMax;
 }
 
 __global__ void k_stride_sample(const int32_t* __restrict__ order, int64_t nsrc, int64_t stride,
@@ -232,7 +243,7 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
     }
     const std::string key = shape_key(g, max_deg);
     TuneChoice c{};
-    if (table_find(key, &c) && (c.variant != KH_VAR_CTA || cta_fits(g))) {
+    if (table_find(g, key, &c)) {
         g.tuned_hdeg2 = c;
         *out = c;
         return KH_OK;
