@@ -273,9 +273,10 @@ int kh_hdegree_exact_noalloc(int64_t n, const int64_t *rowptr, const int32_t *co
  * KH_VAR_AUTO (default): the library's autotuner times the candidate layouts
  * on a sample of the graph's sources at the first such call and keeps the
  * fastest; with the environment variable KH_TUNE_FILE naming a text file, the
- * choice is also recorded there per graph shape class (device SM count, log2
- * n, log2 nnz, log2 of max degree over mean degree) and reused by later
- * processes.  Every layout returns the same degrees.  kh_set_variant forces
+ * choice is also recorded there per version of the kernels and graph shape
+ * class (device SM count, log2 n, log2 nnz, log2 of max degree over mean
+ * degree) and reused by later processes; rows of other versions and rows that
+ * do not fit the graph are passed over.  Every layout returns the same degrees.  kh_set_variant forces
  * a layout (KH_EINVAL for an unknown op or variant, KH_VAR_CTA with n too
  * large, or slices outside [the shared-memory minimum, min(1024, n)]);
  * kh_get_variant returns the layout in force, tuning first if needed, and the

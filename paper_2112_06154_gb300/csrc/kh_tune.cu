@@ -54,10 +54,15 @@ bool g_table_loaded = false;
 
 int ilog2(double x) { return x <= 1.0 ? 0 : (int)std::floor(std::log2(x)); }
 
+// The row's version goes up when the candidate kernels change: a choice measured on
+// other kernels says nothing (rows without one are from before k_hdeg2_cta and the
+// batches of 1024, and pin the sliced layout where it takes twice the time).
+constexpr int kTableVersion = 2;
+
 std::string shape_key(const Graph& g, int64_t max_deg) {
     const double avg = g.n > 0 ? (double)g.nnz / (double)g.n : 0.0;
     char buf[160];
-    snprintf(buf, sizeof(buf), "hdeg2 sm%d n%d e%d s%d", g.ctx->sm_count, ilog2((double)g.n),
+    snprintf(buf, sizeof(buf), "hdeg2 v%d sm%d n%d e%d s%d", kTableVersion, g.ctx->sm_count, ilog2((double)g.n),
              ilog2((double)g.nnz), ilog2(avg > 0 ? (double)max_deg / avg : 1.0));
     return buf;
 }

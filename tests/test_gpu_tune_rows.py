@@ -68,3 +68,14 @@ def test_a_usable_row_is_used(tmp_path):
     key = table.read_text().split("|")[0].strip()
     table.write_text("%s | 2 5 128 1.0 0\n" % key)  # (the tuner offers no 128 threads)
     assert run(table, LARGE, tmp_path / "b.npy") == [2, 5, 128]
+
+
+def test_rows_without_this_version_are_not_used(tmp_path):
+    table = tmp_path / "tune.txt"
+    run(table, SMALL, tmp_path / "a.npy")
+    key = table.read_text().split("|")[0].split()
+    assert key[0] == "hdeg2" and key[1].startswith("v")
+    # as the first builds wrote it, and another version's
+    rows = [" ".join(key[:1] + key[2:]), " ".join([key[0], key[1] + "9"] + key[2:])]
+    table.write_text("".join("%s | 2 5 128 1.0 0\n" % k for k in rows))
+    assert run(table, LARGE, tmp_path / "b.npy")[2] in (256, 512, 1024)
