@@ -1083,10 +1083,8 @@ int launch_hdeg2_cta(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cuda
     a.err = &g.state->err;
     a.updates = &g.state->updates;
     a.bytes = &g.state->bytes[kProfBfs];
-    prof_begin(g, kProfBfs, s);
     kern<<<(int)grid, threads, dyn, s>>>(a);
     count_launch(g, 1);
-    prof_end(g, kProfBfs, s);
     return KH_OK;
 }
 

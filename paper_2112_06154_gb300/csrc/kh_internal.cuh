@@ -240,7 +240,8 @@ void launch_stale_exact(Graph& g, const int* list, const int* d_count, cudaStrea
 // their starting values first (every node); otherwise they must hold them.
 int launch_hdeg2_slice(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s,
                        int slices, int threads, const int32_t* order, int64_t nsrc, bool init);
-// the same with one CTA per source and a bitmap of all n nodes (n <= 819200)
+// the same with one CTA per source and a bitmap of all n nodes (n <= 819200); the
+// caller opens the profiling bracket (large and other sources run beside each other)
 int launch_hdeg2_cta(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s,
                      const int32_t* order, int64_t nsrc, bool large);
 int launch_init2(Graph& g, int32_t* deg, int32_t* cnt, int jlo, int nj, cudaStream_t s);

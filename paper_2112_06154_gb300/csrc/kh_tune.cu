@@ -172,6 +172,9 @@ int run_layout(Graph& g, const TuneChoice& c, int32_t* deg, int32_t* cnt, int jl
         int rc = cnt ? ensure_crank(g, s) : KH_OK;
         if (rc) return rc;
         if ((rc = launch_init2(g, deg, cnt, jlo, nj, s))) return rc;
+        // one bracket around both launches: two would overlap, and each would count
+        // the other's bytes
+        if (split.cta > 0) prof_begin(g, kProfBfs, s);
         if (split.large > 0) {
             // beside the others: alone, the few large sources leave most SMs idle
             // (Chung-Lu n = 200k: 1.70 -> 1.9 ms in line)
@@ -187,6 +190,7 @@ int run_layout(Graph& g, const TuneChoice& c, int32_t* deg, int32_t* cnt, int jl
         rc = launch_hdeg2_cta(g, deg, cnt, jlo, nj, s, order + split.large, split.cta - split.large, false);
         if (split.large > 0) KH_CUDA_TRY(g.ctx, cudaStreamWaitEvent(s, g.ctx->join, 0));
         if (rc) return rc;
+        if (split.cta > 0) prof_end(g, kProfBfs, s);
         return launch_hdeg2_small(g, deg, cnt, jlo, nj, s, order + split.cta, nsrc - split.cta);
     }
     if (c.variant != KH_VAR_SLICED_SMALL)
