@@ -763,25 +763,41 @@ __global__ void k_stale_exact(const int64_t* __restrict__ rowptr, const int32_t*
 
 // The nodes the loss BFS reached keep their state: d (exact when fresh, an
 // upper bound when stale) and the stale lower bound both drop by the loss.
-// Each is one h-degree update (an incremental recomputation).
-__global__ void k_apply_loss(const int32_t* __restrict__ list, const int* __restrict__ nlist,
-                             int32_t* __restrict__ loss, int32_t* __restrict__ d,
-                             const uint8_t* __restrict__ fresh, unsigned long long* __restrict__ lb,
-                             DevState* __restrict__ st, int64_t cap) {
-    const int cnt = (int)min((int64_t)*nlist, cap);
+// Each is one h-degree update (an incremental recomputation), unless its graph
+// has reached the early stop: its remaining nodes leave at the next round's start
+// (k_begin) and are not recomputed.
+struct LossArgs {
+    const int32_t* list;
+    const int* nlist;
+    int32_t* loss;
+    int32_t* d;
+    const uint8_t* fresh;
+    unsigned long long* lb;
+    DevState* st;
+    int64_t cap;
+    int stop;                     // the peel applies the early stop
+    const unsigned long long* c;  // per graph, of this round (the ball's first hop ended it)
+    const int32_t* left;          // batches: alive nodes per graph
+    const int32_t* gid;
+};
+
+__global__ void k_apply_loss(LossArgs a) {
+    const int cnt = (int)min((int64_t)*a.nlist, a.cap);
     if (blockIdx.x == 0 && threadIdx.x == 0 && cnt > 0) {
-        atomicAdd(&st->updates, (unsigned long long)cnt);
-        atomicAdd(&st->bytes[kProfFrontier], 21ull * (unsigned long long)cnt);
+        if (!a.gid && !(a.stop && early_stop(a.c[0], a.st->n_alive_next)))
+            atomicAdd(&a.st->updates, (unsigned long long)cnt);
+        atomicAdd(&a.st->bytes[kProfFrontier], 21ull * (unsigned long long)cnt);
     }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-        const int v = list[i];
-        const int l = loss[v];
-        loss[v] = 0;
-        d[v] -= l;
-        if (!fresh[v]) {
-            const unsigned long long x = lb[v];
-            lb[v] = x > (unsigned long long)l ? x - (unsigned long long)l : 0ull;
+        const int v = a.list[i];
+        const int l = a.loss[v];
+        a.loss[v] = 0;
+        a.d[v] -= l;
+        if (!a.fresh[v]) {
+            const unsigned long long x = a.lb[v];
+            a.lb[v] = x > (unsigned long long)l ? x - (unsigned long long)l : 0ull;
         }
+        if (a.gid && !(a.stop && early_stop(a.c[a.gid[v]], a.left[a.gid[v]]))) atomicAdd(&a.st->updates, 1ull);
     }
 }
 
@@ -941,8 +957,8 @@ void launch_ball_hop(Graph& g, int hop, cudaStream_t s) {
 void launch_apply_loss(Graph& g, cudaStream_t s) {
     const int grid = g.ctx->sm_count * 4;
     prof_begin(g, kProfFrontier, s);
-    k_apply_loss<<<grid, 256, 0, s>>>(g.listL, &g.state->rc[kRcLossCount], g.loss, g.d32, g.fresh,
-                                      g.lb64, g.state, g.n);
+    k_apply_loss<<<grid, 256, 0, s>>>({g.listL, &g.state->rc[kRcLossCount], g.loss, g.d32, g.fresh, g.lb64, g.state,
+                                       g.n, g.dense ? 0 : 1, g.pc, g.pleft, g.gid});
     count_launch(g, 1);
     prof_end(g, kProfFrontier, s);
 }

@@ -131,6 +131,10 @@ __device__ __forceinline__ void end_round(const RoundEnd& r) {
         r.mu[q] = ~0ull;
     }
 }
+// Sec. 5: with c >= |X| - 1 every remaining node has deg_h <= |X| - 1 <= c.
+__device__ __forceinline__ bool early_stop(unsigned long long c, int left) {
+    return left > 0 && c + 1 >= (unsigned long long)left;
+}
 #endif
 RoundEnd round_end(const Graph& g);
 

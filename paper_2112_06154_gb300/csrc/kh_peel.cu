@@ -97,11 +97,6 @@ __device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigne
     return a < b ? a : b;
 }
 
-// Sec. 5: with c >= |X| - 1 every remaining node has deg_h <= |X| - 1 <= c.
-__device__ __forceinline__ bool early_stop(unsigned long long c, int left) {
-    return left > 0 && c + 1 >= (unsigned long long)left;
-}
-
 // Round start.  The previous round ends: its removed nodes leave (alive = 0, dead
 // bitmap bit set), the per-round counters go back to zero, and, in exact peels,
 // the nodes of a graph with c >= |X| - 1 get core c in the round after that one
