@@ -653,9 +653,9 @@ int kh_footprint(int64_t n, int64_t nnz, int32_t h, int64_t M_or_0, double eps, 
     b += (int64_t)(h - 1) * n * cap * 4 + (int64_t)h * n * 4 + n + 4 * n + n / 32 + 1024 +
          (int64_t)2 * 12 * 160 * cap * 4;
     // split parts of heavy nodes: at most nnz / 341 slots (ceil(deg/512) <=
-    // deg/341 for deg > 1024), each cap keys plus counters
-    const int64_t parts = nnz / 341;
-    b += parts * (cap * 4 + 32) + 4 * n;
+    // deg/341 for deg > 1024), each cap keys plus counters; none where no node can
+    // have more than kSplitMin neighbours (each of which lists it in turn)
+    if (n > kh::kSplitMin + 1 && nnz >= 2 * (kh::kSplitMin + 1)) b += nnz / 341 * (cap * 4 + 32) + 4 * n;
     // the peel's compaction buffers (graphs of at least 65536 nodes)
     if (n >= 65536) b += 2 * 8 * (n + 1) + 2 * 4 * nnz + 2 * 4 * (n + 1) + 16 * (n + 1) + 64 * 1024;
     *bytes = b + (1 << 20);
