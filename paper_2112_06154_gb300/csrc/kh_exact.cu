@@ -10,6 +10,7 @@
 // lone frontier vertex) are expanded by the whole CTA.  New vertices are
 // appended to the CTA's queue with one warp-aggregated atomic per warp step.
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 
@@ -20,14 +21,22 @@ namespace kh {
 namespace {
 
 constexpr int kBfsThreads = 256;
-// A peel round has a handful of sources, so at h >= 3 the length of its searches is
-// that of one CTA's: 512 threads where balls are large (mean degree of at least
-// kBfsWideDegree), (k,3)-core of Chung-Lu n = 20k 2103 -> 1554 ms, of R-MAT 13 466 -> 328,
-// (k,4)-core of G(20k, 60k) (mean degree 6) 131 -> 112.  On a grid (mean degree 4, balls of
-// 25 nodes) the wider barriers cost more than they give: 10.6 -> 11.1 ms.  1024 threads:
-// 1400, 283, 112 and 13.1 ms, but 295 against 273 on the (k,4)-core of R-MAT 13.
+// A peel round has a handful of sources, so at h >= 3 its length is that of one CTA's
+// search: 512 threads where balls are large (wide_searches), 256 elsewhere.
+// With the mean degree d and the mean degree q of a neighbour (sum of squares over sum),
+// a ball of a graph without structure has about d (q - 1)^(h-1) nodes at its rim; a
+// lattice, whose degrees hardly vary (q - d below 0.1), far fewer.  Exact cores with
+// 256 -> 512 threads, ms: above the line Chung-Lu n = 20k h = 3 2103 -> 1554, R-MAT 13 h = 3
+// 466 -> 328, Chung-Lu n = 8k at d = 2 / 3 / 4 / 6 h = 3 (rim 95 to 2500) 21.7 -> 20.5, 43.6 ->
+// 39.6, 73.7 -> 65.3, 175 -> 144, G(n, m) with d = 5.1 / 6 / 8 h = 3 (132, 216, 512) 13.2 ->
+// 12.9, 25.4 -> 24.8, 27.6 -> 25.1, d = 3 / 4 / 6 h = 4 (83, 256, 1296) 18.4 -> 18.1, 43.2 ->
+// 41.4, 136 -> 117; below it d = 4 h = 3 (64) 10.8 -> 11.1, a grid h = 3 / 4 / 5 16.0 -> 17.3,
+// 17.5 -> 17.8, 22.8 -> 23.0, a lattice of 30^3 h = 3 / 4 / 5 7.5 -> 8.2, 16.1 -> 17.5, 27.0 ->
+// 28.9 (its rim would be 136 to 3157).  1024 threads on Chung-Lu n = 20k, R-MAT 13, G(20k, 60k)
+// h = 4 and a grid: 1400, 283, 112 and 13.1 ms, but 295 against 273 on R-MAT 13 at h = 4.
 constexpr int kBfsRoundThreads = 512;
-constexpr int kBfsWideDegree = 5;
+constexpr double kBfsWideRim = 80.0;
+constexpr double kBfsWideVary = 0.5;
 constexpr int kHeavyDeg = 128;
 constexpr int kMaxHeavy = 64;
 constexpr uint32_t kFull = 0xffffffffu;
@@ -802,10 +811,11 @@ __global__ void k_apply_loss(LossArgs a) {
 }
 
 // The neighbour of largest degree of each node (ties: the smaller id; -1 for
-// an isolated node), one warp per node.
+// an isolated node), one warp per node; the sum of the squared degrees into *deg2.
 __global__ void k_best_nb(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                          int64_t n, int32_t* __restrict__ best) {
+                          int64_t n, int32_t* __restrict__ best, unsigned long long* deg2) {
     const int lane = threadIdx.x & 31;
+    unsigned long long squares = 0;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
         long long key = -1;  // (degree << 32) | (0x7fffffff - id): max picks largest degree, smallest id
@@ -819,7 +829,17 @@ __global__ void k_best_nb(const int64_t* __restrict__ rowptr, const int32_t* __r
             key = key > o ? key : o;
         }
         if (lane == 0) best[v] = key < 0 ? -1 : (int32_t)(0x7fffffff - (int32_t)(key & 0x7fffffff));
+        const unsigned long long deg = (unsigned long long)(rowptr[v + 1] - rowptr[v]);
+        squares += deg * deg;
     }
+    if (lane == 0 && squares) atomicAdd(deg2, squares);
+}
+
+// (of the peel's searches: the sum of squared degrees is known once a peel has begun)
+bool wide_searches(const Graph& g) {
+    if (g.gid || g.h < 3 || g.nnz == 0) return false;
+    const double d = (double)g.nnz / (double)g.n, q = (double)g.deg2 / (double)g.nnz;
+    return q >= d + kBfsWideVary && d * std::pow(q - 1.0, g.h - 1) >= kBfsWideRim;
 }
 
 int pick_grid(int sm, int per_sm, int64_t work) {
@@ -835,7 +855,8 @@ int ensure_bestnb(Graph& g, cudaStream_t s) {
     int rc = alloc_bytes(g.ctx, (void**)&g.bestnb, sizeof(int32_t) * (size_t)g.n, "best neighbours");
     if (rc) return rc;
     k_best_nb<<<pick_grid(g.ctx->sm_count, 8, (g.n * 32 + 255) / 256), 256, 0, s>>>(g.rowptr, g.col,
-                                                                                   g.n, g.bestnb);
+                                                                                   g.n, g.bestnb,
+                                                                                   &g.state->deg2);
     count_launch(g, 1);
     return KH_OK;
 }
@@ -876,8 +897,7 @@ int launch_hdeg(Graph& g, const int* worklist, const int* d_count, int64_t count
                                              (int)kSmemBitmapMax);
         if (e != cudaSuccess) return check_cuda(g.ctx, e, "cudaFuncSetAttribute(k_hdeg)");
     }
-    const bool wide = round_ctr && !g.gid && g.h >= 3 && g.nnz >= kBfsWideDegree * g.n;
-    const int threads = wide ? kBfsRoundThreads : kBfsThreads;
+    const int threads = round_ctr && wide_searches(g) ? kBfsRoundThreads : kBfsThreads;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, dyn);
     if (e != cudaSuccess) return check_cuda(g.ctx, e, "occupancy(k_hdeg)");

@@ -103,6 +103,7 @@ struct DevState {
     unsigned long long stopped;
     int tune_count;              // sample size of an autotuner measurement
     int nSub;                    // split-part items (standalone level passes)
+    unsigned long long deg2;     // sum of squared degrees, until the first peel reads it
 };
 
 struct Graph;
@@ -553,6 +554,7 @@ struct Graph {
     int sw_force;             // forced sweep threshold bin (0: tuner; -1: no sweeps)
     // each node's neighbour of largest degree (-1: none), for cheap stale bounds
     int32_t *bestnb;
+    unsigned long long deg2;  // sum of squared degrees (0: no peel has run yet)
     // the 2-degree pass layout: forced by kh_set_variant, or chosen by the tuner
     TuneChoice force_hdeg2;
     TuneChoice tuned_hdeg2;

@@ -855,6 +855,7 @@ int run_core(Graph& g, bool sampled, void* out_core, int32_t* round_of_host, boo
     DevState init;
     KH_CUDA_TRY(g.ctx, cudaMemcpyAsync(&init, g.state, sizeof(init), cudaMemcpyDeviceToHost, s));
     KH_CUDA_TRY(g.ctx, cudaStreamSynchronize(s));
+    if (g.deg2 == 0) g.deg2 = init.deg2;
     unsigned long long keep_bytes[kProfKinds];
     memcpy(keep_bytes, init.bytes, sizeof(keep_bytes));
     memset(&init, 0, sizeof(init));
