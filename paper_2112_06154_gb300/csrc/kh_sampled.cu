@@ -436,10 +436,12 @@ constexpr int kKeysPerLane = 4;  // words one lane loads per step (one 16-byte v
 // ones (up to about 8 keys expected at or above t: 2 lanes a list), middle
 // (up to 64: 8 lanes), long (a warp a list) and dense (8 lanes).
 constexpr int kBuckets = 4;
-// Every step of a warp reads at least one of the chunk's lists on by 8 words (a
-// short one, by 2 lanes) or ends a bucket, so no correct walk takes more steps than
-// this; one that does ends the union with kErrLoop.
-constexpr int kWalkSteps = kLuThreads * (kMaxM / 8 + 2) + kBuckets;
+// A bucket's claims over a chunk: its lists, and one in vain of each group of 2 lanes
+// or more.  Every step of a warp claims, reads a list on by 8 words or more, or ends a
+// bucket, so with the claims the walk is bounded; one past them ends the union with
+// kErrLoop.  (A count of the steps took 5% of the estimates of G(2000, 8000) and 1.5% of
+// those of R-MAT 22 in registers; the claims have theirs.)
+constexpr int kMaxClaims = kLuThreads + kLuThreads / 2;
 constexpr int kShort = 0, kMiddle = 1, kDense = 2, kLong = 3;
 
 // Shared state of one node's union.
@@ -503,7 +505,7 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
         sz = sh.sz[li];
     }
 #pragma unroll 1
-    for (int step = 0; step < kWalkSteps; ++step) {
+    for (;;) {
         // one read for the whole warp: lanes that saw a flag at different
         // moments would part ways before the ballots
         int stop = 0;
@@ -517,6 +519,13 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
             int base = 0;
             if (lane == 0) base = atomicAdd(&sh.cq[bk], __popc(need));
             base = __shfl_sync(kFull, base, 0);
+            if (base >= kMaxClaims) {
+                if (lane == 0) {
+                    atomicOr(c.err, kErrLoop);
+                    atomicCAS(&sh.exit, 0, 2);  // the other warps leave too
+                }
+                return;
+            }
             if (li == -1) {
                 const int i = base + __popc(need & ((1u << lead) - 1u));
                 li = -2;
@@ -535,10 +544,9 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
             li = -1;
             continue;
         }
-        // the level likewise: other warps raise it, and the whole warp tests it below
-        int t = 0;
-        if (lane == 0) t = *(volatile int*)&sh.t;
-        t = __shfl_sync(kFull, t, 0);
+        // the lanes need not read this together and other warps raise it, so lanes may
+        // hold different levels (each one valid): only for tests of a lane by itself
+        const int t = *(volatile int*)&sh.t;
         int ins = 0;
         bool done = false;
         if (li >= 0) {
@@ -638,10 +646,6 @@ __device__ __forceinline__ void walk_chunk(const UnionCtx& c, UnionShared& sh, i
                     atomicCAS(&sh.exit, 0, 2);
             }
         }
-    }
-    if (lane == 0) {
-        atomicOr(c.err, kErrLoop);
-        atomicCAS(&sh.exit, 0, 2);  // the other warps leave too
     }
 }
 
@@ -813,7 +817,7 @@ __device__ __forceinline__ int lost_rank(const LevelArgs& a, const UnionShared& 
 // insert is one shared load and, when new, one atomic OR: no probing, no list
 // of used slots and no compaction, and the output is in rank order by itself.
 // The neighbours' meta words are read once per chunk of 128 into shared
-// memory and sorted into buckets by what a list will give (walk_lists).
+// memory and sorted into buckets by what a list will give (walk_chunk).
 //
 // Heavy nodes (degree > kSplitDeg) are split: part j unions the lists of
 // neighbours [j kSplitChunk, (j+1) kSplitChunk) into its own trimmed partial
@@ -840,8 +844,8 @@ __device__ __forceinline__ int lost_rank(const LevelArgs& a, const UnionShared& 
 // the estimates (79.9 ms) and cost 30% in the rounds.
 //
 // LAST: nodes at their last level (estimate, refine); LIST: nodes below it
-// (stored lists); PARTS: the parts of the split nodes, which the launch before
-// planned.  One kernel for all of it runs out of the instruction cache.
+// (stored lists); PARTS: the parts of the split nodes, planned by the kernel that
+// made the list (whole passes: by the launch before).  One kernel for all of it runs out of the instruction cache.
 template <bool LAST, bool LIST, bool PARTS>
 __global__ void __launch_bounds__(kLuThreads, kLuPerSm) k_levelU(LevelArgs a) {
     extern __shared__ __align__(16) uint32_t tab[];

@@ -1,7 +1,7 @@
-"""The step bounds of the claim loops (walk_chunk; the row readers of k_hdeg2_cta and
-k_hdeg2_peel) on the CPU: a model of one warp that reads a whole chunk alone, the most
-steps a warp can take, stays within the bound that the kernels compile in; every such
-loop has a bound."""
+"""The bounds of the claim loops on the CPU.  walk_chunk bounds a chunk's claims: a model of
+the warps' claims, in any order, stays within.  The row readers of k_hdeg2_cta and
+k_hdeg2_peel bound a warp's steps: a model of one warp that reads a whole chunk alone, the
+most steps a warp can take, stays within.  Every such loop has its bound."""
 import os
 import random
 import re
@@ -48,18 +48,38 @@ def steps_of_one_warp(buckets):
     return n
 
 
-@pytest.mark.parametrize("seed", range(4))
+def claims_of_a_chunk(rng, warps, lanes, lens):
+    """The counter's value before each claim of one bucket, warps in any order: a warp claims
+    for all its idle groups at once, a group that gets no list is done."""
+    lists, cq, bases = list(lens), 0, []
+    groups = [[0] * (32 // lanes) for _ in range(warps)]  # words left; -1: done
+    running = set(range(warps))
+    while running:
+        w = rng.choice(sorted(running))
+        g = groups[w]
+        idle = [i for i, left in enumerate(g) if left == 0]
+        if idle:
+            bases.append(cq)
+            for k, i in enumerate(idle):
+                g[i] = lists[cq + k] if cq + k < len(lists) else -1
+            cq += len(idle)
+        if all(left == -1 for left in g):
+            running.discard(w)
+        groups[w] = [left if left < 0 else max(0, left - 4 * lanes) for left in g]
+    return bases
+
+
+@pytest.mark.parametrize("seed", range(6))
 def test_walk_chunk(seed):
     rng = random.Random(seed)
     rows, most = (constant(c, "kh_internal.cuh", "kh_sampled.cu") for c in ("kLuThreads", "kMaxM"))
-    bound = constant("kWalkSteps", "kh_internal.cuh", "kh_sampled.cu")
-    lens = {0: [most] * rows, 1: [rng.randint(1, most) for _ in range(rows)],
-            2: [rng.choice([1, 7, 8, 9, 64, 65, 128, 129]) for _ in range(rows)],
-            3: [most] + [1] * (rows - 1)}[seed]
+    bound = constant("kMaxClaims", "kh_internal.cuh", "kh_sampled.cu")
+    lens = {0: [most] * rows, 1: [rng.randint(1, most) for _ in range(rows)], 2: [1] * rows, 3: [most] + [1] * (rows - 1),
+            4: [rng.choice([1, 7, 8, 9, 64, 65, 128, 129]) for _ in range(rows)], 5: [5] * (rows // 3)}[seed]
     for lanes in (2, 8, 32):
-        assert steps_of_one_warp([(lanes, 4, lens)]) <= bound
-    assert steps_of_one_warp([(lanes, 4, lens[i::4]) for i, lanes in enumerate((32, 8, 8, 2))]) <= bound
-    assert steps_of_one_warp([(lanes, 4, []) for lanes in (32, 8, 8, 2)]) <= bound
+        bases = claims_of_a_chunk(rng, rows // 32, lanes, lens)
+        assert max(bases) < bound
+    assert max(claims_of_a_chunk(rng, rows // 32, 2, [])) < bound
 
 
 @pytest.mark.parametrize("rows", [128, 256, 512])
@@ -73,7 +93,7 @@ def test_row_readers(rows):
 
 def test_every_claim_loop_has_its_bound():
     walk = source("kh_sampled.cu")
-    assert "for (int step = 0; step < kWalkSteps; ++step)" in walk
+    assert walk.count("if (base >= kMaxClaims)") == walk.count("atomicAdd(&sh.cq[") == 1
     for name in ("kh_hdeg2.cu", "kh_exact.cu"):
         text = source(name)
         assert text.count("if (step > row_steps(") == 1
