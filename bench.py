@@ -178,8 +178,8 @@ def parse():
                         "go to the bit-parallel sweeps (default: the tuner's choice)")
     p.add_argument("--union", default="auto",
                    help="schedule of the level-union kernel (kh_set_variant KH_OP_LEVEL_UNION): "
-                        "auto, stepped, free, grouped or grouped:D (a lane group covers 1/D of "
-                        "a list's expected keys)")
+                        "auto, stepped or free (both: a warp per list), grouped or grouped:D (a "
+                        "lane group covers 1/D of a list's expected keys)")
     p.add_argument("--prof", action="store_true",
                    help="--op only: bracket the kernel classes and print their times and "
                         "algorithmic bytes")

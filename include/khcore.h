@@ -26,7 +26,8 @@
  *     memory and the call returns after the results are written.  With
  *     KH_DEVICE_PTR they are device memory of the context's device and the
  *     results are written by work enqueued on the context's stream (kh_sync
- *     waits): kh_ranks, kh_hdegree_exact and kh_sampled_counts only enqueue;
+ *     waits): kh_ranks, kh_hdegree_exact and kh_sampled_counts only enqueue
+ *     (a graph's first such call at an h may also time layouts and wait);
  *     kh_estimate waits for its device error word before returning; the peels
  *     (kh_core_*, kh_dense) read a small device state once per eight rounds
  *     to know when to stop, so they synchronize with the stream while they run
@@ -213,13 +214,14 @@ int kh_peel_stats(kh_graph *g, int64_t *refreshed, int64_t *changed, int64_t *st
  * kh_prof_enable(g, 0) stops the brackets and keeps the counters.
  * kh_prof_read returns, for one class, the summed event time in ms, the number
  * of bracketed launches and the algorithmic bytes the class moved (counted on
- * the device: 8 + 4 deg per expanded vertex for the BFS, 4 per list key read
+ * the device: 8 + 4 deg per expanded vertex for the BFS, at h >= 3 in batches of
+ * 1024 sources the rows their passes read instead, 4 per list key read
  * and written for the list kernels, plus per-node metadata). */
 #define KH_PROF_BFS 0      /* exact h-degree / fixed-level count BFS */
 #define KH_PROF_LEVEL1 1   /* level-1 lists (Alg. 2 at i = 1) */
 #define KH_PROF_LEVELU 2   /* level >= 2 lists (Alg. 2 with Alg. 5's trim) */
 #define KH_PROF_FRONTIER 3 /* removed-set balls and refresh work lists */
-#define KH_PROF_PEEL 4     /* min / select / finish of each round */
+#define KH_PROF_PEEL 4     /* begin / collect / select of each round */
 #define KH_PROF_KINDS 5
 int kh_prof_enable(kh_graph *g, int32_t on);
 int kh_prof_read(kh_graph *g, int32_t kind, double *ms, int64_t *launches, double *alg_bytes);

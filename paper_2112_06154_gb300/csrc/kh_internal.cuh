@@ -61,9 +61,9 @@ constexpr int kSweepMinBin = 16;   // smallest work bin the tuner offers to the 
 // Kernel classes for the profiling counters (kh_prof_read kinds).
 constexpr int kProfBfs = 0;       // exact h-degree / fixed-level count BFS
 constexpr int kProfLevel1 = 1;    // level-1 lists
-constexpr int kProfLevelU = 2;    // level >= 2 lists (hashed union)
+constexpr int kProfLevelU = 2;    // level >= 2 lists (bitmap or hashed union)
 constexpr int kProfFrontier = 3;  // removed-set ball hops, neighbour marking
-constexpr int kProfPeel = 4;      // min, select, finish, advance
+constexpr int kProfPeel = 4;      // begin, collect, select
 constexpr int kProfKinds = 5;
 
 // Per-round counters: every launch inside a peeling round has its own slot, and

@@ -380,9 +380,15 @@ int choose_hdeg2(Graph& g, cudaStream_t s, TuneChoice* out) {
 // h >= 3: bit-parallel batches or a search per source, decided once per graph
 // and h.  The searches' cost per source comes from a probe of every n/152-th node
 // (the device byte counter: 4 bytes a row entry); the batches' cost is known: h - 1
-// pulls over all rows per 1024 sources.  A pull entry (a 128-byte gather, from L2
-// or, once the masks outgrow it, from HBM) costs about kPullCost search entries (a
-// 4-byte read and a bitmap test): measured 16 ps against 2 ps on Chung-Lu n = 200k.
+// pulls over all rows per 1024 sources.  A pull entry (a 128-byte gather) is priced at
+// kPullCost search entries (a 4-byte read and a bitmap test): 16 ps against 2 ps on
+// Chung-Lu n = 200k, mean degree 20.  Both forced, on sparser graphs and on masks far
+// beyond L2, the line stays on the safe side (by the ratio of the prices, batches from 1
+// on; searches / batches in ms): Chung-Lu n = 200k at mean degree 5 (0.44) 11.7 / 22.9,
+// n = 500k (0.33) 62 / 120, n = 800k at 4 (0.16) 112 / 275, G(400k, 2.8M) h = 4 (0.35) 213 /
+// 139.  Above 819,200 nodes the searches' bitmaps leave shared memory and batches win
+// from about 0.1 on: Chung-Lu n = 1M at 4 (0.18) 601 / 425, at 6 (0.33) 1520 / 509, n = 2M
+// (0.11) 1865 / 1666, G(1M, 5M) h = 3 (0.008) 108 / 566, h = 4 (0.05) 958 / 930.
 constexpr int kProbe = 152;
 constexpr double kPullCost = 8.0;
 constexpr double kBatchOverhead = 1.0e7;  // a batch's launches, in search entries
